@@ -131,7 +131,8 @@ psatd_status psatd_init_grid(const psatd_grid* grid, const psatd_mapping* mappin
 /* Release everything the context owns (not caller-bound field storage). */
 void psatd_destroy(psatd_ctx* ctx);
 
-/* Change the step; rebuilds the cos/sin table on the host in float64.  Any finite
+/* Change the step; rebuilds the cos/sin table (float64, rounded once) on the
+ * device and waits for it.  Any finite
  * dt is valid, including negative (time reversal) and large (Sec. 2.1: the
  * vacuum solver is exact in time for any step). */
 psatd_status psatd_set_dt(psatd_ctx* ctx, double dt);
@@ -210,7 +211,7 @@ psatd_status psatd_sample_focal_plane(psatd_ctx* ctx, double x_phys, int ny, int
  * fft and diagnostics return PSATD_ERR_STATE until a pulse
  * or all six components are set again (psatd_sample_focal_plane keeps working,
  * from the spectrum); psatd_time() is T.  The coefficient
- * table for T is built on the host (float64) and cached for the next call with
+ * table for T is built on the device (float64) and cached for the next call with
  * the same T.  With real field storage the spectrum is the half spectrum of
  * real fields (the update is the real-field one, with the projection of B
  * folded in) and the sample is the same interpolant of the real field. */

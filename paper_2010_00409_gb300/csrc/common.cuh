@@ -240,6 +240,13 @@ cudaError_t launch_multi_advance(const MultiProblem<T>* probs, const long long* 
                                  size_t tile_bytes, long long max_items, unsigned* bar, int* err,
                                  unsigned long long limit_ns, unsigned extra, cudaStream_t s, int* grid_out);
 
+// Build the coefficient table of one step dt (coef.cu): C = cos(c|k|dt), S =
+// sin(c|k|dt) over Ntot, or C = 1/Ntot, S = 0 with `projection`; with slot_mode
+// (Nx/2 x mode indices, device memory) the x index is in slot order.
+template <typename T>
+cudaError_t launch_coef(ModeCoef<T>* tab, const GridGeom& g, double dt, bool projection, const int* slot_mode,
+                        cudaStream_t s);
+
 // K2 modes: ROTATE = full step (forward z, update, inverse z); PROJECT = the
 // one-time transverse projection; ROTATE_SPECTRAL = forward z and update only,
 // leaving the spectrum (natural kx, ky, kz order) in storage.

@@ -1,5 +1,5 @@
 // C ABI of the PSATD library (declared in include/psatd.h): argument checks,
-// float64 host tables, device memory, and the order of kernel launches.
+// axis tables, device memory, and the order of kernel launches.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -318,40 +318,29 @@ psatd_status upload_axis_tables(psatd_ctx* c) {
     return PSATD_OK;
 }
 
-// (C/Ntot, S/Ntot, 1/|k|) per |m| octant, float64 then rounded once.
-// slot_order: column p < Nx/2 holds the x mode of half-spectrum slot p (real
-// fields), column Nx/2 the x Nyquist mode.  projection: C = 1/Ntot, S = 0 (with
-// the B projection of the k-space kernel this is the one-time transverse
-// projection).
+// The table (C/Ntot, S/Ntot, 1/|k|) per |m| octant of one step dt into dst (or
+// the step's table), in stream order.  slot_order: column p < Nx/2 holds the x
+// mode of half-spectrum slot p (real fields), column Nx/2 the x Nyquist mode.
+// projection: C = 1/Ntot, S = 0 (with the B projection of the k-space kernel this
+// is the one-time transverse projection).  wait: return when the table is in
+// memory; the tensor-copy-fed k-space kernel reads it before its wait on the
+// previous kernel, so a table whose build no ordinary launch separates from that
+// kernel is waited for here.
+// A stream that is being captured is refused: the table belongs to the context,
+// and a replay would rewrite it under calls that rely on another step.
 template <typename T>
 psatd_status upload_coef(psatd_ctx* c, double dt, DevBuf* dst = nullptr, bool slot_order = false,
-                         bool projection = false) {
+                         bool projection = false, bool wait = true) {
     DevBuf& buf = dst ? *dst : c->coef;
     const psatd_grid& g = c->grid;
-    const int hx = g.Nx / 2 + 1, hy = g.Ny / 2 + 1, hz = g.Nz / 2 + 1;
-    const double ntot = (double)n_cells(g);
-    std::vector<ModeCoef<T>> tab((size_t)hx * hy * hz);
-    for (int az = 0; az < hz; ++az) {
-        const double kz = kTwoPi * az / (g.Nz * g.dz);
-        for (int ay = 0; ay < hy; ++ay) {
-            const double ky = kTwoPi * ay / (g.Ny * g.dy);
-            for (int ax = 0; ax < hx; ++ax) {
-                const int mx = (slot_order && ax < g.Nx / 2) ? plane_rc_slot_mode(ax) : ax;
-                const double kx = kTwoPi * mx / (g.Nx * g.dx);
-                const double km = std::sqrt(kx * kx + ky * ky + kz * kz);
-                ModeCoef<T> m;
-                m.C = (T)((projection ? 1.0 : std::cos(g.c * km * dt)) / ntot);
-                m.S = (T)(projection ? 0.0 : std::sin(g.c * km * dt) / ntot);
-                m.kinv = (T)(km > 0 ? 1.0 / km : 0.0);
-                m.pad = (T)0;
-                tab[((size_t)az * hy + ay) * hx + ax] = m;
-            }
-        }
-    }
-    const size_t bytes = tab.size() * sizeof(ModeCoef<T>);
-    CK(c, ensure_buf(buf, bytes));
-    CK(c, cudaMemcpyAsync(buf.p, tab.data(), bytes, cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
+    const size_t n = (size_t)(g.Nx / 2 + 1) * (g.Ny / 2 + 1) * (g.Nz / 2 + 1);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(c, cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return cuda_fail(c, cudaErrorStreamCaptureUnsupported, "coefficient table");
+    CK(c, ensure_buf(buf, n * sizeof(ModeCoef<T>)));
+    CK(c, launch_coef<T>(static_cast<ModeCoef<T>*>(buf.p), geom(c), dt, projection,
+                         slot_order ? static_cast<const int*>(c->slot_mode.p) : nullptr, c->stream));
+    if (wait) CK(c, cudaStreamSynchronize(c->stream));
     return PSATD_OK;
 }
 
@@ -979,8 +968,8 @@ psatd_status psatd_init_grid(const psatd_grid* grid, const psatd_mapping* mappin
     psatd_status st = PSATD_OK;
     if (e != cudaSuccess) st = cuda_fail(c, e, "cudaGetDevice");
     if (st == PSATD_OK) st = precision == 64 ? upload_axis_tables<double>(c) : upload_axis_tables<float>(c);
-    if (st == PSATD_OK) st = set_coef(c, dt);
     if (st == PSATD_OK && real) st = upload_slot_tables(c);
+    if (st == PSATD_OK) st = set_coef(c, dt);
     if (st == PSATD_OK) {
         e = lib_malloc(reinterpret_cast<void**>(&c->dev_err), sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(c->dev_err, 0, sizeof(int));
@@ -1301,9 +1290,11 @@ psatd_status psatd_focal_one_shot(psatd_ctx* c, const psatd_pulse* pulse, double
                                             "dst) must have run once before, with profiling off");
     }
     if (!c->coef_T_ok || c->coef_T_step != T) {
-        // real fields: the table in the slot order of the half spectrum
-        st = c->prec == 64 ? upload_coef<double>(c, T, &c->coef_T)
-                           : upload_coef<float>(c, T, &c->coef_T, c->real_fields);
+        // real fields: the table in the slot order of the half spectrum (the pulse
+        // initialisation below is an ordinary launch between it and its reader)
+        c->coef_T_ok = false;
+        st = c->prec == 64 ? upload_coef<double>(c, T, &c->coef_T, false, false, false)
+                           : upload_coef<float>(c, T, &c->coef_T, c->real_fields, false, false);
         if (st) return st;
         c->coef_T_ok = true;
         c->coef_T_step = T;
