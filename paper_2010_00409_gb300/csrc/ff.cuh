@@ -65,33 +65,51 @@ __host__ __device__ __forceinline__ float4 cff_from(double re, double im) {
     const FF r = ff_from(re), i = ff_from(im);
     return make_float4(r.h, r.l, i.h, i.l);
 }
-// acc += w v for a float32 complex v
-__device__ __forceinline__ void cff_mac(CFF& acc, const CFF& w, float2 v) {
-    acc.re = ff_add(acc.re, ff_sub(ff_mul_f(w.re, v.x), ff_mul_f(w.im, v.y)));
-    acc.im = ff_add(acc.im, ff_add(ff_mul_f(w.re, v.y), ff_mul_f(w.im, v.x)));
-}
-// acc += w v for a real float32 v
-__device__ __forceinline__ void cff_mac_real(CFF& acc, const CFF& w, float v) {
-    acc.re = ff_add(acc.re, ff_mul_f(w.re, v));
-    acc.im = ff_add(acc.im, ff_mul_f(w.im, v));
-}
-// acc += w v for a double-float complex v
-__device__ __forceinline__ void cff_mac_cff(CFF& acc, const CFF& w, const CFF& v) {
-    acc.re = ff_add(acc.re, ff_sub(ff_mul(w.re, v.re), ff_mul(w.im, v.im)));
-    acc.im = ff_add(acc.im, ff_add(ff_mul(w.re, v.im), ff_mul(w.im, v.re)));
-}
 __device__ __forceinline__ CFF cff_add(const CFF& a, const CFF& b) { return {ff_add(a.re, b.re), ff_add(a.im, b.im)}; }
-// sum over the 32 lanes of a warp (every lane gets the total)
-__device__ __forceinline__ CFF cff_warp_sum(CFF a) {
-    for (int o = 16; o > 0; o >>= 1) {
-        CFF b;
-        b.re.h = __shfl_xor_sync(0xffffffffu, a.re.h, o);
-        b.re.l = __shfl_xor_sync(0xffffffffu, a.re.l, o);
-        b.im.h = __shfl_xor_sync(0xffffffffu, a.im.h, o);
-        b.im.l = __shfl_xor_sync(0xffffffffu, a.im.l, o);
-        a = cff_add(a, b);
-    }
-    return a;
+
+// Compensated dot products (Dot2 of Ogita, Rump and Oishi, "Accurate sum and dot
+// product", 2005): the sum s takes every exact product by a two-sum, the rounding
+// errors and the low-order product terms are summed in c, and s + c is the sum as
+// if formed with twice the float32 precision.  One real term costs 11 (12 for a
+// double-float v) float32 instructions; adding each product to a renormalised
+// pair costs about 17.
+struct Dot2 {
+    float s, c;
+};
+struct Dot2C {
+    Dot2 re, im;
+};
+// d += (wh + wl) v
+__device__ __forceinline__ void dot2_term(Dot2& d, float wh, float wl, float v) {
+    const FF p = two_prod(wh, v), t = two_sum(d.s, p.h);
+    d.s = t.h;
+    d.c += t.l + fmaf(wl, v, p.l);
+}
+// d += (wh + wl) (vh + vl)
+__device__ __forceinline__ void dot2_term(Dot2& d, float wh, float wl, float vh, float vl) {
+    const FF p = two_prod(wh, vh), t = two_sum(d.s, p.h);
+    d.s = t.h;
+    d.c += t.l + fmaf(wh, vl, fmaf(wl, vh, p.l));
+}
+// acc += w v, w a double-float complex value {re.h, re.l, im.h, im.l}
+__device__ __forceinline__ void dot2_mac(Dot2C& acc, const float4& w, float2 v) {
+    dot2_term(acc.re, w.x, w.y, v.x);
+    dot2_term(acc.re, -w.z, -w.w, v.y);
+    dot2_term(acc.im, w.x, w.y, v.y);
+    dot2_term(acc.im, w.z, w.w, v.x);
+}
+__device__ __forceinline__ void dot2_mac_real(Dot2C& acc, const float4& w, float v) {
+    dot2_term(acc.re, w.x, w.y, v);
+    dot2_term(acc.im, w.z, w.w, v);
+}
+__device__ __forceinline__ void dot2_mac_cff(Dot2C& acc, const float4& w, const float4& v) {
+    dot2_term(acc.re, w.x, w.y, v.x, v.y);
+    dot2_term(acc.re, -w.z, -w.w, v.z, v.w);
+    dot2_term(acc.im, w.x, w.y, v.z, v.w);
+    dot2_term(acc.im, w.z, w.w, v.x, v.y);
+}
+__device__ __forceinline__ CFF dot2_value(const Dot2C& a) {
+    return {two_sum(a.re.s, a.re.c), two_sum(a.im.s, a.im.c)};
 }
 
 }  // namespace psatd
