@@ -248,8 +248,9 @@ long long psatd_launch_count(const psatd_ctx* ctx);
 
 /* Kernel selection: AUTO uses the register-resident kernels where the axis
  * length has one (64, 128, 256, 512; the k-space pass for Nz in 64, 128, 256,
- * fed by tensor copies), and the generic shared-memory Stockham kernels
- * elsewhere; REGISTER is AUTO without the tensor-copy feed; GENERIC forces the
+ * fed by tensor copies), in float32 compile-time two-pass kernels for
+ * the other lengths to 256 that are a product of two radices up to 16, and the
+ * generic mixed-radix kernels elsewhere; REGISTER is AUTO without the tensor-copy feed; GENERIC forces the
  * generic kernels everywhere.  All compute the same transform; default AUTO. */
 enum { PSATD_PATH_AUTO = 0, PSATD_PATH_GENERIC = 1, PSATD_PATH_REGISTER = 2 };
 psatd_status psatd_set_kernel_path(psatd_ctx* ctx, int path);
@@ -343,7 +344,7 @@ psatd_status psatd_multi_advance(psatd_ctx* const* ctxs, int n_ctx, const int* n
 
 /* Autotuner of the batched advance: on copies of the fields (the contexts'
  * fields are left unchanged), times trial_steps steps of the whole batch for
- * every distinct radix schedule (radices 8/4/5/3/2 or 4/5/3/2, largest or
+ * every distinct radix schedule (the fewest radices up to 16, largest or
  * smallest first) and tile-width scale (1/2, 1, 2) of each axis length in turn
  * (coordinate descent), keeps the fastest and caches it per (precision, axis
  * length) for later psatd_multi_advance calls in this process.  Writes the best

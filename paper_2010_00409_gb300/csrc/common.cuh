@@ -158,18 +158,26 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// 1D plan of one axis: N = prod(radix[0..npass)), radices in {2,3,4,5,8}
+// 1D plan of one axis: N = prod(radix[0..npass)), radices up to 16 (narrow plans)
+// or 32 out of those fft_mixed.cuh has a register DFT for; N = 1 is one radix 1
 // ---------------------------------------------------------------------------
-constexpr int kMaxPass = 16;
+constexpr int kMaxPass = 8;
 struct AxisPlan {
     int N;
     int npass;
     int radix[kMaxPass];
+    // multipliers of fdiv (fft_mixed.cuh) by N / radix[p], by level p's M / radix[p]
+    // and by the first level's N / radix[0]: 25 instructions each if every thread
+    // works them out
+    unsigned div_nb[kMaxPass], div_l[kMaxPass], div_run;
 };
 
-// Host: factor N into 8, 4, 5, 3, 2 (largest radices first).  Returns false if
-// N has another prime factor.
-bool make_plan(int N, AxisPlan* p);
+// Host: factor N into the fewest radices up to max_radix (16, 20 or 32; then the
+// smallest largest radix), largest first.  Returns false if N has a prime factor
+// other than 2, 3 and 5.
+bool make_plan(int N, AxisPlan* p, int max_radix = 16);
+// Set a plan's division multipliers from its radices.
+void finish_plan(AxisPlan* p);
 
 // ---------------------------------------------------------------------------
 // Per-mode table entry: C/Ntot, S/Ntot, 1/|k| (0 at k = 0).
@@ -205,6 +213,7 @@ template <typename T> struct Tables {
     const T* k[3];              // k_a[i] = 2 pi m(i) / (N_a d_a)
     const ModeCoef<T>* coef;    // (Nz/2+1) x (Ny/2+1) x (Nx/2+1)
     AxisPlan plan[3];
+    const cplx<T>* twp[3];      // the plan's twiddles in position order (fft_mixed.cuh)
     int tile_shift = 0;         // generic kernels: tile width scaled by 2^tile_shift (autotuner)
 };
 
@@ -213,7 +222,7 @@ template <typename T> struct Tables {
 // the tile widths of the x (rows per tile), y and z (x-columns per tile) phases.
 template <typename T> struct MultiProblem {
     cplx<T>* f;
-    const cplx<T>* tw[3];
+    const cplx<T>* tp[3];       // twiddles of the plans below, in position order
     const T* k[3];
     const ModeCoef<T>* coef;
     int N[3];
@@ -222,10 +231,10 @@ template <typename T> struct MultiProblem {
     AxisPlan plan[3];
 };
 
-// Shared-memory bytes of one tile of the phase along `axis` (N_axis points,
-// W pencils): two Stockham buffers for x and y, six components and a partner
-// buffer for the fused z pass.
-template <typename T> size_t multi_tile_bytes(int axis, int N_axis, int W);
+// Shared-memory bytes of one tile of the phase along `axis` (plan pl,
+// W pencils): the pencils of one component for x and y, of six for the fused z
+// pass.
+template <typename T> size_t multi_tile_bytes(int axis, const AxisPlan& pl, int W);
 
 // Persistent cooperative launch advancing nprob boxes by up to nsteps PSATD
 // steps (box p by its own probs[p].nsteps <= nsteps).

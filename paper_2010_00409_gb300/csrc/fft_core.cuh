@@ -1,15 +1,7 @@
-// Device FFT building blocks: radix-2/3/4/5/8 butterflies and a Stockham
-// (self-sorting) pass over a tile of pencils held in shared memory.
+// Device FFT building blocks: radix-2/3/4/5/8 butterflies.
 //
 // Sign convention: S = -1 is the forward transform (kernel exp(-2 pi i nk/N)),
 // S = +1 the inverse; neither is normalised.
-//
-// Stockham decimation-in-time, mixed radix: after the passes with radices
-// R_1..R_{p-1} (product Ns), pass p with radix R reads element j + r*N/R of the
-// input (r < R, j < N/R), multiplies it by exp(S 2 pi i r (j mod Ns)/(Ns R)),
-// applies the R-point DFT and writes the outputs to
-// (j div Ns)*Ns*R + (j mod Ns) + r*Ns.  After the last pass the data are in
-// natural order.
 #pragma once
 
 #include "common.cuh"
@@ -107,35 +99,56 @@ __host__ __device__ __forceinline__ void bfly8(cplx<T>* v) {
     v[3] = badd(e3, w3); v[7] = bsub(e3, w3);
 }
 
-template <typename T, int S>
-__host__ __device__ __forceinline__ void bfly3(cplx<T>& a0, cplx<T>& a1, cplx<T>& a2) {
-    const T h = (T)0.86602540378443864676;   // sin(2 pi / 3)
-    cplx<T> t = cadd(a1, a2), u = csub(a1, a2);
-    cplx<T> m = mk<T>(a0.x - (T)0.5 * t.x, a0.y - (T)0.5 * t.y);
-    cplx<T> v = cmul_si(cscale(u, h), S);
-    a0 = cadd(a0, t);
-    a1 = cadd(m, v);
-    a2 = csub(m, v);
+// x * C for a constant C.  In float32 the rounding residue of C is added by one more
+// multiply (as in mul_rsqrt2), so the constant's rounding does not scale the
+// field's energy by the same factor every step.
+template <typename T> __host__ __device__ __forceinline__ T mul_const(T x, double C) {
+    if constexpr (sizeof(T) == 4) {
+        const float hi = (float)C, lo = (float)(C - (double)hi);
+        return fmaf(x, hi, x * lo);
+    } else {
+        return x * (T)C;
+    }
 }
 
 template <typename T, int S>
+__host__ __device__ __forceinline__ void bfly3(cplx<T>& a0, cplx<T>& a1, cplx<T>& a2) {
+    constexpr double h = 0.86602540378443864676;   // sin(2 pi / 3)
+    cplx<T> t = badd(a1, a2), u = bsub(a1, a2);
+    cplx<T> m = mk<T>(a0.x - (T)0.5 * t.x, a0.y - (T)0.5 * t.y);
+    u = mk<T>(mul_const<T>(u.x, h), mul_const<T>(u.y, h));
+    a0 = badd(a0, t);
+    add_sub_si<cplx<T>, S>(m, u, a1, a2);
+}
+
+// x * A + y * B for constants A, B, with their rounding residues in float32
+template <typename T> __host__ __device__ __forceinline__ T dot_const(T x, double A, T y, double B) {
+    if constexpr (sizeof(T) == 4) {
+        const float ah = (float)A, al = (float)(A - (double)ah), bh = (float)B, bl = (float)(B - (double)bh);
+        return fmaf(x, ah, fmaf(y, bh, fmaf(x, al, y * bl)));
+    } else {
+        return x * (T)A + y * (T)B;
+    }
+}
+
+// 5-point DFT: the even part as a0 - t/4 +- (sqrt 5 / 4)(t1 - t2), t = t1 + t2 (one
+// constant instead of cos(2 pi / 5) and cos(4 pi / 5)).
+template <typename T, int S>
 __host__ __device__ __forceinline__ void bfly5(cplx<T>* a) {
-    const T c1 = (T)0.30901699437494742410;    // cos(2 pi / 5)
-    const T c2 = (T)-0.80901699437494742410;   // cos(4 pi / 5)
-    const T s1 = (T)0.95105651629515357212;    // sin(2 pi / 5)
-    const T s2 = (T)0.58778525229247312917;    // sin(4 pi / 5)
-    cplx<T> t1 = cadd(a[1], a[4]), t2 = cadd(a[2], a[3]);
-    cplx<T> u1 = csub(a[1], a[4]), u2 = csub(a[2], a[3]);
-    cplx<T> a0 = a[0];
-    cplx<T> p1 = mk<T>(a0.x + c1 * t1.x + c2 * t2.x, a0.y + c1 * t1.y + c2 * t2.y);
-    cplx<T> p2 = mk<T>(a0.x + c2 * t1.x + c1 * t2.x, a0.y + c2 * t1.y + c1 * t2.y);
-    cplx<T> q1 = cmul_si(mk<T>(s1 * u1.x + s2 * u2.x, s1 * u1.y + s2 * u2.y), S);
-    cplx<T> q2 = cmul_si(mk<T>(s2 * u1.x - s1 * u2.x, s2 * u1.y - s1 * u2.y), S);
-    a[0] = cadd(a0, cadd(t1, t2));
-    a[1] = cadd(p1, q1);
-    a[4] = csub(p1, q1);
-    a[2] = cadd(p2, q2);
-    a[3] = csub(p2, q2);
+    constexpr double q5 = 0.55901699437494742410;   // sqrt(5) / 4
+    constexpr double s1 = 0.95105651629515357212;    // sin(2 pi / 5)
+    constexpr double s2 = 0.58778525229247312917;    // sin(4 pi / 5)
+    cplx<T> t1 = badd(a[1], a[4]), t2 = badd(a[2], a[3]);
+    cplx<T> u1 = bsub(a[1], a[4]), u2 = bsub(a[2], a[3]);
+    cplx<T> t = badd(t1, t2), d = bsub(t1, t2);
+    cplx<T> m = mk<T>(a[0].x - (T)0.25 * t.x, a[0].y - (T)0.25 * t.y);
+    cplx<T> e = mk<T>(mul_const<T>(d.x, q5), mul_const<T>(d.y, q5));
+    cplx<T> p1 = badd(m, e), p2 = bsub(m, e);
+    cplx<T> q1 = mk<T>(dot_const<T>(u1.x, s1, u2.x, s2), dot_const<T>(u1.y, s1, u2.y, s2));
+    cplx<T> q2 = mk<T>(dot_const<T>(u1.x, s2, u2.x, -s1), dot_const<T>(u1.y, s2, u2.y, -s1));
+    a[0] = badd(a[0], t);
+    add_sub_si<cplx<T>, S>(p1, q1, a[1], a[4]);
+    add_sub_si<cplx<T>, S>(p2, q2, a[2], a[3]);
 }
 
 template <typename T, int R, int S>
@@ -146,99 +159,5 @@ __host__ __device__ __forceinline__ void dft_r(cplx<T>* v) {
     else if constexpr (R == 5) bfly5<T, S>(v);
     else if constexpr (R == 8) bfly8<T, S>(v);
 }
-
-// Shared-memory layout of a tile of W pencils: element i of pencil w sits at
-// w * P + pad32(i), pad32(i) = i + i / 32.  The one unused slot per 32 elements
-// spreads the stride-R stores of the early Stockham passes (R consecutive
-// outputs per thread) over the banks, and the pencil stride P (odd, at least
-// pad32(N - 1) + 1) keeps the row-by-row tile loads of strided axes on
-// distinct banks.
-__host__ __device__ __forceinline__ int pad32(int i) { return i + (i >> 5); }
-__host__ __device__ __forceinline__ int pencil_stride(int N) { return (N + ((N - 1) >> 5)) | 1; }
-
-// Division by a per-pass constant d as a multiply-high: q = umulhi(n, m) with
-// m = ceil(2^32 / d) equals n / d for 0 <= n < 2^16 and 1 <= d < 2^16 (the
-// error term n (m - 2^32/d) / 2^32 < 2^-16 stays below the gap 1/d to the next
-// integer); d = 1 is taken apart.  For d >= 2, ceil(2^32 / d) = (2^32 - 1) / d
-// + 1 (a 32-bit division, once per pass).
-struct FastDiv {
-    unsigned m;
-    int d;
-};
-__host__ __device__ __forceinline__ FastDiv fast_div(int d) {
-    FastDiv f;
-    f.d = d;
-    f.m = d <= 1 ? 0u : 0xFFFFFFFFu / (unsigned)d + 1u;
-    return f;
-}
-#ifdef __CUDACC__
-__device__ __forceinline__ int fdiv(int n, const FastDiv& f) {
-    return f.d <= 1 ? n : (int)__umulhi((unsigned)n, f.m);
-}
-
-// One Stockham pass over `W` pencils of length N (layout above) in `in`,
-// written to `out`.  Work items b = tid, tid + nthr, ... < W*N/R (fewer than
-// 2^16).  tw[t] = exp(-2 pi i t / N); the inverse uses its conjugate.
-template <typename T, int R, int S>
-__device__ __forceinline__ void stockham_pass(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, int N,
-                                              int Ns, int W, int P, const cplx<T>* __restrict__ tw, int tid,
-                                              int nthr) {
-    const int nb = N / R;
-    const int tstride = N / (Ns * R);
-    const FastDiv dnb = fast_div(nb), dns = fast_div(Ns);
-    for (int b = tid; b < W * nb; b += nthr) {
-        const int w = fdiv(b, dnb);
-        const int j = b - w * nb;
-        const cplx<T>* src = in + (size_t)w * P;
-        cplx<T>* dst = out + (size_t)w * P;
-        cplx<T> v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = src[pad32(j + r * nb)];
-        const int jq = fdiv(j, dns);
-        const int k = j - jq * Ns;
-        if (Ns > 1) {
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                const cplx<T> wv = tw[PSATD_IX((r * k) * tstride, N)];
-                v[r] = (S < 0) ? cmul(v[r], wv) : cmulc(v[r], wv);
-            }
-        }
-        dft_r<T, R, S>(v);
-        const int idx = jq * Ns * R + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) dst[pad32(idx + r * Ns)] = v[r];
-    }
-}
-
-template <typename T, int S>
-__device__ __forceinline__ void stockham_dispatch(int R, const cplx<T>* in, cplx<T>* out, int N, int Ns, int W,
-                                                  int P, const cplx<T>* tw, int tid, int nthr) {
-    switch (R) {
-        case 2: stockham_pass<T, 2, S>(in, out, N, Ns, W, P, tw, tid, nthr); break;
-        case 3: stockham_pass<T, 3, S>(in, out, N, Ns, W, P, tw, tid, nthr); break;
-        case 4: stockham_pass<T, 4, S>(in, out, N, Ns, W, P, tw, tid, nthr); break;
-        case 5: stockham_pass<T, 5, S>(in, out, N, Ns, W, P, tw, tid, nthr); break;
-        default: stockham_pass<T, 8, S>(in, out, N, Ns, W, P, tw, tid, nthr); break;
-    }
-}
-#endif
-
-#ifdef __CUDACC__
-// Full transform of a shared-memory tile, ping-ponging between a and b.
-// Returns the buffer that holds the result.  Must be called by the whole block.
-template <typename T, int S>
-__device__ __forceinline__ cplx<T>* fft_tile(cplx<T>* a, cplx<T>* b, const AxisPlan& pl, int W,
-                                             int P, const cplx<T>* tw) {
-    int Ns = 1;
-    for (int p = 0; p < pl.npass; ++p) {
-        const int R = pl.radix[p];
-        stockham_dispatch<T, S>(R, a, b, pl.N, Ns, W, P, tw, threadIdx.x, blockDim.x);
-        __syncthreads();
-        cplx<T>* t = a; a = b; b = t;
-        Ns *= R;
-    }
-    return a;
-}
-#endif
 
 }  // namespace psatd

@@ -1,0 +1,267 @@
+// float32 transforms of axis lengths N = R1 R2 (both radices at most 16) with the
+// radices, the tile and every shared-memory offset fixed at compile time: the
+// two-pass case of fft_mixed.cuh, whose passes this file repeats in the same
+// arithmetic order without the run-time index arithmetic.  At run time that arithmetic
+// (divisions of the item index, strides, the dispatch over radices) was a third to a
+// half of the instructions (58, 87 and 138 a value for the x, y and k-space passes of
+// a 180 x 135 x 150 box against 39, 57 and 109 here), and with 24 warps an SM the
+// passes were bound by instruction issue and not by memory.  Measured on that box
+// (350 MB a pass), run-time passes against these: x 78 -> 59 us (5.9 TB/s), y 97 ->
+// 69 us, k-space 147 -> 126 us.
+//
+//   cols    y or z: 16 x-columns (128 bytes a row) by R1 threads, one item of each
+//           pass a thread
+//   rows    x: as many rows as give 256 threads at R1 a row
+//   kspace  z forward, the per-mode update, z inverse for the six components of 8
+//           x-columns at one y, the spectra kept digit-reversed in shared memory
+//
+// Lengths: those whose plan of radices up to 16 has two passes (two_pass_entry).
+// float64 stays with the run-time passes: it is bound by the float64 pipe.
+#pragma once
+
+#include "fft_mixed.cuh"
+#include "mode_update.cuh"
+
+namespace psatd {
+
+struct TwoPassArgs {
+    float2* data;
+    const float2* tp;                       // position-ordered twiddles, W_N^{jk} at k R2 + j
+    int axis, Nx, Ny, Nz, ncomp;
+};
+struct TwoPassModes {
+    const float *kx, *ky, *kz;
+    const ModeCoef<float>* coef;
+    int mode;
+    float scale;
+};
+struct TwoPassEntry {
+    int N, R1;
+    int cols_threads, rows_threads, rows_per_block, kspace_smem;
+    void (*cols[2])(TwoPassArgs);           // forward, inverse
+    void (*rows[2])(TwoPassArgs);
+    void (*kspace)(TwoPassArgs, TwoPassModes);
+};
+// The kernels of length N, or null.
+const TwoPassEntry* two_pass_entry(int N);
+
+#ifdef __CUDACC__
+constexpr int kTwoW = 16, kTwoKW = 8, kTwoKThreads = 256;
+
+template <int R1, int R2> struct TwoCfg {
+    static constexpr int N = R1 * R2;
+    static_assert(R1 >= R2, "the first radix is the larger");
+    static constexpr int cols_threads = (R1 * kTwoW + 31) / 32 * 32;
+    // registers: 64 a thread where the first DFT has at most 12 points, else 80
+    static constexpr int cols_blocks = (R1 <= 12 ? 1024 : 768) / cols_threads;
+    static constexpr int G = 256 / R1;                                  // rows per block
+    static constexpr int rows_threads = (G * R1 + 31) / 32 * 32;
+    static constexpr int rows_blocks = (R1 <= 12 ? 1024 : 768) / rows_threads;
+    static constexpr int run = R2 | 1, P = (R1 * run) | 1;              // row layout of fft_mixed.cuh
+};
+
+// multiply v[k] by the position-ordered twiddles W_N^{jk} (conjugated for S > 0)
+template <int S, int R1, int R2>
+__device__ __forceinline__ void two_twiddle(float2 (&v)[R1], const float2* __restrict__ tp, int j) {
+    static_for<1, R1>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const float2 w = tp[PSATD_IX(k * R2 + j, R1 * R2)];
+        v[k] = S < 0 ? cmul(v[k], w) : cmulc(v[k], w);
+    });
+}
+
+template <int R1, int R2, int S>
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::cols_threads, TwoCfg<R1, R2>::cols_blocks)
+two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
+    constexpr int W = kTwoW;
+    __shared__ float2 sm[R1 * R2 * W];
+    const unsigned ntile = (unsigned)(a.Nx + W - 1) / W, outer = a.axis == 1 ? a.Nz : a.Ny;
+    const unsigned rest = blockIdx.x / ntile, x0 = (blockIdx.x - rest * ntile) * W;
+    const unsigned comp = rest / outer, o = rest - comp * outer;
+    const size_t plane = (size_t)a.Nx * a.Ny, stride = a.axis == 1 ? (size_t)a.Nx : plane;
+    const unsigned c = threadIdx.x % W, t = threadIdx.x / W;
+    float2* base = a.data + comp * plane * a.Nz + (a.axis == 1 ? o * plane : (size_t)o * a.Nx) + x0 + c;
+    const GBuf<float2> F{a.data, (long long)a.ncomp * plane * a.Nz};
+    const bool col = x0 + c < (unsigned)a.Nx;
+    if (col && t < R2) {
+        float2 v[R1];
+        const float2* p = base + t * stride;
+        static_for<0, R1>([&](auto rc) {
+            v[decltype(rc)::value] = F.at(p, 0);
+            p += R2 * stride;
+        });
+        reg_dft<float, S, R1>(v);
+        two_twiddle<S, R1, R2>(v, a.tp, t);
+        static_for<0, R1>([&](auto rc) { sm[(decltype(rc)::value * R2 + t) * W + c] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+    if (col && t < R1) {
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = sm[(t * R2 + decltype(rc)::value) * W + c]; });
+        reg_dft<float, S, R2>(v);
+        float2* p = base + t * stride;
+        static_for<0, R2>([&](auto rc) {
+            F.at(p, 0) = v[decltype(rc)::value];
+            p += R1 * stride;
+        });
+    }
+}
+
+template <int R1, int R2, int S>
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::rows_threads, TwoCfg<R1, R2>::rows_blocks)
+two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
+    using Cfg = TwoCfg<R1, R2>;
+    constexpr int N = R1 * R2, G = Cfg::G;
+    __shared__ float2 sm[G * Cfg::P];
+    const long long rows = (long long)a.ncomp * a.Nz * a.Ny, row0 = (long long)blockIdx.x * G;
+    const int nrow = (int)min((long long)G, rows - row0);
+    float2* base = a.data + row0 * N;
+    const GBuf<float2> F{a.data, rows * N};
+    const int tid = threadIdx.x;
+    if (tid < nrow * R2) {
+        const int w = tid / R2, j = tid - w * R2;
+        const float2* p = base + w * N + j;
+        float2 v[R1];
+        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = F.at(p, decltype(rc)::value * R2); });
+        reg_dft<float, S, R1>(v);
+        two_twiddle<S, R1, R2>(v, a.tp, j);
+        float2* s = sm + w * Cfg::P + j;
+        static_for<0, R1>([&](auto rc) { s[decltype(rc)::value * Cfg::run] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+    if (tid < nrow * R1) {
+        const int w = tid / R1, u = tid - w * R1;
+        const float2* s = sm + w * Cfg::P + u * Cfg::run;
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value]; });
+        reg_dft<float, S, R2>(v);
+        float2* p = base + w * N + u;
+        static_for<0, R2>([&](auto rc) { F.at(p, decltype(rc)::value * R1) = v[decltype(rc)::value]; });
+    }
+}
+
+template <int R1, int R2>
+__global__ void __launch_bounds__(kTwoKThreads, 3)
+two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__ TwoPassModes md) {
+    constexpr int W = kTwoKW, N = R1 * R2, SLOT = N * W, TH = kTwoKThreads;
+    extern __shared__ __align__(16) unsigned char two_smem[];
+    float2* F = reinterpret_cast<float2*>(two_smem);              // [6][position][W]
+    const int Nx = a.Nx, Ny = a.Ny, tid = threadIdx.x;
+    const unsigned ntile = (unsigned)(Nx + W - 1) / W;
+    const int y = (int)(blockIdx.x / ntile), x0 = (int)(blockIdx.x - y * ntile) * W;
+    const size_t plane = (size_t)Nx * Ny, cstride = plane * N;
+    float2* base = a.data + (size_t)y * Nx + x0;
+    const GBuf<float2> G{a.data, 6LL * (long long)cstride};
+    const int nw = min(W, Nx - x0);
+
+    // forward: level 0 from the field, level 1 in place
+#pragma unroll 1
+    for (int i = tid; i < 6 * R2 * W; i += TH) {
+        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
+        if (c >= nw) continue;
+        const float2* p = base + q * cstride + j * plane + c;
+        float2 v[R1];
+        static_for<0, R1>([&](auto rc) {
+            v[decltype(rc)::value] = G.at(p, 0);
+            p += R2 * plane;
+        });
+        reg_dft<float, -1, R1>(v);
+        two_twiddle<-1, R1, R2>(v, a.tp, j);
+        float2* s = F + q * SLOT + j * W + c;
+        static_for<0, R1>([&](auto rc) { s[decltype(rc)::value * R2 * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < 6 * R1 * W; i += TH) {
+        const int c = i % W, u = i / W;                           // u = q R1 + k1: runs of R2 positions
+        if (c >= nw) continue;
+        float2* s = F + u * (R2 * W) + c;
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
+        reg_dft<float, -1, R2>(v);
+        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+
+    // the update of every mode: position k1 R2 + k2 holds k_z = k1 + R1 k2
+    const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1, ay = min(y, Ny - y);
+    const float kyv = md.ky[PSATD_IX(y, Ny)];
+    const bool spectral = md.mode == KS_ROTATE_SPECTRAL || md.mode == KS_ROTATE_SPECTRAL_PROJ;
+#pragma unroll 1
+    for (int e = tid; e < SLOT; e += TH) {
+        const int c = e % W, pos = e / W, k1 = pos / R2, n = k1 + (pos - k1 * R2) * R1;
+        if (c >= nw) continue;
+        const int ix = x0 + c, ax = min(ix, Nx - ix), az = min(n, N - n);
+        const ModeCoef<float> m =
+            md.coef[PSATD_IX(((size_t)az * Nyh + ay) * Nxh + ax, (long long)(N / 2 + 1) * Nyh * Nxh)];
+        const float nx = md.kx[PSATD_IX(ix, Nx)] * m.kinv, ny = kyv * m.kinv, nz = md.kz[PSATD_IX(n, N)] * m.kinv;
+        float2 f[6];
+        static_for<0, 6>([&](auto qc) { f[decltype(qc)::value] = F[decltype(qc)::value * SLOT + e]; });
+        mode_update<float>(&f[0], &f[1], &f[2], &f[3], &f[4], &f[5], nx, ny, nz, m.C, m.S, md.mode, md.scale);
+        if (spectral) {                                           // stored in natural order
+            float2* p = base + n * plane + c;
+            static_for<0, 6>([&](auto qc) {
+                G.at(p, 0) = f[decltype(qc)::value];
+                p += cstride;
+            });
+        } else {
+            static_for<0, 6>([&](auto qc) { F[decltype(qc)::value * SLOT + e] = f[decltype(qc)::value]; });
+        }
+    }
+    if (spectral) return;
+    __syncthreads();
+
+    // inverse: the levels backwards, level 0 to the field
+#pragma unroll 1
+    for (int i = tid; i < 6 * R1 * W; i += TH) {
+        const int c = i % W, u = i / W;
+        if (c >= nw) continue;
+        float2* s = F + u * (R2 * W) + c;
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
+        reg_dft<float, +1, R2>(v);
+        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < 6 * R2 * W; i += TH) {
+        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
+        if (c >= nw) continue;
+        const float2* s = F + q * SLOT + j * W + c;
+        float2 v[R1];
+        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * R2 * W]; });
+        two_twiddle<+1, R1, R2>(v, a.tp, j);
+        reg_dft<float, +1, R1>(v);
+        float2* p = base + q * cstride + j * plane + c;
+        static_for<0, R1>([&](auto rc) {
+            G.at(p, 0) = v[decltype(rc)::value];
+            p += R2 * plane;
+        });
+    }
+}
+
+template <int R1, int R2> TwoPassEntry two_pass_make() {
+    using Cfg = TwoCfg<R1, R2>;
+    TwoPassEntry e{};
+    e.N = R1 * R2;
+    e.R1 = R1;
+    e.cols_threads = Cfg::cols_threads;
+    e.rows_threads = Cfg::rows_threads;
+    e.rows_per_block = Cfg::G;
+    e.kspace_smem = 6 * R1 * R2 * kTwoKW * (int)sizeof(float2);
+    e.cols[0] = two_cols_kernel<R1, R2, -1>;
+    e.cols[1] = two_cols_kernel<R1, R2, +1>;
+    e.rows[0] = two_rows_kernel<R1, R2, -1>;
+    e.rows[1] = two_rows_kernel<R1, R2, +1>;
+    e.kspace = two_kspace_kernel<R1, R2>;
+    return e;
+}
+#endif
+
+// The entries of one translation unit each (fft_two_*.cu).
+const TwoPassEntry* two_pass_part0(int N);
+const TwoPassEntry* two_pass_part1(int N);
+const TwoPassEntry* two_pass_part2(int N);
+const TwoPassEntry* two_pass_part3(int N);
+
+}  // namespace psatd

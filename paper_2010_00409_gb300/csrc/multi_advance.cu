@@ -11,10 +11,10 @@
 // launch runs n steps, i.e. 5 n - 1 barriers, without returning to the host;
 // a box with fewer steps of its own skips its items in the later steps.
 //
-// Work items (the generic shared-memory Stockham tiles of fft_core.cuh, so any
-// axis length with factors 2, 3, 5 works):
+// Work items (the in-place mixed-radix passes of fft_mixed.cuh with radices up to
+// 16, so any axis length with factors 2, 3, 5 works):
 //   x: W_x consecutive rows of one box (contiguous in memory);
-//   y: W_y consecutive x-columns at one (component, z), read row by row;
+//   y: W_y consecutive x-columns at one (component, z);
 //   z: W_z consecutive x-columns at one y, all six components: forward z
 //      transforms, the update of every mode of the tile, inverse z transforms.
 // The radix schedule of each axis and the three tile widths come from the host
@@ -28,7 +28,7 @@
 // does every other block at the next barrier it cannot pass, so no block spins
 // forever.  Field loads go around L1 (cache-global) so that no block reads a
 // line another block rewrote in the previous phase.
-#include "fft_reg.cuh"
+#include "fft_mixed.cuh"
 #include "tma.cuh"
 
 namespace psatd {
@@ -79,119 +79,91 @@ __device__ bool grid_barrier(unsigned* bar, unsigned target, int* err, unsigned 
 
 // x phase: rows row0 .. row0 + nrow - 1 of the box ([6][Nz][Ny] rows of Nx).
 template <typename T, int S>
-__device__ void x_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
-    const int Nx = P.N[0], W = P.W[0], Pp = pencil_stride(Nx);
-    const long long rows = 6LL * P.N[1] * P.N[2];
-    const long long row0 = item * W;
-    const int nrow = (int)min((long long)W, rows - row0);
-    cplx<T>* A = sm;
-    cplx<T>* B = sm + (size_t)W * Pp;
-    cplx<T>* base = P.f + row0 * Nx;
-    const GBuf<cplx<T>> F{P.f, rows * Nx};
-    const int n = nrow * Nx;
-    const FastDiv dn = fast_div(Nx);
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int w = fdiv(e, dn), i = e - w * Nx;
-        A[w * Pp + pad32(i)] = __ldcg(&F.at(base, e));
-    }
-    __syncthreads();
-    const cplx<T>* res = fft_tile<T, S>(A, B, P.plan[0], nrow, Pp, P.tw[0]);
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int w = fdiv(e, dn), i = e - w * Nx;
-        F.at(base, e) = res[w * Pp + pad32(i)];
-    }
+__device__ __forceinline__ void x_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
+    const int Nx = P.N[0], W = P.W[0];
+    const long long rows = 6LL * P.N[1] * P.N[2], row0 = item * W;
+    MixTile<T> t;
+    t.base = P.f + row0 * Nx;
+    t.buf = GBuf<cplx<T>>{P.f, rows * Nx};
+    t.cstride = 0;
+    t.stride = 1;
+    t.logw = 0;
+    t.nw = (int)min((long long)W, rows - row0);
+    t.nq = 1;
+    t.slot = 0;
+    t.P = row_stride(Nx, P.plan[0].radix[0]);
+    t.run = row_run(Nx, P.plan[0].radix[0]);
+    t.gap = t.run - Nx / P.plan[0].radix[0];
+    mix_transform<T, S, kNarrow, true, true>(t, sm, P.plan[0], P.tp[0]);
 }
 
 // y phase: x-columns x0 .. x0 + nw - 1 of plane (comp, z).
 template <typename T, int S>
-__device__ void y_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
-    const int Nx = P.N[0], Ny = P.N[1], Nz = P.N[2], W = P.W[1], Pp = pencil_stride(Ny);
+__device__ __forceinline__ void y_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
+    const int Nx = P.N[0], Ny = P.N[1], Nz = P.N[2], W = P.W[1];
     const int ntile = (Nx + W - 1) / W;
-    const int t = (int)(item % ntile);
-    const long long rest = item / ntile;                      // comp * Nz + z
-    const int z = (int)(rest % Nz), comp = (int)(rest / Nz);
-    const int x0 = t * W, nw = min(W, Nx - x0);
-    const size_t plane = (size_t)Nx * Ny;
-    cplx<T>* A = sm;
-    cplx<T>* B = sm + (size_t)W * Pp;
-    cplx<T>* base = P.f + (size_t)comp * plane * Nz + (size_t)z * plane + x0;
-    const GBuf<cplx<T>> F{P.f, 6LL * (long long)plane * Nz};
-    const int n = Ny * nw;
-    const FastDiv dw = fast_div(nw);
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int r = fdiv(e, dw), w = e - r * nw;
-        A[w * Pp + pad32(r)] = __ldcg(&F.at(base, (long long)r * Nx + w));
-    }
-    __syncthreads();
-    const cplx<T>* res = fft_tile<T, S>(A, B, P.plan[1], nw, Pp, P.tw[1]);
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int r = fdiv(e, dw), w = e - r * nw;
-        F.at(base, (long long)r * Nx + w) = res[w * Pp + pad32(r)];
-    }
+    const unsigned rest = (unsigned)item / (unsigned)ntile;                   // comp * Nz + z
+    const int tile = (int)((unsigned)item - rest * ntile);
+    const long long plane = (long long)Nx * Ny;
+    const int x0 = tile * W;
+    MixTile<T> t;
+    t.base = P.f + rest * plane + x0;
+    t.buf = GBuf<cplx<T>>{P.f, 6LL * plane * Nz};
+    t.cstride = 0;
+    t.stride = Nx;
+    t.logw = 31 - __clz(W);
+    t.nw = min(W, Nx - x0);
+    t.nq = 1;
+    t.slot = 0;
+    t.P = t.run = t.gap = 0;
+    mix_transform<T, S, kNarrow, false, true>(t, sm, P.plan[1], P.tp[1]);
 }
 
-// z pass of one tile, transforming component c of F in place (scratch as the
-// Stockham partner buffer).
-template <typename T, int S>
-__device__ void z_transform(cplx<T>* Fc, cplx<T>* scratch, const MultiProblem<T>& P, int nw, int Pp) {
-    cplx<T>* res = fft_tile<T, S>(Fc, scratch, P.plan[2], nw, Pp, P.tw[2]);
-    if (res != Fc) {
-        for (int e = threadIdx.x; e < nw * Pp; e += blockDim.x) Fc[e] = scratch[e];
-        __syncthreads();
-    }
-}
-
-// z phase: x-columns x0 .. x0 + nw - 1 at one y, all six components.
+// z phase: x-columns x0 .. x0 + nw - 1 at one y, all six components: forward z
+// transforms, the update of every mode on the digit-reversed spectra, inverse z
+// transforms.
 template <typename T>
-__device__ void z_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
-    const int Nx = P.N[0], Ny = P.N[1], Nz = P.N[2], W = P.W[2], Pp = pencil_stride(Nz);
+__device__ __forceinline__ void z_tile(const MultiProblem<T>& P, long long item, cplx<T>* sm) {
+    const int Nx = P.N[0], Ny = P.N[1], Nz = P.N[2], W = P.W[2], logw = 31 - __clz(W);
     const int ntile = (Nx + W - 1) / W;
-    const int t = (int)(item % ntile);
-    const int y = (int)(item / ntile);
-    const int x0 = t * W, nw = min(W, Nx - x0);
-    const size_t plane = (size_t)Nx * Ny, cstride = plane * Nz, ct = (size_t)W * Pp;
-    cplx<T>* F = sm;                                          // [6][W][Pp]
-    cplx<T>* scratch = sm + 6 * ct;                           // [W][Pp]
-    cplx<T>* base = P.f + (size_t)y * Nx + x0;
-    const GBuf<cplx<T>> G{P.f, 6LL * (long long)cstride};
-    const int n = Nz * nw;
-    const FastDiv dw = fast_div(nw), dz = fast_div(Nz);
-    for (int c = 0; c < 6; ++c)
-        for (int e = threadIdx.x; e < n; e += blockDim.x) {
-            const int r = fdiv(e, dw), w = e - r * nw;
-            F[c * ct + w * Pp + pad32(r)] = __ldcg(&G.at(base, c * cstride + (size_t)r * plane + w));
-        }
-    __syncthreads();
-    for (int c = 0; c < 6; ++c) z_transform<T, -1>(F + c * ct, scratch, P, nw, Pp);
+    const int y = (int)((unsigned)item / (unsigned)ntile), tile = (int)item - y * ntile, x0 = tile * W, ct = Nz << logw;
+    const long long plane = (long long)Nx * Ny, cstride = plane * Nz;
+    MixTile<T> t;
+    t.base = P.f + (long long)y * Nx + x0;
+    t.buf = GBuf<cplx<T>>{P.f, 6LL * cstride};
+    t.cstride = cstride;
+    t.stride = plane;
+    t.logw = logw;
+    t.nw = min(W, Nx - x0);
+    t.nq = 6;
+    t.slot = ct;
+    t.P = t.run = t.gap = 0;
+    mix_forward<T, kNarrow, true>(t, sm, P.plan[2], P.tp[2]);
 
     const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1;
     const int ay = min(y, Ny - y);
     const T ky = P.k[1][PSATD_IX(y, Ny)];
     const long long ncoef = (long long)(Nz / 2 + 1) * Nyh * Nxh;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int w = fdiv(e, dz), r = e - w * Nz;
-        const int ix = x0 + w;
-        const int ax = min(ix, Nx - ix), az = min(r, Nz - r);
+    for (int e = threadIdx.x; e < ct; e += blockDim.x) {
+        const int c = e & (W - 1), n = mix_frequency(P.plan[2], e >> logw);
+        if (c >= t.nw) continue;
+        const int ix = x0 + c;
+        const int ax = min(ix, Nx - ix), az = min(n, Nz - n);
         const ModeCoef<T> m = P.coef[PSATD_IX(((size_t)az * Nyh + ay) * Nxh + ax, ncoef)];
-        cplx<T>* o = F + w * Pp + pad32(r);
+        cplx<T>* o = sm + e;
         cplx<T> Ex = o[0], Ey = o[ct], Ez = o[2 * ct], Bx = o[3 * ct], By = o[4 * ct], Bz = o[5 * ct];
         rotate_mode<T>(Ex, Ey, Ez, Bx, By, Bz, P.k[0][PSATD_IX(ix, Nx)] * m.kinv, ky * m.kinv,
-                       P.k[2][PSATD_IX(r, Nz)] * m.kinv, m.C, m.S);
+                       P.k[2][PSATD_IX(n, Nz)] * m.kinv, m.C, m.S);
         o[0] = Ex; o[ct] = Ey; o[2 * ct] = Ez;
         o[3 * ct] = Bx; o[4 * ct] = By; o[5 * ct] = Bz;
     }
     __syncthreads();
-    for (int c = 0; c < 6; ++c) z_transform<T, +1>(F + c * ct, scratch, P, nw, Pp);
-
-    for (int c = 0; c < 6; ++c)
-        for (int e = threadIdx.x; e < n; e += blockDim.x) {
-            const int r = fdiv(e, dw), w = e - r * nw;
-            G.at(base, c * cstride + (size_t)r * plane + w) = F[c * ct + w * Pp + pad32(r)];
-        }
+    mix_inverse<T, kNarrow>(t, sm, P.plan[2], P.tp[2]);
 }
 
+// float32: three blocks per SM (85 registers a thread, tiles of at most 72 KB)
 template <typename T>
-__global__ void __launch_bounds__(kMT)
+__global__ void __launch_bounds__(kMT, sizeof(T) == 4 ? 3 : 2)
 multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long* __restrict__ prefix, int nprob,
                      int nsteps, unsigned* bar, unsigned long long* ticket, int* err, unsigned long long limit_ns,
                      unsigned extra) {
@@ -210,12 +182,16 @@ multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long*
             // items are handed out one at a time from a global ticket counter, so
             // blocks that drew cheap items (small boxes) take more of them; every
             // block stops at its first ticket past the phase, so the phase uses
-            // exactly total + gridDim.x tickets
+            // exactly total + gridDim.x tickets.  Thread 0 draws the next ticket when
+            // an item begins, so the counter's round trip (about 1 us against 2 to 3 us
+            // for a tile) is over when the item ends.
+            unsigned long long drawn = 0;
+            if (threadIdx.x == 0) s_item = (long long)(atomicAdd(ticket, 1ull) - base);
+            __syncthreads();
             for (;;) {
-                if (threadIdx.x == 0) s_item = (long long)(atomicAdd(ticket, 1ull) - base);
-                __syncthreads();
                 const long long g = s_item;
                 if (g >= total) break;
+                if (threadIdx.x == 0) drawn = atomicAdd(ticket, 1ull);
                 int lo = 0, hi = nprob - 1;                     // the box p with pre[p] <= g < pre[p + 1]
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
@@ -237,8 +213,11 @@ multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long*
                     else if (ph == 3) y_tile<T, +1>(*P, item, tile);
                     else x_tile<T, +1>(*P, item, tile);
                 }
-                __syncthreads();                                // the next item reuses s_item, the descriptor and tile
+                __syncthreads();                                // every thread has read s_item, the descriptor and the tile
+                if (threadIdx.x == 0) s_item = (long long)(drawn - base);
+                __syncthreads();
             }
+            __syncthreads();                                    // s_item is read before the next phase writes it
             base += (unsigned long long)total + gridDim.x;
             if (s == nsteps - 1 && ph == 4) return;
             ++nbar;
@@ -250,9 +229,9 @@ multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long*
 }  // namespace
 
 template <typename T>
-size_t multi_tile_bytes(int axis, int N_axis, int W) {
+size_t multi_tile_bytes(int axis, const AxisPlan& pl, int W) {
     const size_t es = sizeof(cplx<T>);
-    return (axis == 2 ? 7 : 2) * (size_t)W * pencil_stride(N_axis) * es;
+    return (size_t)W * es * (axis == 0 ? (size_t)row_stride(pl.N, pl.radix[0]) : (size_t)(axis == 2 ? 6 : 1) * pl.N);
 }
 
 template <typename T>
@@ -287,8 +266,8 @@ cudaError_t launch_multi_advance(const MultiProblem<T>* probs, const long long* 
     return cudaLaunchKernelEx(&cfg, k, probs, prefix, nprob, nsteps, bar, ticket, err, limit_ns, extra);
 }
 
-template size_t multi_tile_bytes<float>(int, int, int);
-template size_t multi_tile_bytes<double>(int, int, int);
+template size_t multi_tile_bytes<float>(int, const AxisPlan&, int);
+template size_t multi_tile_bytes<double>(int, const AxisPlan&, int);
 template cudaError_t launch_multi_advance<float>(const MultiProblem<float>*, const long long*, int, int, size_t,
                                                  long long, unsigned*, int*, unsigned long long, unsigned,
                                                  cudaStream_t, int*);

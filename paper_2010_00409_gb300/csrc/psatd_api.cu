@@ -19,6 +19,8 @@
 
 #include "../../include/psatd.h"
 #include "common.cuh"
+#include "fft_mixed.cuh"
+#include "fft_two.cuh"
 #include "tma.cuh"
 
 using namespace psatd;
@@ -29,18 +31,67 @@ namespace psatd {
 void debug_register_reader(long long (*reader)(long long*, long long*));
 #endif
 
-bool make_plan(int N, AxisPlan* p) {
-    p->N = N;
-    p->npass = 0;
-    int n = N;
-    const int rs[5] = {8, 4, 5, 3, 2};
-    for (int r : rs) {
-        while (n % r == 0 && p->npass < kMaxPass) {
-            p->radix[p->npass++] = r;
-            n /= r;
+namespace {
+const int kRadices[] = {32, 30, 27, 25, 24, 20, 18, 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+
+// Extend cur (radices so far, non-increasing) by a factorisation of n; best keeps
+// the fewest passes, then the smallest largest radix, then the smallest sum.
+void search_plan(int n, int max_radix, AxisPlan* cur, int sum, AxisPlan* best, int* best_sum) {
+    if (n == 1) {
+        const bool first = best->npass == 0;
+        if (first || cur->npass < best->npass ||
+            (cur->npass == best->npass && (cur->radix[0] < best->radix[0] ||
+                                           (cur->radix[0] == best->radix[0] && sum < *best_sum)))) {
+            *best = *cur;
+            *best_sum = sum;
         }
+        return;
     }
-    return n == 1;
+    if (cur->npass >= (best->npass ? best->npass : kMaxPass)) return;
+    for (int r : kRadices) {
+        if (r > max_radix || n % r) continue;
+        cur->radix[cur->npass++] = r;
+        search_plan(n / r, r, cur, sum + r, best, best_sum);
+        --cur->npass;
+    }
+}
+
+std::vector<AxisPlan> plan_table(int max_radix) {
+    std::vector<AxisPlan> t(2049);
+    for (int N = 0; N <= 2048; ++N) {
+        AxisPlan cur{}, best{};
+        int n = N, sum = 0;
+        for (int f : {2, 3, 5})
+            while (n > 1 && n % f == 0) n /= f;
+        cur.N = best.N = N;
+        if (N == 1) {
+            best.npass = 1;
+            best.radix[0] = 1;
+        } else if (N > 1 && n == 1) {
+            search_plan(N, max_radix, &cur, 0, &best, &sum);
+        }
+        finish_plan(&best);
+        t[N] = best;
+    }
+    return t;
+}
+}  // namespace
+
+void finish_plan(AxisPlan* p) {
+    int M = p->N;
+    for (int i = 0; i < p->npass; ++i) {
+        p->div_nb[i] = div_multiplier(p->N / p->radix[i]);
+        p->div_l[i] = div_multiplier(M / p->radix[i]);
+        M /= p->radix[i];
+    }
+    p->div_run = p->npass ? div_multiplier(p->N / p->radix[0]) : 0u;
+}
+
+bool make_plan(int N, AxisPlan* p, int max_radix) {
+    static const std::vector<AxisPlan> t16 = plan_table(16), t20 = plan_table(20), t32 = plan_table(32);
+    if (N < 1 || N > 2048) return false;
+    *p = (max_radix >= 32 ? t32 : max_radix >= 20 ? t20 : t16)[N];
+    return p->npass > 0;
 }
 
 }  // namespace psatd
@@ -102,6 +153,10 @@ struct psatd_ctx {
 
     // tables (device)
     DevBuf tw[3], k[3], coef;
+    // position-ordered twiddles of the context's plan, then of the batched advance's
+    // radix schedules (values from each one's start)
+    DevBuf twp[3];
+    int twp_at[3][3] = {{0}};
     AxisPlan plan[3];
 
     // longitudinal profile of PSATD_PULSE_PROFILE pulses (psatd_set_pulse_profile)
@@ -271,10 +326,23 @@ Tables<T> tables(const psatd_ctx* c) {
         tb.tw[a] = static_cast<const cplx<T>*>(c->tw[a].p);
         tb.k[a] = static_cast<const T*>(c->k[a].p);
         tb.plan[a] = c->plan[a];
+        tb.twp[a] = static_cast<const cplx<T>*>(c->twp[a].p) + c->twp_at[a][0];
     }
     tb.coef = static_cast<const ModeCoef<T>*>(c->coef.p);
     for (int a = 0; a < 3; ++a) tb.tw2[a] = static_cast<const cplx<T>*>(c->tw2[a].p);
     return tb;
+}
+
+// Radix schedules the batch autotuner chooses from for an axis of N points: the
+// radices of make_plan (up to 16) largest first (0) or smallest first (1).
+constexpr int kPlanVariants = 2;
+bool make_plan_variant(int N, int variant, AxisPlan* p) {
+    if (!make_plan(N, p)) return false;
+    if (variant & 1) {
+        std::reverse(p->radix, p->radix + p->npass);
+        finish_plan(p);
+    }
+    return true;
 }
 
 int axis_n(const psatd_grid& g, int a) { return a == 0 ? g.Nx : (a == 1 ? g.Ny : g.Nz); }
@@ -304,6 +372,24 @@ psatd_status upload_axis_tables(psatd_ctx* c) {
         CK(c, ensure_buf(c->k[a], N * sizeof(T)));
         CK(c, cudaMemcpy(c->tw[a].p, tw.data(), N * sizeof(cplx<T>), cudaMemcpyHostToDevice));
         CK(c, cudaMemcpy(c->k[a].p, k.data(), N * sizeof(T), cudaMemcpyHostToDevice));
+        // position-ordered twiddles: level p (blocks of M, radix R, L = M / R) holds
+        // W_M^{jk} at k L + j
+        std::vector<cplx<T>> tp;
+        for (int v = -1; v < kPlanVariants; ++v) {
+            AxisPlan pl = c->plan[a];
+            if (v >= 0) make_plan_variant(N, v, &pl);
+            c->twp_at[a][v + 1] = (int)tp.size();
+            int M = N;
+            for (int p = 0; p + 1 < pl.npass; ++p) {
+                const int R = pl.radix[p], L = M / R;
+                for (int kk = 0; kk < R; ++kk)
+                    for (int j = 0; j < L; ++j) tp.push_back(tw[(size_t)j * kk % M * (N / M)]);
+                M = L;
+            }
+        }
+        if (tp.empty()) tp.push_back(tw[0]);
+        CK(c, ensure_buf(c->twp[a], tp.size() * sizeof(cplx<T>)));
+        CK(c, cudaMemcpy(c->twp[a].p, tp.data(), tp.size() * sizeof(cplx<T>), cudaMemcpyHostToDevice));
         if (N == 512 || N == 1024) {
             // the register kernels read W^{i j} for i, j < 32 along a thread-indexed j
             std::vector<cplx<T>> t2(32 * 32);
@@ -482,6 +568,58 @@ psatd_status check_device_error(psatd_ctx* c) {
     return PSATD_OK;
 }
 
+}  // namespace
+
+const TwoPassEntry* psatd::two_pass_entry(int N) {
+    const TwoPassEntry* e = two_pass_part0(N);
+    if (!e) e = two_pass_part1(N);
+    if (!e) e = two_pass_part2(N);
+    if (!e) e = two_pass_part3(N);
+    return e;
+}
+
+namespace {
+
+// The compile-time two-pass transform of one axis; cudaErrorNotSupported (nothing
+// launched) for float64 and lengths without one.
+template <typename T>
+cudaError_t fft_axis_two(cplx<T>* data, int ncomp, const GridGeom& g, const Tables<T>& tb, int axis, int dir,
+                         cudaStream_t s) {
+    if constexpr (sizeof(T) == 4) {
+        const AxisPlan& pl = tb.plan[axis];
+        const TwoPassEntry* e = two_pass_entry(pl.N);
+        if (!e || pl.npass != 2 || pl.radix[0] != e->R1) return cudaErrorNotSupported;
+        const TwoPassArgs a{data, tb.twp[axis], axis, g.Nx, g.Ny, g.Nz, ncomp};
+        const long long blocks =
+            axis == 0 ? ((long long)ncomp * g.Nz * g.Ny + e->rows_per_block - 1) / e->rows_per_block
+                      : (long long)ncomp * (axis == 1 ? g.Nz : g.Ny) * ((g.Nx + 15) / 16);
+        if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+        void* args[] = {const_cast<TwoPassArgs*>(&a)};
+        const void* k = reinterpret_cast<const void*>(axis == 0 ? e->rows[dir > 0] : e->cols[dir > 0]);
+        return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(axis == 0 ? e->rows_threads : e->cols_threads), args, 0, s);
+    }
+    return cudaErrorNotSupported;
+}
+
+// The compile-time fused k-space pass (any KspaceMode), as above.
+template <typename T>
+cudaError_t kspace_two(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, int mode, double scale, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4) {
+        const AxisPlan& pl = tb.plan[2];
+        const TwoPassEntry* e = two_pass_entry(pl.N);
+        if (!e || pl.npass != 2 || pl.radix[0] != e->R1) return cudaErrorNotSupported;
+        const TwoPassArgs a{data, tb.twp[2], 2, g.Nx, g.Ny, g.Nz, 6};
+        const TwoPassModes m{tb.k[0], tb.k[1], tb.k[2], tb.coef, mode, (float)scale};
+        const void* k = reinterpret_cast<const void*>(e->kspace);
+        const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, e->kspace_smem);
+        if (r != cudaSuccess) return r;
+        void* args[] = {const_cast<TwoPassArgs*>(&a), const_cast<TwoPassModes*>(&m)};
+        return cudaLaunchKernel(k, dim3((unsigned)((long long)g.Ny * ((g.Nx + 7) / 8))), dim3(256), args,
+                                (size_t)e->kspace_smem, s);
+    }
+    return cudaErrorNotSupported;
+}
+
 template <typename T>
 cudaError_t fft_axis(psatd_ctx* c, cplx<T>* data, int ncomp, int axis, int dir, int kind) {
     const GridGeom g = geom(c);
@@ -490,6 +628,7 @@ cudaError_t fft_axis(psatd_ctx* c, cplx<T>* data, int ncomp, int axis, int dir, 
     return timed(c, kind < 0 ? axis : kind, [&] {
         if (c->kernel_path != PSATD_PATH_GENERIC) {
             cudaError_t e = launch_fft_axis_fast<T>(data, ncomp, g, tb, axis, dir, c->stream);
+            if (e == cudaErrorNotSupported) e = fft_axis_two<T>(data, ncomp, g, tb, axis, dir, c->stream);
             if (e != cudaErrorNotSupported) {
                 ++c->launches;
                 return e;
@@ -609,6 +748,13 @@ cudaError_t spectral_pass(psatd_ctx* c, int mode, double scale) {
                 return r;
             }
         }
+        if (c->kernel_path != PSATD_PATH_GENERIC) {
+            cudaError_t r = kspace_two<T>(f, g, tb, mode, scale, c->stream);
+            if (r != cudaErrorNotSupported) {
+                ++c->launches;
+                return r;
+            }
+        }
         return launch_kspace_z<T>(f, g, tb, mode, scale, c->stream, &c->launches);
     });
     if (e != cudaSuccess) return e;
@@ -709,6 +855,11 @@ cudaError_t one_shot_spectrum(psatd_ctx* c, bool project_b) {
             cudaError_t r = launch_kspace_tma<T>(c->field_map, f, g, tb, c->dev_err, c->stream, true, project_b);
             if (r != cudaErrorNotSupported) return r;
         }
+        if (c->kernel_path != PSATD_PATH_GENERIC) {
+            cudaError_t r = kspace_two<T>(f, g, tb, project_b ? KS_ROTATE_SPECTRAL_PROJ : KS_ROTATE_SPECTRAL, 0.0,
+                                          c->stream);
+            if (r != cudaErrorNotSupported) return r;
+        }
         --c->launches;
         return launch_kspace_z<T>(f, g, tb, project_b ? KS_ROTATE_SPECTRAL_PROJ : KS_ROTATE_SPECTRAL, 0.0,
                                   c->stream, &c->launches);
@@ -719,29 +870,6 @@ cudaError_t one_shot_spectrum(psatd_ctx* c, bool project_b) {
 // ---------------------------------------------------------------------------
 // Persistent batched advance (multi_advance.cu)
 
-// Radix schedules the batch autotuner chooses from for an axis of N points:
-// 0 radices 8, 4, 5, 3, 2 largest first (make_plan), 1 the same radices smallest
-// first, 2 radices 4, 5, 3, 2 (no 8) largest first, 3 those smallest first.
-constexpr int kPlanVariants = 4;
-bool make_plan_variant(int N, int variant, AxisPlan* p) {
-    AxisPlan q;
-    q.N = N;
-    q.npass = 0;
-    int n = N;
-    static const int with8[5] = {8, 4, 5, 3, 2}, no8[4] = {4, 5, 3, 2};
-    const int* rs = (variant & 2) ? no8 : with8;
-    const int nr = (variant & 2) ? 4 : 5;
-    for (int i = 0; i < nr; ++i)
-        while (n % rs[i] == 0 && q.npass < kMaxPass) {
-            q.radix[q.npass++] = rs[i];
-            n /= rs[i];
-        }
-    if (n != 1) return false;
-    if (variant & 1) std::reverse(q.radix, q.radix + q.npass);
-    *p = q;
-    return true;
-}
-
 bool same_plan(const AxisPlan& a, const AxisPlan& b) {
     if (a.N != b.N || a.npass != b.npass) return false;
     for (int i = 0; i < a.npass; ++i)
@@ -749,13 +877,10 @@ bool same_plan(const AxisPlan& a, const AxisPlan& b) {
     return true;
 }
 
-// Shared-memory budget of one tile: four blocks of 256 threads per SM in
-// float32 (64 registers a thread), two in float64 (more registers).
-#ifndef PSATD_MULTI_BUDGET_F32
-#define PSATD_MULTI_BUDGET_F32 (56 * 1024)
-#endif
+// Shared-memory budget of one tile: three blocks of 256 threads per SM in float32
+// (85 registers a thread), two in float64 (more registers).
 template <typename T> constexpr size_t multi_tile_budget() {
-    return sizeof(T) == 4 ? (size_t)(PSATD_MULTI_BUDGET_F32) : (size_t)(100 * 1024);
+    return sizeof(T) == 4 ? (size_t)(72 * 1024) : (size_t)(100 * 1024);
 }
 constexpr size_t kMultiHeader = 256;              // barrier counter at the start of the batch buffer
 constexpr int kMultiMaxN = 1024;
@@ -775,17 +900,21 @@ MultiChoice multi_choice(int prec, int N) {
     return it == g_multi_tuned.end() ? MultiChoice{} : it->second;
 }
 
-// Tile width of the phase along `axis`: x rows (~2048 points per tile), y
-// x-columns (128 contiguous bytes per row), z x-columns (64 bytes, six
-// components held), scaled by 2^scale and halved until the tile fits.
+// Tile width of the phase along `axis`: x rows (about 256 first-pass items per
+// tile), y x-columns (128 contiguous bytes per row), z x-columns (64 bytes, six
+// components held), scaled by 2^scale and halved until the tile fits; the column
+// counts are powers of two.
 template <typename T>
-int multi_width(int axis, const psatd_grid& g, int scale) {
+int multi_width(int axis, const psatd_grid& g, const AxisPlan& pl, int scale) {
     const int es = (int)sizeof(cplx<T>);
     const int N = axis_n(g, axis);
-    int w = axis == 0 ? std::max(1, std::min(64, 2048 / std::max(N, 1))) : std::min(g.Nx, (axis == 1 ? 128 : 64) / es);
+    int w = 1;
+    if (axis == 0) w = std::max(1, std::min(128, 256 * pl.radix[0] / std::max(N, 1)));
+    else
+        while (w < g.Nx && w < (axis == 1 ? 128 : 64) / es) w *= 2;
     w = scale > 0 ? (w << scale) : (scale < 0 ? (w >> -scale) : w);
-    w = std::max(1, std::min(w, axis == 0 ? 128 : g.Nx));
-    while (w > 1 && multi_tile_bytes<T>(axis, N, w) > multi_tile_budget<T>()) w /= 2;
+    w = std::max(1, std::min(w, axis == 0 ? 256 : 32));
+    while (w > 1 && multi_tile_bytes<T>(axis, pl, w) > multi_tile_budget<T>()) w /= 2;
     return w;
 }
 
@@ -815,7 +944,6 @@ psatd_status multi_prepare(psatd_ctx* const* ctxs, int n, const int* steps, void
         P.coef = static_cast<const ModeCoef<T>*>(c->coef.p);
         P.nsteps = steps[p];
         for (int a = 0; a < 3; ++a) {
-            P.tw[a] = static_cast<const cplx<T>*>(c->tw[a].p);
             P.k[a] = static_cast<const T*>(c->k[a].p);
             P.N[a] = axis_n(c->grid, a);
             MultiChoice ch = multi_choice(c->prec, P.N[a]);
@@ -823,9 +951,10 @@ psatd_status multi_prepare(psatd_ctx* const* ctxs, int n, const int* steps, void
                 auto it = choice->find(P.N[a]);
                 if (it != choice->end()) ch = it->second;
             }
-            if (!make_plan_variant(P.N[a], ch.variant, &P.plan[a])) make_plan(P.N[a], &P.plan[a]);
-            P.W[a] = multi_width<T>(a, c->grid, ch.scale);
-            tile = std::max(tile, multi_tile_bytes<T>(a, P.N[a], P.W[a]));
+            make_plan_variant(P.N[a], ch.variant, &P.plan[a]);
+            P.tp[a] = static_cast<const cplx<T>*>(c->twp[a].p) + c->twp_at[a][1 + (ch.variant & 1)];
+            P.W[a] = multi_width<T>(a, c->grid, P.plan[a], ch.scale);
+            tile = std::max(tile, multi_tile_bytes<T>(a, P.plan[a], P.W[a]));
         }
         const long long Nx = P.N[0], Ny = P.N[1], Nz = P.N[2];
         const long long items[3] = {(6 * Nz * Ny + P.W[0] - 1) / P.W[0], 6 * Nz * ((Nx + P.W[1] - 1) / P.W[1]),
@@ -962,7 +1091,14 @@ psatd_status psatd_init_grid(const psatd_grid* grid, const psatd_mapping* mappin
     c->prec = precision;
     c->real_fields = real;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
-    for (int a = 0; a < 3; ++a) make_plan(Ns[a], &c->plan[a]);
+    // radices beyond 16 only where they save a pass; float64 stops at 20 (a register
+    // DFT of more points would not fit the register file)
+    for (int a = 0; a < 3; ++a) {
+        AxisPlan wide;
+        make_plan(Ns[a], &c->plan[a]);
+        make_plan(Ns[a], &wide, precision == 64 ? 20 : 32);
+        if (wide.npass < c->plan[a].npass) c->plan[a] = wide;
+    }
 
     cudaError_t e = cudaGetDevice(&c->device);
     psatd_status st = PSATD_OK;
@@ -1005,7 +1141,7 @@ void psatd_destroy(psatd_ctx* c) {
     else cudaDeviceSynchronize();
     if (c->own_fields && c->fields) lib_free(c->fields);
     if (c->dev_err) lib_free(c->dev_err);
-    for (int a = 0; a < 3; ++a) { free_buf(c->tw[a]); free_buf(c->k[a]); }
+    for (int a = 0; a < 3; ++a) { free_buf(c->tw[a]); free_buf(c->k[a]); free_buf(c->twp[a]); }
     free_buf(c->coef);
     free_buf(c->coef_T);
     free_buf(c->coef_proj);
