@@ -16,20 +16,23 @@
 // per-mode complex mixing, GELU, the bias sums, the MSE loss and Adam are small
 // elementwise / reduction kernels.  Tensors are float32; GEMM tiles are rounded
 // to bfloat16 (float32 accumulation).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <new>
 #include <random>
 #include <string>
+#include <utility>
 #include <vector>
+
+#include <cuda_bf16.h>
 
 #include "../../include/psatd.h"
 #include "common.cuh"
+#include "ff.cuh"
 
 namespace psatd {
-
-
 
 namespace {
 
@@ -72,35 +75,236 @@ __global__ void bias_act_kernel(float* z, float* a, const float* __restrict__ bi
     }
 }
 
-// g_z = g_a * act'(z); g_z may be g_a
-__global__ void act_back_kernel(const float* __restrict__ z, const float* ga, float* gz,
-                                long long n, int use_gelu) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-        gz[e] = use_gelu ? ga[e] * gelu_grad(z[e]) : ga[e];
-}
+// ------------------------------------------------------------ reductions
+// Sums over voxels run in double-float (ff.cuh) per thread and in float64 from the
+// block's partial sum on: a float64 sum of every element is bound by the float64
+// pipe (1/64 of the float32 rate) and took 2.1 ms for 67 M gradients, one block a
+// channel.  Rows are cut into kRowChunks pieces so that every SM takes part.
+constexpr int kRowChunks = 32;
 
-// gbias[c] = sum over b, v of g[b][c][v]   (one block per channel)
-__global__ void bias_grad_kernel(const float* __restrict__ g, float* __restrict__ gbias, int B, int C, long long nv) {
-    const int c = blockIdx.x;
-    double s = 0.0;
-    for (int b = 0; b < B; ++b) {
-        const float* row = g + ((long long)b * C + c) * nv;
-        for (long long v = threadIdx.x; v < nv; v += blockDim.x) s += row[v];
-    }
-    __shared__ double sh[256];
-    sh[threadIdx.x] = s;
+// Block sum of one double-float per thread; thread 0 returns it.
+__device__ __forceinline__ double block_sum_ff(FF s) {
+    __shared__ double sh[32];
+    double v = (double)s.h + (double)s.l;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) gbias[c] = (float)sh[0];
+    v = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w];
+    return v;
 }
 
-// Per-mode complex mixing.  Spectra laid out [part][mode][b][ch]; weights
-// R[part][mode][i][o].  U[mode][b][o] = sum_i V[mode][b][i] R[mode][i][o].
-__global__ void mix_fwd_kernel(const float* __restrict__ V, const float* __restrict__ R, float* __restrict__ U,
-                               int modes, int B, int C) {
+// The gradient through an activation and its bias, one read of each operand: with
+// GELU gz = ga * gelu'(z), else gz = ga (not written); partial[c][b * kRowChunks +
+// chunk] = the sum of the block's gz.  Block (b C + c) kRowChunks + chunk; nv is a multiple of 4.
+template <bool GELU>
+__global__ void __launch_bounds__(256)
+act_back_kernel(const float* __restrict__ z, const float* ga, float* gz, int B, int C,          // gz may be ga
+                long long nv, double* __restrict__ partial) {
+    const int row = blockIdx.x / kRowChunks, chunk = blockIdx.x % kRowChunks, c = row % C, b = row / C;
+    const long long n4 = nv / 4, per = (n4 + kRowChunks - 1) / kRowChunks;
+    const long long lo = chunk * per, hi = min(n4, lo + per), off = (long long)row * n4;
+    const float4 *z4 = reinterpret_cast<const float4*>(z) + off, *g4 = reinterpret_cast<const float4*>(ga) + off;
+    float4* o4 = reinterpret_cast<float4*>(gz) + off;
+    FF s{0.f, 0.f};
+    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        float4 g = g4[i];
+        if constexpr (GELU) {
+            const float4 v = z4[i];
+            g = make_float4(g.x * gelu_grad(v.x), g.y * gelu_grad(v.y), g.z * gelu_grad(v.z), g.w * gelu_grad(v.w));
+            o4[i] = g;
+        }
+        const FF p = two_sum(g.x, g.y), q = two_sum(g.z, g.w);
+        s = ff_add(s, ff_add(p, q));
+    }
+    const double t = block_sum_ff(s);
+    if (threadIdx.x == 0) partial[(long long)c * B * kRowChunks + b * kRowChunks + chunk] = t;
+}
+
+// gbias[c] = the sum of its n partials (one warp a channel, fixed order)
+__global__ void bias_reduce_kernel(const double* __restrict__ partial, int n, float* __restrict__ gbias) {
+    const double* p = partial + (long long)blockIdx.x * n;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32) s += p[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) gbias[blockIdx.x] = (float)s;
+}
+
+// ------------------------------------------------------------ pointwise weight gradients
+// gW[o][i] = sum over b, v of gZ[b][o][v] X[b][i][v], operands rounded to bfloat16
+// (float32 accumulation): an outer-product reduction over 2 M voxels into 1024
+// values, bound by the one read of gZ and X.  A warp walks voxels 16 at a time;
+// every operand row is read as float4 (a 16-voxel run is two full sectors a row),
+// straight into the fragments of mma.m16n8k16: the four voxels a lane holds are its
+// four k slots, the same in both operands, so nothing passes through shared memory.
+// (tcgen05 would pad the 32 rows to 128 and stage both operands in shared memory:
+// that form took 1.33 ms a layer at 8 x 64^3 voxels, this one 0.09 ms, 6.0 TB/s.)
+// Block: 32 x 32 tile (o0, i0) = blockIdx.y, z; splits of the voxels = blockIdx.x.
+// Partial tiles go to part[split][Mo][Ni]; wgrad_reduce_kernel adds them in order.
+constexpr int kWgWarps = 8;
+
+__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
+    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<uint32_t*>(&v);
+}
+
+__global__ void __launch_bounds__(32 * kWgWarps, 2)
+wgrad_kernel(const float* __restrict__ gZ, const float* __restrict__ X, int B, int Mo, int Ni, long long nv,
+             float* __restrict__ part) {
+    __shared__ float sh[kWgWarps][32][33];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int o0 = blockIdx.y * 32, i0 = blockIdx.z * 32;
+    const long long runs = (nv + 15) / 16, total = runs * B;       // 16-voxel runs, batch by batch (nv % 4 == 0)
+    const long long nw = (long long)gridDim.x * kWgWarps, w0 = (long long)blockIdx.x * kWgWarps + warp;
+    float acc[2][4][4] = {};
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto fetch = [&](long long r, float4 (&a)[4], float4 (&x)[4]) {
+        const long long b = r / runs, v = (r - b * runs) * 16 + 4 * t;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int o = o0 + 8 * k + g, i = i0 + 8 * k + g;
+            a[k] = o < Mo && v < nv ? __ldcs(reinterpret_cast<const float4*>(gZ + (b * Mo + o) * nv + v)) : zero;
+            x[k] = i < Ni && v < nv ? __ldcs(reinterpret_cast<const float4*>(X + (b * Ni + i) * nv + v)) : zero;
+        }
+    };
+    float4 a[4], x[4];
+    long long r = w0;
+    if (r < total) fetch(r, a, x);
+    while (r < total) {
+        uint32_t af[4][2], xf[4][2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            af[k][0] = bf16x2(a[k].x, a[k].y); af[k][1] = bf16x2(a[k].z, a[k].w);
+            xf[k][0] = bf16x2(x[k].x, x[k].y); xf[k][1] = bf16x2(x[k].z, x[k].w);
+        }
+        r += nw;
+        if (r < total) fetch(r, a, x);
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                             "{%0,%1,%2,%3};"
+                             : "+f"(acc[m][n][0]), "+f"(acc[m][n][1]), "+f"(acc[m][n][2]), "+f"(acc[m][n][3])
+                             : "r"(af[2 * m][0]), "r"(af[2 * m + 1][0]), "r"(af[2 * m][1]), "r"(af[2 * m + 1][1]),
+                               "r"(xf[n][0]), "r"(xf[n][1]));
+    }
+    // c0, c1: row g, columns 2t, 2t + 1; c2, c3: row g + 8
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            sh[warp][16 * m + g][8 * n + 2 * t] = acc[m][n][0];
+            sh[warp][16 * m + g][8 * n + 2 * t + 1] = acc[m][n][1];
+            sh[warp][16 * m + g + 8][8 * n + 2 * t] = acc[m][n][2];
+            sh[warp][16 * m + g + 8][8 * n + 2 * t + 1] = acc[m][n][3];
+        }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+        const int o = e >> 5, i = e & 31;
+        if (o0 + o >= Mo || i0 + i >= Ni) continue;
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWgWarps; ++w) s += sh[w][o][i];
+        part[((long long)blockIdx.x * Mo + o0 + o) * Ni + i0 + i] = s;
+    }
+}
+
+// gW[e] = sum over the splits (a warp an element, float64)
+__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int splits, int n, float* __restrict__ gW) {
+    const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (e >= n) return;
+    double s = 0.0;
+    for (int k = lane; k < splits; k += 32) s += (double)part[(long long)k * n + e];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) gW[e] = (float)s;
+}
+
+// ------------------------------------------------------------ per-mode complex mixing
+// Spectra laid out [part][mode][b][ch]; weights R[part][mode][i][o].  A block takes
+// one mode, its spectra and (backward through the input) its weights in shared
+// memory, and a thread four outputs that share each weight, so weights are read from
+// memory once and in full lines; bound by the weights' traffic (57 MB a layer at
+// 6912 modes and 32 channels).  A thread an output read the weights of the backward
+// pass a row apart per lane: 62, 388 and 94 us a layer (forward, input, weights) at a
+// batch of 8; now 48, 54 and 47 us.
+// A mode's spectra stay in global memory (same layout) where they exceed mix_stage's
+// limit.
+constexpr int kMixStage = 96 * 1024;
+
+// acc + (x y + z w) in a fixed order of roundings: the product z w, x y added to it in
+// one fused operation, the sum.  (Spectra are rounded to bfloat16 by the next
+// contraction, so a different order, although no less exact, moves the network's
+// output by 4e-5.)
+__device__ __forceinline__ float add_dot(float acc, float x, float y, float z, float w) {
+    return __fadd_rn(acc, __fmaf_rn(x, y, __fmul_rn(z, w)));
+}
+
+// The spectra of one mode, [part][B][C]: staged at sm (stage != 0) or in place.
+struct MixSpec { const float *re, *im; };
+__device__ __forceinline__ MixSpec mix_spec(const float* g, long long per, int mode, int BC, float* sm, bool stage) {
+    const float *re = g + (long long)mode * BC, *im = re + per;
+    if (!stage) return {re, im};
+    for (int e = threadIdx.x; e < BC; e += blockDim.x) {
+        sm[e] = re[e];
+        sm[BC + e] = im[e];
+    }
+    return {sm, sm + BC};
+}
+
+// U[mode][b][o] = sum_i V[mode][b][i] R[mode][i][o].  From four samples on a thread
+// takes (mode, four b, o), several modes a block when one has few threads' work; the
+// modes' spectra are contiguous, so they are staged together.
+__global__ void __launch_bounds__(256, 4)
+mix_fwd_kernel(const float* __restrict__ V, const float* __restrict__ R, float* __restrict__ U, int modes, int B, int C,
+               int per_block, int stage) {
+    extern __shared__ float mix_sm[];                              // [2][per_block][B][C]
+    constexpr int BT = 4;
+    const long long per = (long long)modes * B * C;
+    const int mode0 = blockIdx.x * per_block, nm = min(per_block, modes - mode0), BC = B * C;
+    const float *vre = V + (long long)mode0 * BC, *vim = vre + per;
+    if (stage) {
+        for (int e = threadIdx.x; e < nm * BC; e += blockDim.x) {
+            mix_sm[e] = vre[e];
+            mix_sm[per_block * BC + e] = vim[e];
+        }
+        vre = mix_sm;
+        vim = mix_sm + per_block * BC;
+    }
+    __syncthreads();
+    const int groups = (B + BT - 1) / BT;
+    for (int e = threadIdx.x; e < nm * groups * C; e += blockDim.x) {
+        const int o = e % C, gm = e / C, m = gm / groups, b0 = (gm - m * groups) * BT, mode = mode0 + m;
+        const float* rr = R + (long long)mode * C * C + o;
+        const float* ri = rr + (long long)modes * C * C;
+        const float *ar = vre + m * BC, *ai = vim + m * BC;
+        float ur[BT] = {}, ui[BT] = {};
+#pragma unroll 8
+        for (int i = 0; i < C; ++i) {
+            const float c = rr[i * C], d = ri[i * C];
+#pragma unroll
+            for (int k = 0; k < BT; ++k) {
+                const int bb = min(b0 + k, B - 1);
+                const float a = ar[bb * C + i], b = ai[bb * C + i];
+                ur[k] = add_dot(ur[k], a, c, -b, d);
+                ui[k] = add_dot(ui[k], b, c, a, d);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < BT; ++k)
+            if (b0 + k < B) {
+                const long long q = ((long long)mode * B + b0 + k) * C + o;
+                U[q] = ur[k];
+                U[per + q] = ui[k];
+            }
+    }
+}
+
+// The same with a thread an output, for one to three samples (a weight then serves
+// at most three outputs: 15 us a layer at one sample against 23 us for the above).
+__global__ void mix_fwd_few_kernel(const float* __restrict__ V, const float* __restrict__ R, float* __restrict__ U,
+                                   int modes, int B, int C) {
     const long long per = (long long)modes * B * C;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per; e += (long long)gridDim.x * blockDim.x) {
         const int o = (int)(e % C);
@@ -113,55 +317,91 @@ __global__ void mix_fwd_kernel(const float* __restrict__ V, const float* __restr
         float ur = 0.f, ui = 0.f;
         for (int i = 0; i < C; ++i) {
             const float a = vr[i], b = vi[i], c = rr[i * C], d = ri[i * C];
-            ur += a * c - b * d;
-            ui += a * d + b * c;
+            ur = add_dot(ur, a, c, -b, d);
+            ui = add_dot(ui, b, c, a, d);
         }
         U[e] = ur;
         U[per + e] = ui;
     }
 }
 
-// gV[mode][b][i] = sum_o (gUr R_r + gUi R_i, -gUr R_i + gUi R_r)
-__global__ void mix_back_input_kernel(const float* __restrict__ gU, const float* __restrict__ R, float* __restrict__ gV,
-                                      int modes, int B, int C) {
+// gV[mode][b][i] = sum_o (gUr R_r + gUi R_i, -gUr R_i + gUi R_r): thread i, four b a
+// thread, rows of R a row stride of C + 1 apart in shared memory, `rows` at a time.
+__global__ void mix_back_input_kernel(const float* __restrict__ gU, const float* __restrict__ R,
+                                      float* __restrict__ gV, int modes, int B, int C, int rows, int stage) {
+    extern __shared__ float mix_sm[];                              // [2][B][C] gradients, [2][rows][C + 1] weights
     const long long per = (long long)modes * B * C;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per; e += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(e % C);
-        const long long mb = e / C;
-        const int mode = (int)(mb / B);
-        const float* gr = gU + mb * C;
-        const float* gi = gU + per + mb * C;
-        const float* rr = R + (long long)mode * C * C + (long long)i * C;
-        const float* ri = R + (long long)modes * C * C + (long long)mode * C * C + (long long)i * C;
-        float vr = 0.f, vi = 0.f;
-        for (int o = 0; o < C; ++o) {
-            vr += gr[o] * rr[o] + gi[o] * ri[o];
-            vi += -gr[o] * ri[o] + gi[o] * rr[o];
+    const int mode = blockIdx.x, BC = B * C, ld = C + 1;
+    float *wr = mix_sm + (stage ? 2 * BC : 0), *wi = wr + rows * ld;
+    const MixSpec u = mix_spec(gU, per, mode, BC, mix_sm, stage);
+    const float* rr = R + (long long)mode * C * C;
+    const float* ri = R + (long long)modes * C * C + (long long)mode * C * C;
+    const int groups = (B + 3) / 4;
+    for (int r0 = 0; r0 < C; r0 += rows) {
+        const int nr = min(rows, C - r0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nr * C; e += blockDim.x) {
+            const int i = e / C, o = e - i * C;
+            wr[i * ld + o] = rr[r0 * C + e];
+            wi[i * ld + o] = ri[r0 * C + e];
         }
-        gV[e] = vr;
-        gV[per + e] = vi;
+        __syncthreads();
+        for (int e = threadIdx.x; e < groups * nr; e += blockDim.x) {
+            const int i = e % nr, b0 = (e / nr) * 4;
+            float vr[4] = {}, vi[4] = {};
+#pragma unroll 4
+            for (int o = 0; o < C; ++o) {
+                const float c = wr[i * ld + o], d = wi[i * ld + o];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int bb = min(b0 + k, B - 1);
+                    const float a = u.re[bb * C + o], b = u.im[bb * C + o];
+                    vr[k] = add_dot(vr[k], a, c, b, d);
+                    vi[k] = add_dot(vi[k], b, c, -a, d);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (b0 + k < B) {
+                    const long long q = ((long long)mode * B + b0 + k) * C + r0 + i;
+                    gV[q] = vr[k];
+                    gV[per + q] = vi[k];
+                }
+        }
     }
 }
 
-// gR[mode][i][o] = sum_b (gUr Vr + gUi Vi, -gUr Vi + gUi Vr)
-__global__ void mix_back_weight_kernel(const float* __restrict__ gU, const float* __restrict__ V, float* __restrict__ gR,
-                                       int modes, int B, int C) {
-    const long long per = (long long)modes * B * C;
-    const long long nw = (long long)modes * C * C;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nw; e += (long long)gridDim.x * blockDim.x) {
-        const int o = (int)(e % C);
-        const int i = (int)((e / C) % C);
-        const int mode = (int)(e / ((long long)C * C));
-        float sr = 0.f, si = 0.f;
+// gR[mode][i][o] = sum_b (gUr Vr + gUi Vi, -gUr Vi + gUi Vr): thread o, four i a
+// thread.
+__global__ void mix_back_weight_kernel(const float* __restrict__ gU, const float* __restrict__ V,
+                                       float* __restrict__ gR, int modes, int B, int C, int stage) {
+    extern __shared__ float mix_sm[];                              // [2][B][C] gradients, [2][B][C] spectra
+    const long long per = (long long)modes * B * C, nw = (long long)modes * C * C;
+    const int mode = blockIdx.x, BC = B * C;
+    const MixSpec u = mix_spec(gU, per, mode, BC, mix_sm, stage);
+    const MixSpec v = mix_spec(V, per, mode, BC, mix_sm + 2 * BC, stage);
+    __syncthreads();
+    float* out = gR + (long long)mode * C * C;
+    const int groups = (C + 3) / 4;
+    for (int e = threadIdx.x; e < groups * C; e += blockDim.x) {
+        const int o = e % C, i0 = (e / C) * 4;
+        float sr[4] = {}, si[4] = {};
         for (int b = 0; b < B; ++b) {
-            const long long base = ((long long)mode * B + b) * C;
-            const float gr = gU[base + o], gi = gU[per + base + o];
-            const float vr = V[base + i], vi = V[per + base + i];
-            sr += gr * vr + gi * vi;
-            si += -gr * vi + gi * vr;
+            const float gr = u.re[b * C + o], gi = u.im[b * C + o];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = min(i0 + k, C - 1);
+                const float vr = v.re[b * C + i], vi = v.im[b * C + i];
+                sr[k] = add_dot(sr[k], gr, vr, gi, vi);
+                si[k] = add_dot(si[k], gi, vr, -gr, vi);
+            }
         }
-        gR[e] = sr;
-        gR[nw + e] = si;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k < C) {
+                out[(i0 + k) * C + o] = sr[k];
+                out[nw + (i0 + k) * C + o] = si[k];
+            }
     }
 }
 
@@ -223,7 +463,8 @@ struct psatd_fno {
     std::vector<float*> act, pre, T1, T2, T3, U3, W1, W2;
     float *feat = nullptr, *hq = nullptr, *zq = nullptr, *out = nullptr, *gbuf0 = nullptr, *gbuf1 = nullptr;
     float *gT = nullptr, *gT2 = nullptr, *gout = nullptr;
-    double* partial = nullptr;
+    double *partial = nullptr, *bpart = nullptr;     // loss partials, bias-gradient partials
+    float* wpart = nullptr;                          // weight-gradient partials
     int adam_t = 0;
     std::string err = "no error";
 };
@@ -252,6 +493,12 @@ GemmArgs G(int M, int N, int K, const float* A, long long sAm, long long sAk, co
     g.C = C; g.sCb0 = sCb; g.sCm = sCm; g.sCn = sCn;
     g.alpha = 1.f; g.beta = beta; g.ksplit = 1;
     return g;
+}
+
+// Voxel splits of a weight gradient: with its 32 x 32 tiles about two blocks an SM
+int wgrad_splits(int Mo, int Ni) {
+    const int tiles = ((Mo + 31) / 32) * ((Ni + 31) / 32);
+    return std::max(1, 2 * 152 / tiles);
 }
 
 int freq_t(int j, int m, int P) { return j < m ? j : P - 2 * m + j; }
@@ -369,7 +616,12 @@ psatd_status psatd_fno_create(const psatd_fno_config* cfg, unsigned long long se
          alloc(&f->out, B * f->NO * NV) && alloc(&f->gbuf0, std::max(B * f->H * NV, big)) &&
          alloc(&f->gbuf1, std::max(B * f->H * NV, big)) && alloc(&f->gT, std::max(big, nW1)) &&
          alloc(&f->gT2, std::max(big, nW1)) && alloc(&f->gout, B * f->NO * NV);
-    ok = ok && cudaMalloc(&f->partial, 4096 * sizeof(double)) == cudaSuccess;
+    ok = ok && cudaMalloc(&f->partial, 4096 * sizeof(double)) == cudaSuccess &&
+         cudaMalloc(&f->bpart, (size_t)B * kRowChunks * std::max(std::max(C, f->H), f->NO) * sizeof(double)) == cudaSuccess;
+    long long wmax = 0;
+    for (auto mn : {std::pair<int, int>(f->NO, f->H), {f->H, C}, {C, C}, {C, FI}})
+        wmax = std::max(wmax, (long long)wgrad_splits(mn.first, mn.second) * mn.first * mn.second);
+    ok = ok && alloc(&f->wpart, wmax);
     if (!ok) {
         psatd_fno_destroy(f);
         return PSATD_ERR_OOM;
@@ -405,6 +657,8 @@ void psatd_fno_destroy(psatd_fno* f) {
         for (float* p : *v)
             if (p) cudaFree(p);
     if (f->partial) cudaFree(f->partial);
+    if (f->bpart) cudaFree(f->bpart);
+    if (f->wpart) cudaFree(f->wpart);
     delete f;
 }
 
@@ -423,6 +677,49 @@ const char* psatd_fno_last_error(const psatd_fno* f) { return f ? f->err.c_str()
 }  // extern "C"
 
 namespace {
+
+// Launches of the mixing kernels: shared memory for the staged spectra (sets, four
+// bytes a value) and, backward through the input, as many weight rows as fit.
+template <typename K>
+cudaError_t mix_smem(K k, size_t bytes) {
+    return bytes > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
+                             : cudaSuccess;
+}
+int mix_threads(int n) { return std::min(256, std::max(32, (n + 31) / 32 * 32)); }
+
+cudaError_t mix_fwd(psatd_fno* f, const float* V, const float* R, float* U, int B) {
+    if (B < 4) {
+        mix_fwd_few_kernel<<<grid_for((long long)f->MODES * B * f->C), 256, 0, f->stream>>>(V, R, U, f->MODES, B, f->C);
+        return cudaGetLastError();
+    }
+    const int items = (B + 3) / 4 * f->C;                          // of one mode
+    const int per_block = std::max(1, 256 / items);
+    const size_t need = (size_t)2 * per_block * B * f->C * sizeof(float);
+    const int stage = need <= (size_t)kMixStage;
+    const cudaError_t e = mix_smem(mix_fwd_kernel, stage ? need : 0);
+    if (e != cudaSuccess) return e;
+    mix_fwd_kernel<<<(f->MODES + per_block - 1) / per_block, mix_threads(per_block * items), stage ? need : 0,
+                     f->stream>>>(V, R, U, f->MODES, B, f->C, per_block, stage);
+    return cudaGetLastError();
+}
+
+cudaError_t mix_back(psatd_fno* f, const float* gU, const float* V, const float* R, float* gR, float* gV, int B) {
+    const int C = f->C;
+    const size_t spec = (size_t)2 * B * C * sizeof(float);
+    int stage = 2 * spec <= (size_t)kMixStage;
+    cudaError_t e = mix_smem(mix_back_weight_kernel, stage ? 2 * spec : 0);
+    if (e != cudaSuccess) return e;
+    mix_back_weight_kernel<<<f->MODES, mix_threads((C + 3) / 4 * C), stage ? 2 * spec : 0, f->stream>>>(
+        gU, V, gR, f->MODES, B, C, stage);
+    stage = spec <= (size_t)kMixStage;
+    const size_t row = (size_t)2 * (C + 1) * sizeof(float);
+    const int rows = (int)std::min<size_t>(C, kMixStage / row);
+    const size_t bytes = (stage ? spec : 0) + rows * row;
+    if ((e = mix_smem(mix_back_input_kernel, bytes)) != cudaSuccess) return e;
+    mix_back_input_kernel<<<f->MODES, mix_threads((B + 3) / 4 * rows), bytes, f->stream>>>(gU, R, gV, f->MODES, B, C,
+                                                                                         rows, stage);
+    return cudaGetLastError();
+}
 
 // forward pass; leaves activations for the backward pass
 psatd_status fno_forward(psatd_fno* f, const float* prm, int B) {
@@ -449,8 +746,7 @@ psatd_status fno_forward(psatd_fno* f, const float* prm, int B) {
         FCK(launch_gemm(G((int)Mz, 2 * NT, P, f->T2[l], P, 1, f->By1, 2 * NT, 1, f->T3[l], 1, Mz, 0.f), s));
         FCK(launch_gemm(G((int)Mz, 2 * NT, P, f->T2[l] + Mz * P, P, 1, f->By2, 2 * NT, 1, f->T3[l], 1, Mz, 1.f), s));
         // mode mixing: T3 = [part][kz][ky][kx][b][c] = [part][mode][b][c]
-        mix_fwd_kernel<<<grid_for((long long)f->MODES * B * C), 256, 0, s>>>(f->T3[l], f->par + f->o_R[l], f->U3[l],
-                                                                            f->MODES, B, C);
+        FCK(mix_fwd(f, f->T3[l], f->par + f->o_R[l], f->U3[l], B));
         // Zi: rows r = (ky,kx,b,o), K = kz (stride Mz); out W1[(part,z)][r]
         FCK(launch_gemm(G((int)Mz, 2 * P, NT, f->U3[l], 1, Mz, f->Bz1, 2 * P, 1, f->W1[l], 1, Mz, 0.f), s));
         FCK(launch_gemm(G((int)Mz, 2 * P, NT, f->U3[l] + (long long)NT * Mz, 1, Mz, f->Bz2, 2 * P, 1, f->W1[l], 1, Mz, 1.f), s));
@@ -490,16 +786,26 @@ psatd_status fno_forward(psatd_fno* f, const float* prm, int B) {
     return PSATD_OK;
 }
 
-// weight gradient gW (Mo x Ni) = sum_b gZ[b] (Mo x NV) * X[b]^T (NV x Ni), split over NV
+// weight gradient gW (Mo x Ni) = sum_b gZ[b] (Mo x NV) * X[b]^T (NV x Ni)
 cudaError_t weight_grad(psatd_fno* f, int Mo, int Ni, const float* gZ, const float* X, float* gW, int B) {
-    for (int b = 0; b < B; ++b) {
-        GemmArgs g = G(Mo, Ni, (int)f->NV, gZ + (long long)b * Mo * f->NV, f->NV, 1, X + (long long)b * Ni * f->NV, 1,
-                       f->NV, gW, Ni, 1, b == 0 ? 0.f : 1.f);
-        g.ksplit = (int)std::min<long long>(256, (f->NV + 4095) / 4096);
-        cudaError_t e = launch_gemm(g, f->stream);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const dim3 grid(wgrad_splits(Mo, Ni), (Mo + 31) / 32, (Ni + 31) / 32);
+    wgrad_kernel<<<grid, 32 * kWgWarps, 0, f->stream>>>(gZ, X, B, Mo, Ni, f->NV, f->wpart);
+    wgrad_reduce_kernel<<<(Mo * Ni + 7) / 8, 256, 0, f->stream>>>(f->wpart, (int)grid.x, Mo * Ni, gW);
+    return cudaGetLastError();
+}
+
+// bias gradient of gz (no activation): gbias[c] = sum over b, v
+cudaError_t bias_grad(psatd_fno* f, const float* gz, float* gbias, int B, int C) {
+    act_back_kernel<false><<<B * C * kRowChunks, 256, 0, f->stream>>>(nullptr, gz, nullptr, B, C, f->NV, f->bpart);
+    bias_reduce_kernel<<<C, 32, 0, f->stream>>>(f->bpart, B * kRowChunks, gbias);
+    return cudaGetLastError();
+}
+
+// gz = ga * gelu'(z) and its bias gradient
+cudaError_t gelu_back(psatd_fno* f, const float* z, const float* ga, float* gz, float* gbias, int B, int C) {
+    act_back_kernel<true><<<B * C * kRowChunks, 256, 0, f->stream>>>(z, ga, gz, B, C, f->NV, f->bpart);
+    bias_reduce_kernel<<<C, 32, 0, f->stream>>>(f->bpart, B * kRowChunks, gbias);
+    return cudaGetLastError();
 }
 
 psatd_status fno_backward(psatd_fno* f, int B) {
@@ -508,22 +814,27 @@ psatd_status fno_backward(psatd_fno* f, int B) {
     cudaStream_t s = f->stream;
     float* g = f->grad;
     // output layer: gout holds dL/dout
-    bias_grad_kernel<<<NO, 256, 0, s>>>(f->gout, g + f->o_q2_b, B, NO, NV);
+    FCK(bias_grad(f, f->gout, g + f->o_q2_b, B, NO));
     FCK(weight_grad(f, NO, H, f->gout, f->hq, g + f->o_q2_w, B));
     // g_h = Wq2^T gout ; g_zq = g_h * gelu'(zq)
     FCK(launch_gemm(G(H, (int)NV, NO, f->par + f->o_q2_w, 1, H, f->gout, NV, 1, f->gbuf0, NV, 1, 0.f, B, 0, NO * NV,
                       H * NV), s));
-    act_back_kernel<<<grid_for(B * H * NV), 256, 0, s>>>(f->zq, f->gbuf0, f->gbuf0, B * H * NV, 1);
-    bias_grad_kernel<<<H, 256, 0, s>>>(f->gbuf0, g + f->o_q1_b, B, H, NV);
+    FCK(gelu_back(f, f->zq, f->gbuf0, f->gbuf0, g + f->o_q1_b, B, H));
     FCK(weight_grad(f, H, C, f->gbuf0, f->act[f->L], g + f->o_q1_w, B));
     // g_a(L) = Wq1^T g_zq
-    float* ga = f->gbuf1;
+    float *ga = f->gbuf1, *other = f->gbuf0;
     FCK(launch_gemm(G(C, (int)NV, H, f->par + f->o_q1_w, 1, C, f->gbuf0, NV, 1, ga, NV, 1, 0.f, B, 0, H * NV, C * NV), s));
     for (int l = f->L - 1; l >= 0; --l) {
-        // g_z = g_a * act'(z)
-        float* gz = f->gbuf0;
-        act_back_kernel<<<grid_for(B * C * NV), 256, 0, s>>>(f->pre[l + 1], ga, gz, B * C * NV, l + 1 < f->L ? 1 : 0);
-        bias_grad_kernel<<<C, 256, 0, s>>>(gz, g + f->o_b[l], B, C, NV);
+        // g_z = g_a * act'(z); the last layer has no activation: g_z is g_a, and the
+        // gradient of its input goes to the other buffer
+        float* gz = ga;
+        if (l + 1 < f->L) {
+            gz = other;
+            FCK(gelu_back(f, f->pre[l + 1], ga, gz, g + f->o_b[l], B, C));
+        } else {
+            FCK(bias_grad(f, gz, g + f->o_b[l], B, C));
+            std::swap(ga, other);
+        }
         FCK(weight_grad(f, C, C, gz, f->act[l], g + f->o_W[l], B));
         // g_v (pointwise part) = W^T g_z -> ga (act[l] gradient), overwritten
         FCK(launch_gemm(G(C, (int)NV, C, f->par + f->o_W[l], 1, C, gz, NV, 1, ga, NV, 1, 0.f, B, 0, C * NV, C * NV), s));
@@ -553,9 +864,8 @@ psatd_status fno_backward(psatd_fno* f, int B) {
             FCK(launch_gemm(G((int)Mz, NT, 2 * P, gW1, 1, Mz, part == 0 ? f->Bz1 : f->Bz2, 1, 2 * P,
                               gU + (long long)part * NT * Mz, 1, Mz, 0.f), s));
         // mixing: weights and spectra
-        mix_back_weight_kernel<<<grid_for((long long)f->MODES * C * C), 256, 0, s>>>(gU, f->T3[l], g + f->o_R[l], f->MODES, B, C);
         float* gV = f->gT2;
-        mix_back_input_kernel<<<grid_for((long long)f->MODES * B * C), 256, 0, s>>>(gU, f->par + f->o_R[l], gV, f->MODES, B, C);
+        FCK(mix_back(f, gU, f->T3[l], f->par + f->o_R[l], g + f->o_R[l], gV, B));
         // adjoint of Z: g_T2[part] (rows (ky,kx,b,c), K = z) = gV (rows, 2NT) * By_part^T
         float* gT2 = f->gT;
         for (int part = 0; part < 2; ++part)
@@ -571,10 +881,8 @@ psatd_status fno_backward(psatd_fno* f, int B) {
         FCK(launch_gemm(G((int)M1, P, 2 * m, gT1, 1, M1, f->Fx, 1, 2 * m, ga, P, 1, 1.f), s));
     }
     // lift
-    float* gz = f->gbuf0;
-    act_back_kernel<<<grid_for(B * C * NV), 256, 0, s>>>(f->pre[0], ga, gz, B * C * NV, 0);
-    bias_grad_kernel<<<C, 256, 0, s>>>(gz, g + f->o_lift_b, B, C, NV);
-    FCK(weight_grad(f, C, FI, gz, f->feat, g + f->o_lift_w, B));
+    FCK(bias_grad(f, ga, g + f->o_lift_b, B, C));
+    FCK(weight_grad(f, C, FI, ga, f->feat, g + f->o_lift_w, B));
     FCK(cudaGetLastError());
     return PSATD_OK;
 }
