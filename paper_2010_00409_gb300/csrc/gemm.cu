@@ -20,12 +20,18 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // tcgen05.mma (kind::f16, bf16 x bf16 -> f32) with the accumulators in tensor
-// memory.  A kernel that allocates tensor memory runs one block per SM, so the
-// grid is one persistent block of 512 threads per SM; tile 128 (M) x BN (N), K
-// in blocks of 64.  Two-stage pipeline: while the tensor core multiplies the
-// operands of one K block, the threads stage the next one, and while the MMAs
-// of tile t run, the threads read tile t-1's accumulators (two accumulators of
-// BN columns in tensor memory).
+// memory.  Tile 128 (M) x BN (N), K in blocks of 64, two operand stages (the
+// threads stage one K block while the tensor core multiplies the other).
+//
+// The surrogate's contractions are thin (one K block a tile, 24 to 128 columns) and
+// bound by their operands' traffic, and a tile is a chain: loads, rounding and
+// stores to shared memory, MMAs, accumulator reads, stores.  So the chains of
+// several blocks of 256 threads per SM overlap (five, four or three for BN = 32, 64,
+// 128: shared memory and registers; the occupancy query answers one block for a kernel
+// that allocates tensor memory, but the SM runs as many as the 512 tensor-memory
+// columns allow, and each block takes only the BN it accumulates into).  One block of
+// 512 threads per SM with two accumulators, the form before, left the memory at a
+// quarter of its rate: 2^20 x 24 x 64 took 242 us, 94 us (3.9 TB/s) now.
 //
 // Staging: each thread takes 8 consecutive k of one row, rounds them to
 // bfloat16 and writes them as one 16-byte row of a "core matrix" (8 rows x 8
@@ -38,7 +44,7 @@ namespace {
 // refilled) and, after a tile's last K block, to the accumulator's mbarrier
 // (the tile may be read).  All waits are bounded; an expired wait sets
 // g_gemm_error (gemm_take_error reads and clears it).
-constexpr int TBM = 128, TBK = 64, kTcThreads = 512;
+constexpr int TBM = 128, TBK = 64, kTcThreads = 256;
 __device__ int g_gemm_error;
 
 __device__ __forceinline__ uint32_t tc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -73,7 +79,8 @@ template <int BN> struct TcCfg {
     static constexpr int kStageA = TBM * TBK * 2;             // bytes of one A stage
     static constexpr int kStageB = BN * TBK * 2;
     static constexpr int kSmem = 2 * (kStageA + kStageB);
-    static constexpr int kCols = 2 * BN;                      // two accumulators
+    static constexpr int kCols = BN;                          // tensor-memory columns (a power of two, >= 32)
+    static constexpr int kBlocks = BN == 32 ? 5 : (BN == 64 ? 4 : 3);   // per SM
 };
 
 struct TcTile {
@@ -110,13 +117,33 @@ __device__ __forceinline__ TcTile tc_tile(const GemmArgs& g, int tile, int ntm, 
 // (then 8 consecutive k from a multiple of 8 are two aligned float4 loads)
 // Only the first kcs 8-column chunks are staged (the MMAs of a short last K
 // block read no further).
+template <int ROWS> constexpr int tc_items() { return (ROWS * (TBK / 8) + kTcThreads - 1) / kTcThreads; }
+
+// Row r and chunk kc of a thread's n-th item.  Contiguous k (vec): a warp takes 8 rows
+// x 4 chunks, 128 contiguous bytes of each row, and its 8-lane groups store 8 rows of
+// one chunk, one core matrix (conflict-free); with 32 rows a warp, each load touched
+// 32 lines.  Otherwise 32 rows of one chunk (contiguous where the rows are).
+template <int ROWS>
+__device__ __forceinline__ bool tc_item(int n, bool vec, int kcs, int& r, int& kc) {
+    const int i = threadIdx.x + n * kTcThreads;
+    if (vec) {
+        const int w = i >> 5, lane = i & 31;
+        r = (w % (ROWS / 8)) * 8 + (lane & 7);
+        kc = (w / (ROWS / 8)) * 4 + (lane >> 3);
+    } else {
+        r = i % ROWS;
+        kc = i / ROWS;
+    }
+    return kc < kcs;
+}
+
 template <int ROWS>
 __device__ __forceinline__ void tc_stage(unsigned char* dst, const float* __restrict__ src, long long s_r,
                                          long long s_k, int r0, int nrows, int k0, int kend, bool vec, int kcs) {
-    const int items = ROWS * kcs;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < items; i += kTcThreads) {
-        const int r = i % ROWS, kc = i / ROWS;
+#pragma unroll
+    for (int n = 0; n < tc_items<ROWS>(); ++n) {
+        int r, kc;
+        if (!tc_item<ROWS>(n, vec, kcs, r, kc)) continue;
         const int gr = r0 + r, gk = k0 + kc * 8;
         float v[8];
         if (vec && gr < nrows && gk + 8 <= kend) {
@@ -125,8 +152,12 @@ __device__ __forceinline__ void tc_stage(unsigned char* dst, const float* __rest
             v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
             v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
         } else {
+            const float* p = src + gr * s_r + gk * s_k;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = (gr < nrows && gk + q < kend) ? src[gr * s_r + (gk + q) * s_k] : 0.f;
+            for (int q = 0; q < 8; ++q) {
+                v[q] = (gr < nrows && gk + q < kend) ? *p : 0.f;
+                p += s_k;
+            }
         }
         uint4 w;
         w.x = pack_bf16x2(v[0], v[1]);
@@ -137,38 +168,24 @@ __device__ __forceinline__ void tc_stage(unsigned char* dst, const float* __rest
     }
 }
 
-// Epilogue.  Warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the rows of
-// its lane quarter); the kTcThreads / 128 warps of one quarter split the
-// columns (cols each), read in loads of 8.  With beta != 0 the thread's C
-// values are loaded first (tc_epilogue_c, issued before the wait on the
-// accumulator, so their latency overlaps the MMAs).
-template <int BN> struct TcEpi {
-    static constexpr int parts = kTcThreads / 128, cols = BN / parts;
+// Epilogue.  Warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the rows of its
+// lane quarter); the two warps of one quarter split the columns, read in loads of 8.
+template <int BN>
+__device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, uint32_t acc_addr, bool have) {
+    constexpr int parts = kTcThreads / 128, cols = BN / parts;
     static_assert(cols % 8 == 0, "column split");
-};
-
-template <int BN>
-__device__ __forceinline__ void tc_epilogue_c(const GemmArgs& g, const TcTile& t, float (&cv)[TcEpi<BN>::cols]) {
-    constexpr int cols = TcEpi<BN>::cols;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m = t.m0 + 32 * (warp & 3) + lane, c0 = (warp >> 2) * cols;
-    const bool need = g.ksplit == 1 && g.beta != 0.f && m < g.M;
-#pragma unroll
-    for (int i = 0; i < cols; ++i) {
-        const int n = t.n0 + c0 + i;
-        cv[i] = (need && n < g.N) ? t.C[m * g.sCm + n * g.sCn] : 0.f;
-    }
-}
-
-template <int BN>
-__device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, uint32_t acc_addr, bool have,
-                                            const float (&cv)[TcEpi<BN>::cols]) {
-    constexpr int cols = TcEpi<BN>::cols;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quarter = warp & 3;
     const int m = t.m0 + 32 * quarter + lane, c0 = (warp >> 2) * cols;
-#pragma unroll
+    const bool row = m < g.M, need = g.ksplit == 1 && g.beta != 0.f && row;
+#pragma unroll 1
     for (int cc = 0; cc < cols; cc += 8) {
+        if (t.n0 + c0 + cc >= g.N) break;                      // (the same for every lane)
+        float* dst = t.C + m * g.sCm + (t.n0 + c0 + cc) * g.sCn;
+        const int nv = min(8, g.N - (t.n0 + c0 + cc));
+        float cv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cv[i] = (need && i < nv) ? dst[i * g.sCn] : 0.f;
         uint32_t r[8];
         if (have) {
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -180,15 +197,13 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
 #pragma unroll
             for (int i = 0; i < 8; ++i) r[i] = 0u;
         }
-        if (m < g.M) {
+        if (row) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const int n = t.n0 + c0 + cc + i;
-                if (n < g.N) {
-                    float* dst = t.C + m * g.sCm + n * g.sCn;
+                if (i < nv) {
                     const float v = g.alpha * __uint_as_float(r[i]);
-                    if (g.ksplit > 1) atomicAdd(dst, v);
-                    else *dst = (g.beta == 0.f) ? v : v + g.beta * cv[cc + i];
+                    if (g.ksplit > 1) atomicAdd(dst + i * g.sCn, v);
+                    else dst[i * g.sCn] = (g.beta == 0.f) ? v : v + g.beta * cv[i];
                 }
             }
         }
@@ -197,11 +212,11 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
 }
 
 template <int BN>
-__global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
+__global__ void __launch_bounds__(kTcThreads, TcCfg<BN>::kBlocks) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
     using Cfg = TcCfg<BN>;
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     __shared__ uint32_t tmem_base;
-    __shared__ __align__(8) uint64_t sbar[2], abar[2];
+    __shared__ __align__(8) uint64_t sbar[2], abar;
     const int tid = threadIdx.x, warp = tid >> 5;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(&tmem_base)),
@@ -209,16 +224,15 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(GemmArgs g, int ntm
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 2; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(&sbar[i])), "r"(1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(&abar[i])), "r"(1) : "memory");
-        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(&abar)), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base;
+    const uint32_t acc = tmem_base;
     // instruction descriptor: D f32, A and B bf16, both K-major, N = BN, M = 128
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                ((uint32_t)(TBM >> 4) << 24);
@@ -228,14 +242,9 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(GemmArgs g, int ntm
                       (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
     bool ok = true;
     uint32_t it = 0, tl = 0;
-    TcTile prev{};
 #pragma unroll 1
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tl) {
-        // every thread has finished waiting on the accumulator barriers before
-        // thread 0 commits to them again (also when a tile has no K block)
-        __syncthreads();
         const TcTile t = tc_tile(g, tile, ntm, ntn, BN);
-        const uint32_t acc = tmem + (tl & 1) * BN;
 #pragma unroll 1
         for (int kb = 0; kb < t.nkb; ++kb, ++it) {
             const int s = it & 1;
@@ -247,6 +256,7 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(GemmArgs g, int ntm
             tc_stage<TBM>(As, t.A, g.sAm, g.sAk, t.m0, g.M, k0, t.kend, vecA, 2 * nkk);
             tc_stage<BN>(Bs, t.B, g.sBn, g.sBk, t.n0, g.N, k0, t.kend, vecB, 2 * nkk);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> tensor-core reads
+            // (every thread has also read the previous tile's accumulator by now)
             __syncthreads();
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -263,31 +273,22 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(GemmArgs g, int ntm
                 tc_commit(&sbar[s]);
             }
         }
-        if (tid == 0) tc_commit(&abar[tl & 1]);          // this tile's accumulator (immediate when nkb = 0)
-        if (tl > 0) {                                     // read the previous tile while these MMAs run
-            float cv[TcEpi<BN>::cols];
-            tc_epilogue_c<BN>(g, prev, cv);
-            ok = tc_wait(&abar[(tl - 1) & 1], ((tl - 1) >> 1) & 1) && ok;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            tc_epilogue<BN>(g, prev, tmem + ((tl - 1) & 1) * BN, prev.nkb > 0, cv);
-        }
-        prev = t;
-    }
-    if (tl > 0) {
-        float cv[TcEpi<BN>::cols];
-        tc_epilogue_c<BN>(g, prev, cv);
-        ok = tc_wait(&abar[(tl - 1) & 1], ((tl - 1) >> 1) & 1) && ok;
+        // the tile's accumulator, once its MMAs are done (immediate when it has no K
+        // block; then the barrier keeps thread 0's commits behind every thread's wait)
+        if (t.nkb == 0) __syncthreads();
+        if (tid == 0) tc_commit(&abar);
+        ok = tc_wait(&abar, tl & 1) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tc_epilogue<BN>(g, prev, tmem + ((tl - 1) & 1) * BN, prev.nkb > 0, cv);
+        tc_epilogue<BN>(g, t, acc, t.nkb > 0);
     }
     if (!ok) {
         if (tid == 0) atomicExch(&g_gemm_error, 1);
-        // second bounded waits: no MMA may still write the accumulators at dealloc
-        for (int i = 0; i < 2; ++i) tc_wait(&abar[i], 0), tc_wait(&abar[i], 1);
+        // second bounded waits: no MMA may still write the accumulator at dealloc
+        tc_wait(&abar, 0), tc_wait(&abar, 1);
     }
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::kCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(acc), "r"(Cfg::kCols) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -521,21 +522,18 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
         if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
         auto k = bi == 0 ? gemm_tc_kernel<32> : (bi == 1 ? gemm_tc_kernel<64> : gemm_tc_kernel<128>);
         const int smem = bi == 0 ? TcCfg<32>::kSmem : (bi == 1 ? TcCfg<64>::kSmem : TcCfg<128>::kSmem);
-        // one resident block per SM (a kernel that allocates tensor memory runs
-        // one block per SM), persistent over the tiles
-        static int sms = 0, per_sm[3] = {0, 0, 0}, smem_launch[3] = {0, 0, 0};
-        if (!per_sm[bi]) {
+        // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
+        static int sms = 0, smem_launch[3] = {0, 0, 0};
+        const int per_sm[3] = {TcCfg<32>::kBlocks, TcCfg<64>::kBlocks, TcCfg<128>::kBlocks};
+        if (!smem_launch[bi]) {
             int dev = 0;
             cudaGetDevice(&dev);
             if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (sms < 1) sms = 1;
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
-            int occ = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kTcThreads, smem);
+            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
             if (e != cudaSuccess) return e;
-            if (occ < 1) return cudaErrorInvalidConfiguration;
-            per_sm[bi] = occ;
             smem_launch[bi] = smem;
         }
         const long long cap = (long long)sms * per_sm[bi];
