@@ -414,6 +414,20 @@ struct GemmArgs {
     long long sCb0, sCb1, sCm, sCn;
     float alpha, beta;
     int ksplit;
+    // Optional (null / 0), with ksplit 1:
+    //  A2, B2  a second product of the same shape and strides, accumulated apart:
+    //          C = alpha A2 B2 + alpha A B + beta C, added in that order;
+    //  nsplit  columns n >= nsplit of C lie c_split elements further on;
+    //  bias    bias[m] is added to row m of the result (after beta C);
+    //  act     the result, through GELU if gelu is set, goes here too (layout of C),
+    //          and to C itself only if store_c is set.
+    const float *A2 = nullptr, *B2 = nullptr;
+    int nsplit = 0;
+    long long c_split = 0;
+    const float* bias = nullptr;
+    float* act = nullptr;
+    bool gelu = false, store_c = true;
+    bool swapped = false;         // set by the launcher: rows and columns exchanged
 };
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s);
 

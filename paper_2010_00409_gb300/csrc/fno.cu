@@ -58,21 +58,8 @@ __global__ void features_kernel(const float* __restrict__ prm, int np, int B, in
     }
 }
 
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float x) {
     return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
-// z[b][c][v] += bias[c]; a = act(z) (act = GELU if gelu else identity); a may be z
-__global__ void bias_act_kernel(float* z, float* a, const float* __restrict__ bias,
-                                int B, int C, long long nv, int use_gelu) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)B * C * nv;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)((e / nv) % C);
-        const float v = z[e] + bias[c];
-        z[e] = v;
-        a[e] = use_gelu ? gelu(v) : v;
-    }
 }
 
 // ------------------------------------------------------------ reductions
@@ -591,16 +578,22 @@ psatd_status psatd_fno_create(const psatd_fno_config* cfg, unsigned long long se
             bx1[(size_t)k * P + x] = (float)(w * std::cos(th));
             bx2[(size_t)k * P + x] = (float)(-w * std::sin(th));
         }
-    ok = ok && alloc(&f->Fx, fx.size()) && alloc(&f->By1, by1.size()) && alloc(&f->By2, by2.size()) &&
-         alloc(&f->Bz1, bz1.size()) && alloc(&f->Bz2, bz2.size()) && alloc(&f->Bx1, bx1.size()) &&
-         alloc(&f->Bx2, bx2.size());
+    // the two matrices of a pair lie one behind the other: the adjoint stages take both
+    // as one operand
+    ok = ok && alloc(&f->Fx, fx.size()) && alloc(&f->By1, 2 * by1.size()) && alloc(&f->Bz1, 2 * bz1.size()) &&
+         alloc(&f->Bx1, 2 * bx1.size());
+    if (ok) {
+        f->By2 = f->By1 + by1.size();
+        f->Bz2 = f->Bz1 + bz1.size();
+        f->Bx2 = f->Bx1 + bx1.size();
+    }
     // activations for max batch
     const long long B = f->maxB, NV = f->NV;
     const long long nT1 = 2LL * m * B * C * P * P, nT2 = 2LL * NT * m * B * C * P, nT3 = 2LL * f->MODES * B * C;
     const long long nW1 = 2LL * P * NT * m * B * C, nW2 = 2LL * P * P * m * B * C;
     for (int l = 0; l <= L && ok; ++l) {
         float *a = nullptr, *z = nullptr;
-        ok = alloc(&a, B * C * NV) && alloc(&z, B * C * NV);
+        ok = alloc(&a, B * C * NV) && (l == 0 || alloc(&z, B * C * NV));   // (the lift has no pre-activation)
         f->act.push_back(a);
         f->pre.push_back(z);
     }
@@ -649,7 +642,7 @@ psatd_status psatd_fno_create(const psatd_fno_config* cfg, unsigned long long se
 void psatd_fno_destroy(psatd_fno* f) {
     if (!f) return;
     if (f->stream) cudaStreamSynchronize(f->stream);
-    float* ps[] = {f->par, f->grad, f->m1, f->m2, f->Fx, f->By1, f->By2, f->Bz1, f->Bz2, f->Bx1, f->Bx2,
+    float* ps[] = {f->par, f->grad, f->m1, f->m2, f->Fx, f->By1, f->Bz1, f->Bx1,
                    f->feat, f->hq, f->zq, f->out, f->gbuf0, f->gbuf1, f->gT, f->gT2, f->gout};
     for (float* p : ps)
         if (p) cudaFree(p);
@@ -721,16 +714,32 @@ cudaError_t mix_back(psatd_fno* f, const float* gU, const float* V, const float*
     return cudaGetLastError();
 }
 
-// forward pass; leaves activations for the backward pass
-psatd_status fno_forward(psatd_fno* f, const float* prm, int B) {
+// A product followed by a bias per row of C and, with gelu, the activation; the
+// pre-activation is kept in C if `keep`.
+GemmArgs with_bias(GemmArgs g, const float* bias, float* act, bool gelu, bool keep) {
+    g.bias = bias;
+    g.act = act;
+    g.gelu = gelu;
+    g.store_c = keep;
+    return g;
+}
+
+// the complex stages: C = A B + A2 B2 (real and imaginary part)
+GemmArgs paired(GemmArgs g, const float* A2, const float* B2) {
+    g.A2 = A2;
+    g.B2 = B2;
+    return g;
+}
+
+// forward pass; with `train` it leaves the pre-activations for the backward pass
+psatd_status fno_forward(psatd_fno* f, const float* prm, int B, bool train) {
     const int P = f->P, C = f->C, m = f->m, NT = f->NT, FI = f->NP + 3;
     const long long NV = f->NV;
     cudaStream_t s = f->stream;
     features_kernel<<<grid_for(B * FI * NV), 256, 0, s>>>(prm, f->NP, B, P, f->feat);
-    // lift: pre0[b] = W_lift (C x FI) feat[b] (FI x NV)
-    FCK(launch_gemm(G(C, (int)NV, FI, f->par + f->o_lift_w, FI, 1, f->feat, NV, 1, f->pre[0], NV, 1, 0.f, B, 0,
-                      FI * NV, C * NV), s));
-    bias_act_kernel<<<grid_for(B * C * NV), 256, 0, s>>>(f->pre[0], f->act[0], f->par + f->o_lift_b, B, C, NV, 0);
+    // lift: act0[b] = W_lift (C x FI) feat[b] (FI x NV) + b_lift
+    FCK(launch_gemm(with_bias(G(C, (int)NV, FI, f->par + f->o_lift_w, FI, 1, f->feat, NV, 1, f->act[0], NV, 1, 0.f, B, 0,
+                                FI * NV, C * NV), f->par + f->o_lift_b, nullptr, false, true), s));
     for (int l = 0; l < f->L; ++l) {
         const float* v = f->act[l];
         float* z = f->pre[l + 1];
@@ -739,49 +748,41 @@ psatd_status fno_forward(psatd_fno* f, const float* prm, int B) {
         FCK(launch_gemm(G((int)M1, 2 * m, P, v, P, 1, f->Fx, 2 * m, 1, f->T1[l], 1, M1, 0.f), s));
         // Y: rows (kx,b,c,z) per part, contract y; out [(part,ky)][rows]
         const long long Mh = (long long)m * B * C * P;
-        FCK(launch_gemm(G((int)Mh, 2 * NT, P, f->T1[l], P, 1, f->By1, 2 * NT, 1, f->T2[l], 1, Mh, 0.f), s));
-        FCK(launch_gemm(G((int)Mh, 2 * NT, P, f->T1[l] + Mh * P, P, 1, f->By2, 2 * NT, 1, f->T2[l], 1, Mh, 1.f), s));
+        FCK(launch_gemm(paired(G((int)Mh, 2 * NT, P, f->T1[l], P, 1, f->By1, 2 * NT, 1, f->T2[l], 1, Mh, 0.f),
+                               f->T1[l] + Mh * P, f->By2), s));
         // Z: rows (ky,kx,b,c) per part, contract z
         const long long Mz = (long long)NT * m * B * C;
-        FCK(launch_gemm(G((int)Mz, 2 * NT, P, f->T2[l], P, 1, f->By1, 2 * NT, 1, f->T3[l], 1, Mz, 0.f), s));
-        FCK(launch_gemm(G((int)Mz, 2 * NT, P, f->T2[l] + Mz * P, P, 1, f->By2, 2 * NT, 1, f->T3[l], 1, Mz, 1.f), s));
+        FCK(launch_gemm(paired(G((int)Mz, 2 * NT, P, f->T2[l], P, 1, f->By1, 2 * NT, 1, f->T3[l], 1, Mz, 0.f),
+                               f->T2[l] + Mz * P, f->By2), s));
         // mode mixing: T3 = [part][kz][ky][kx][b][c] = [part][mode][b][c]
         FCK(mix_fwd(f, f->T3[l], f->par + f->o_R[l], f->U3[l], B));
         // Zi: rows r = (ky,kx,b,o), K = kz (stride Mz); out W1[(part,z)][r]
-        FCK(launch_gemm(G((int)Mz, 2 * P, NT, f->U3[l], 1, Mz, f->Bz1, 2 * P, 1, f->W1[l], 1, Mz, 0.f), s));
-        FCK(launch_gemm(G((int)Mz, 2 * P, NT, f->U3[l] + (long long)NT * Mz, 1, Mz, f->Bz2, 2 * P, 1, f->W1[l], 1, Mz, 1.f), s));
+        FCK(launch_gemm(paired(G((int)Mz, 2 * P, NT, f->U3[l], 1, Mz, f->Bz1, 2 * P, 1, f->W1[l], 1, Mz, 0.f),
+                               f->U3[l] + (long long)NT * Mz, f->Bz2), s));
         // Yi: W1[part][z][ky][Q], Q = (kx,b,o); batch z, rows Q, K = ky; out W2[(part,y)][z][Q]
         const long long Q = (long long)m * B * C;
-        FCK(launch_gemm(G((int)Q, 2 * P, NT, f->W1[l], 1, Q, f->Bz1, 2 * P, 1, f->W2[l], 1, (long long)P * Q, 0.f, P,
-                          (long long)NT * Q, 0, Q), s));
-        FCK(launch_gemm(G((int)Q, 2 * P, NT, f->W1[l] + (long long)P * NT * Q, 1, Q, f->Bz2, 2 * P, 1, f->W2[l], 1,
-                          (long long)P * Q, 1.f, P, (long long)NT * Q, 0, Q), s));
+        FCK(launch_gemm(paired(G((int)Q, 2 * P, NT, f->W1[l], 1, Q, f->Bz1, 2 * P, 1, f->W2[l], 1, (long long)P * Q, 0.f, P,
+                                 (long long)NT * Q, 0, Q), f->W1[l] + (long long)P * NT * Q, f->Bz2), s));
         // Xi: W2[part][y][z][kx][(b,o)]; batch (y, z), rows (b,o), K = kx; out z[(b,o)][z][y][x]
         {
             GemmArgs g = G(B * C, P, m, f->W2[l], 1, (long long)B * C, f->Bx1, P, 1, z, NV, 1, 0.f);
             g.nb0 = P; g.nb1 = P;
             g.sAb0 = (long long)P * Q; g.sAb1 = Q;               // y, z
             g.sCb0 = P; g.sCb1 = (long long)P * P;
-            FCK(launch_gemm(g, s));
-            g.A = f->W2[l] + (long long)P * P * Q;
-            g.B = f->Bx2;
-            g.beta = 1.f;
-            FCK(launch_gemm(g, s));
+            FCK(launch_gemm(paired(g, f->W2[l] + (long long)P * P * Q, f->Bx2), s));
         }
-        // pointwise W v added: z[b] += W (C x C) v[b]
-        FCK(launch_gemm(G(C, (int)NV, C, f->par + f->o_W[l], C, 1, v, NV, 1, z, NV, 1, 1.f, B, 0, C * NV, C * NV), s));
-        bias_act_kernel<<<grid_for(B * C * NV), 256, 0, s>>>(z, f->act[l + 1], f->par + f->o_b[l], B, C, NV,
-                                                            l + 1 < f->L ? 1 : 0);
+        // pointwise W v added, bias and activation: z[b] += W (C x C) v[b] + b, act = GELU(z)
+        // (the last layer has none, and its backward pass needs no z)
+        const bool gelu = l + 1 < f->L;
+        FCK(launch_gemm(with_bias(G(C, (int)NV, C, f->par + f->o_W[l], C, 1, v, NV, 1, z, NV, 1, 1.f, B, 0, C * NV,
+                                    C * NV), f->par + f->o_b[l], f->act[l + 1], gelu, train && gelu), s));
     }
     // projection
     const int H = f->H, NO = f->NO;
-    FCK(launch_gemm(G(H, (int)NV, C, f->par + f->o_q1_w, C, 1, f->act[f->L], NV, 1, f->zq, NV, 1, 0.f, B, 0, C * NV,
-                      H * NV), s));
-    bias_act_kernel<<<grid_for(B * H * NV), 256, 0, s>>>(f->zq, f->hq, f->par + f->o_q1_b, B, H, NV, 1);
-    FCK(launch_gemm(G(NO, (int)NV, H, f->par + f->o_q2_w, H, 1, f->hq, NV, 1, f->out, NV, 1, 0.f, B, 0, H * NV,
-                      NO * NV), s));
-    // bias only (no activation): out += b, in place
-    bias_act_kernel<<<grid_for(B * NO * NV), 256, 0, s>>>(f->out, f->out, f->par + f->o_q2_b, B, NO, NV, 0);
+    FCK(launch_gemm(with_bias(G(H, (int)NV, C, f->par + f->o_q1_w, C, 1, f->act[f->L], NV, 1, f->zq, NV, 1, 0.f, B, 0,
+                                C * NV, H * NV), f->par + f->o_q1_b, f->hq, true, train), s));
+    FCK(launch_gemm(with_bias(G(NO, (int)NV, H, f->par + f->o_q2_w, H, 1, f->hq, NV, 1, f->out, NV, 1, 0.f, B, 0,
+                                H * NV, NO * NV), f->par + f->o_q2_b, nullptr, false, true), s));
     FCK(cudaGetLastError());
     return PSATD_OK;
 }
@@ -806,6 +807,14 @@ cudaError_t gelu_back(psatd_fno* f, const float* z, const float* ga, float* gz, 
     act_back_kernel<true><<<B * C * kRowChunks, 256, 0, f->stream>>>(z, ga, gz, B, C, f->NV, f->bpart);
     bias_reduce_kernel<<<C, 32, 0, f->stream>>>(f->bpart, B * kRowChunks, gbias);
     return cudaGetLastError();
+}
+
+// An adjoint stage for both parts at once: columns n >= n of the second part lie
+// part_stride elements after the first's.
+GemmArgs both_parts(GemmArgs g, int n, long long part_stride) {
+    g.nsplit = n;
+    g.c_split = part_stride - n * g.sCn;
+    return g;
 }
 
 psatd_status fno_backward(psatd_fno* f, int B) {
@@ -842,40 +851,29 @@ psatd_status fno_backward(psatd_fno* f, int B) {
         const long long Q = (long long)m * B * C, Mz = (long long)NT * m * B * C, Mh = (long long)m * B * C * P;
         float* gW2 = f->gT;        // layout of W2
         {
-            GemmArgs a = G(B * C, m, P, gz, NV, 1, f->Bx1, 1, P, gW2, 1, (long long)B * C, 0.f);
+            GemmArgs a = G(B * C, 2 * m, P, gz, NV, 1, f->Bx1, 1, P, gW2, 1, (long long)B * C, 0.f);
             a.nb0 = P; a.nb1 = P;
             a.sAb0 = P; a.sAb1 = (long long)P * P;              // gz[(b,o)][z][y][x]: y stride P, z stride P^2
             a.sCb0 = (long long)P * Q; a.sCb1 = Q;
-            FCK(launch_gemm(a, s));
-            a.B = f->Bx2;
-            a.C = gW2 + (long long)P * P * Q;
-            FCK(launch_gemm(a, s));
+            FCK(launch_gemm(both_parts(a, m, (long long)P * P * Q), s));
         }
         // adjoint of Yi: g_W1[part'] = sum over (part, y) of gW2 rows; W2 = W1re*Bz1 + W1im*Bz2
         float* gW1 = f->gT2;
-        for (int part = 0; part < 2; ++part) {
-            GemmArgs a = G((int)Q, NT, 2 * P, gW2, 1, (long long)P * Q, part == 0 ? f->Bz1 : f->Bz2, 1, 2 * P,
-                           gW1 + (long long)part * P * NT * Q, 1, Q, 0.f, P, Q, 0, (long long)NT * Q);
-            FCK(launch_gemm(a, s));
-        }
+        FCK(launch_gemm(both_parts(G((int)Q, 2 * NT, 2 * P, gW2, 1, (long long)P * Q, f->Bz1, 1, 2 * P, gW1, 1, Q, 0.f, P,
+                                     Q, 0, (long long)NT * Q), NT, (long long)P * NT * Q), s));
         // adjoint of Zi: g_U[part'] rows (ky,kx,b,o), K over (part,z) of gW1
         float* gU = f->gT;
-        for (int part = 0; part < 2; ++part)
-            FCK(launch_gemm(G((int)Mz, NT, 2 * P, gW1, 1, Mz, part == 0 ? f->Bz1 : f->Bz2, 1, 2 * P,
-                              gU + (long long)part * NT * Mz, 1, Mz, 0.f), s));
+        FCK(launch_gemm(both_parts(G((int)Mz, 2 * NT, 2 * P, gW1, 1, Mz, f->Bz1, 1, 2 * P, gU, 1, Mz, 0.f), NT,
+                                   (long long)NT * Mz), s));
         // mixing: weights and spectra
         float* gV = f->gT2;
         FCK(mix_back(f, gU, f->T3[l], f->par + f->o_R[l], g + f->o_R[l], gV, B));
         // adjoint of Z: g_T2[part] (rows (ky,kx,b,c), K = z) = gV (rows, 2NT) * By_part^T
         float* gT2 = f->gT;
-        for (int part = 0; part < 2; ++part)
-            FCK(launch_gemm(G((int)Mz, P, 2 * NT, gV, 1, Mz, part == 0 ? f->By1 : f->By2, 1, 2 * NT,
-                              gT2 + (long long)part * Mz * P, P, 1, 0.f), s));
+        FCK(launch_gemm(both_parts(G((int)Mz, 2 * P, 2 * NT, gV, 1, Mz, f->By1, 1, 2 * NT, gT2, P, 1, 0.f), P, Mz * P), s));
         // adjoint of Y: g_T1[part] (rows (kx,b,c,z), K = y)
         float* gT1 = f->gT2;
-        for (int part = 0; part < 2; ++part)
-            FCK(launch_gemm(G((int)Mh, P, 2 * NT, gT2, 1, Mh, part == 0 ? f->By1 : f->By2, 1, 2 * NT,
-                              gT1 + (long long)part * Mh * P, P, 1, 0.f), s));
+        FCK(launch_gemm(both_parts(G((int)Mh, 2 * P, 2 * NT, gT2, 1, Mh, f->By1, 1, 2 * NT, gT1, P, 1, 0.f), P, Mh * P), s));
         // adjoint of X: g_v += gT1 (rows (b,c,z,y), 2m) * Fx^T
         const long long M1 = (long long)B * C * P * P;
         FCK(launch_gemm(G((int)M1, P, 2 * m, gT1, 1, M1, f->Fx, 1, 2 * m, ga, P, 1, 1.f), s));
@@ -893,7 +891,7 @@ extern "C" {
 
 psatd_status psatd_fno_forward(psatd_fno* f, const float* params_dev, int batch, float* out_dev) {
     if (!f || !params_dev || batch < 1 || batch > f->maxB) return fno_fail(f, PSATD_ERR_ARG, "bad arguments");
-    psatd_status st = fno_forward(f, params_dev, batch);
+    psatd_status st = fno_forward(f, params_dev, batch, false);
     if (st) return st;
     if (out_dev && out_dev != f->out) {
         FCK(cudaMemcpyAsync(out_dev, f->out, (size_t)batch * f->NO * f->NV * sizeof(float), cudaMemcpyDeviceToDevice,
@@ -906,7 +904,7 @@ psatd_status psatd_fno_loss_backward(psatd_fno* f, const float* params_dev, int 
                                      double* loss) {
     if (!f || !params_dev || !target_dev || batch < 1 || batch > f->maxB)
         return fno_fail(f, PSATD_ERR_ARG, "bad arguments");
-    psatd_status st = fno_forward(f, params_dev, batch);
+    psatd_status st = fno_forward(f, params_dev, batch, true);
     if (st) return st;
     const long long n = (long long)batch * f->NO * f->NV;
     const int nb = std::min(4096, grid_for(n));

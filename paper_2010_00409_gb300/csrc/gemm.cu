@@ -75,19 +75,17 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-template <int BN> struct TcCfg {
+template <int BN, bool DUAL> struct TcCfg {
     static constexpr int kStageA = TBM * TBK * 2;             // bytes of one A stage
     static constexpr int kStageB = BN * TBK * 2;
     static constexpr int kSmem = 2 * (kStageA + kStageB);
-    static constexpr int kCols = BN;                          // tensor-memory columns (a power of two, >= 32)
-    static constexpr int kBlocks = BN == 32 ? 5 : (BN == 64 ? 4 : 3);   // per SM
+    static constexpr int kCols = DUAL ? 2 * BN : BN;          // tensor-memory columns (a power of two, >= 32)
+    static constexpr int kBlocks = BN == 32 && !DUAL ? 5 : (BN <= 64 ? 4 : 3);   // per SM
 };
 
 struct TcTile {
     int m0, n0, kbeg, kend, nkb;
-    const float* A;
-    const float* B;
-    float* C;
+    long long offA, offB, offC;
 };
 
 __device__ __forceinline__ TcTile tc_tile(const GemmArgs& g, int tile, int ntm, int ntn, int BN) {
@@ -99,9 +97,9 @@ __device__ __forceinline__ TcTile tc_tile(const GemmArgs& g, int tile, int ntm, 
     const int split = bz % g.ksplit;
     const int bidx = bz / g.ksplit;
     const int b0 = bidx / g.nb1, b1 = bidx % g.nb1;
-    t.A = g.A + b0 * g.sAb0 + b1 * g.sAb1;
-    t.B = g.B + b0 * g.sBb0 + b1 * g.sBb1;
-    t.C = g.C + b0 * g.sCb0 + b1 * g.sCb1;
+    t.offA = b0 * g.sAb0 + b1 * g.sAb1;
+    t.offB = b0 * g.sBb0 + b1 * g.sBb1;
+    t.offC = b0 * g.sCb0 + b1 * g.sCb1;
     t.m0 = mt * TBM;
     t.n0 = nt * BN;
     const int kchunk = ((g.K + g.ksplit - 1) / g.ksplit + TBK - 1) / TBK * TBK;
@@ -168,9 +166,20 @@ __device__ __forceinline__ void tc_stage(unsigned char* dst, const float* __rest
     }
 }
 
+__device__ __forceinline__ void tc_ld8(uint32_t (&r)[8], uint32_t addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+}
+
+__device__ __forceinline__ float tc_gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+
 // Epilogue.  Warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the rows of its
 // lane quarter); the two warps of one quarter split the columns, read in loads of 8.
-template <int BN>
+// With a bias or an activation the result passes through them here: as a pass of its
+// own over the field (read, write back, write the activation) they took 235 us a layer
+// at 8 x 32 x 64^3 values, 0.2 ms of an inference.
+template <int BN, bool DUAL>
 __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, uint32_t acc_addr, bool have) {
     constexpr int parts = kTcThreads / 128, cols = BN / parts;
     static_assert(cols % 8 == 0, "column split");
@@ -178,32 +187,45 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
     const int quarter = warp & 3;
     const int m = t.m0 + 32 * quarter + lane, c0 = (warp >> 2) * cols;
     const bool row = m < g.M, need = g.ksplit == 1 && g.beta != 0.f && row;
+    long long crow = t.offC + m * g.sCm;
+    if (g.swapped && g.nsplit > 0 && m >= g.nsplit) crow += g.c_split;
+    const float brow = (g.bias && !g.swapped && row) ? g.bias[m] : 0.f;
 #pragma unroll 1
     for (int cc = 0; cc < cols; cc += 8) {
-        if (t.n0 + c0 + cc >= g.N) break;                      // (the same for every lane)
-        float* dst = t.C + m * g.sCm + (t.n0 + c0 + cc) * g.sCn;
-        const int nv = min(8, g.N - (t.n0 + c0 + cc));
+        const int n0 = t.n0 + c0 + cc;
+        if (n0 >= g.N) break;                                  // (the same for every lane)
+        const int nv = min(8, g.N - n0);
+        long long at = crow + n0 * g.sCn;
+        // a column split falls on a multiple of 8 or is found column by column
+        const int split = (!g.swapped && g.nsplit > 0) ? g.nsplit - n0 : 8;
+        auto off = [&](int i) { return at + i * g.sCn + (i >= split ? g.c_split : 0); };
         float cv[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) cv[i] = (need && i < nv) ? dst[i * g.sCn] : 0.f;
-        uint32_t r[8];
+        for (int i = 0; i < 8; ++i) cv[i] = (need && i < nv) ? g.C[off(i)] : 0.f;
+        uint32_t r[8], r2[8];
+        const uint32_t col = acc_addr + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(c0 + cc);
         if (have) {
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7])
-                         : "r"(acc_addr + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(c0 + cc)));
+            tc_ld8(r, col);
+            if constexpr (DUAL) tc_ld8(r2, col + BN);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = 0u;
+            for (int i = 0; i < 8; ++i) r[i] = r2[i] = 0u;
         }
         if (row) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 if (i < nv) {
-                    const float v = g.alpha * __uint_as_float(r[i]);
-                    if (g.ksplit > 1) atomicAdd(dst + i * g.sCn, v);
-                    else dst[i * g.sCn] = (g.beta == 0.f) ? v : v + g.beta * cv[i];
+                    float v = g.alpha * __uint_as_float(r[i]);
+                    if (g.ksplit > 1) {
+                        atomicAdd(&g.C[off(i)], v);
+                        continue;
+                    }
+                    if (g.beta != 0.f) v = v + g.beta * cv[i];
+                    if constexpr (DUAL) v = g.alpha * __uint_as_float(r2[i]) + v;
+                    if (g.bias) v = v + (g.swapped ? g.bias[n0 + i] : brow);
+                    if (g.store_c) g.C[off(i)] = v;
+                    if (g.act) g.act[off(i)] = g.gelu ? tc_gelu(v) : v;
                 }
             }
         }
@@ -211,9 +233,9 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kTcThreads, TcCfg<BN>::kBlocks) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
-    using Cfg = TcCfg<BN>;
+template <int BN, bool DUAL>
+__global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
+    using Cfg = TcCfg<BN, DUAL>;
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t sbar[2], abar;
@@ -237,36 +259,39 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<BN>::kBlocks) gemm_tc_kernel
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                ((uint32_t)(TBM >> 4) << 24);
     const bool vecA = g.sAk == 1 && (g.sAm & 3) == 0 && (g.sAb0 & 3) == 0 && (g.sAb1 & 3) == 0 &&
-                      (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+                      ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.A2)) & 15) == 0;
     const bool vecB = g.sBk == 1 && (g.sBn & 3) == 0 && (g.sBb0 & 3) == 0 && (g.sBb1 & 3) == 0 &&
-                      (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
+                      ((reinterpret_cast<uintptr_t>(g.B) | reinterpret_cast<uintptr_t>(g.B2)) & 15) == 0;
     bool ok = true;
     uint32_t it = 0, tl = 0;
 #pragma unroll 1
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tl) {
         const TcTile t = tc_tile(g, tile, ntm, ntn, BN);
+        // K blocks of the first product, then (DUAL) of the second into its own columns
 #pragma unroll 1
-        for (int kb = 0; kb < t.nkb; ++kb, ++it) {
-            const int s = it & 1;
+        for (int kq = 0; kq < (DUAL ? 2 * t.nkb : t.nkb); ++kq, ++it) {
+            const bool second = DUAL && kq >= t.nkb;
+            const int s = it & 1, kb = second ? kq - t.nkb : kq;
             if (it >= 2) ok = tc_wait(&sbar[s], ((it - 2) >> 1) & 1) && ok;     // stage s read by the MMAs
             unsigned char* As = tc_raw + s * (Cfg::kStageA + Cfg::kStageB);
             unsigned char* Bs = As + Cfg::kStageA;
             const int k0 = t.kbeg + kb * TBK;
             const int nkk = min(TBK / 16, (t.kend - k0 + 15) / 16);         // K = 16 MMAs with data
-            tc_stage<TBM>(As, t.A, g.sAm, g.sAk, t.m0, g.M, k0, t.kend, vecA, 2 * nkk);
-            tc_stage<BN>(Bs, t.B, g.sBn, g.sBk, t.n0, g.N, k0, t.kend, vecB, 2 * nkk);
+            tc_stage<TBM>(As, (second ? g.A2 : g.A) + t.offA, g.sAm, g.sAk, t.m0, g.M, k0, t.kend, vecA, 2 * nkk);
+            tc_stage<BN>(Bs, (second ? g.B2 : g.B) + t.offB, g.sBn, g.sBk, t.n0, g.N, k0, t.kend, vecB, 2 * nkk);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> tensor-core reads
             // (every thread has also read the previous tile's accumulator by now)
             __syncthreads();
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t d = acc + (second ? BN : 0);
 #pragma unroll 1
                 for (int kk = 0; kk < nkk; ++kk) {
                     const uint64_t ad = tc_desc(tc_smem(As) + kk * 2 * (TBM / 8) * 128, (TBM / 8) * 128, 128);
                     const uint64_t bd = tc_desc(tc_smem(Bs) + kk * 2 * (BN / 8) * 128, (BN / 8) * 128, 128);
                     const uint32_t accum = (kb > 0 || kk > 0) ? 1u : 0u;
                     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc),
+                                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
                                  "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
                                  : "memory");
                 }
@@ -279,7 +304,7 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<BN>::kBlocks) gemm_tc_kernel
         if (tid == 0) tc_commit(&abar);
         ok = tc_wait(&abar, tl & 1) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tc_epilogue<BN>(g, t, acc, t.nkb > 0);
+        tc_epilogue<BN, DUAL>(g, t, acc, t.nkb > 0);
     }
     if (!ok) {
         if (tid == 0) atomicExch(&g_gemm_error, 1);
@@ -494,12 +519,39 @@ __global__ void scale_kernel(GemmArgs g) {
 
 }  // namespace
 
+namespace {
+template <int BN, bool DUAL>
+cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
+    using Cfg = TcCfg<BN, DUAL>;
+    const long long ntm = (g.M + TBM - 1) / TBM, ntn = (g.N + BN - 1) / BN;
+    const long long ntiles = ntm * ntn * (long long)g.nb0 * g.nb1 * g.ksplit;
+    if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    auto k = gemm_tc_kernel<BN, DUAL>;
+    // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        sms = n < 1 ? 1 : n;
+    }
+    const long long cap = (long long)sms * Cfg::kBlocks;
+    k<<<(unsigned)(ntiles < cap ? ntiles : cap), kTcThreads, Cfg::kSmem, s>>>(g, (int)ntm, (int)ntn, (int)ntiles);
+    return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
     if (a.M <= 0 || a.N <= 0 || a.nb0 <= 0 || a.nb1 <= 0) return cudaSuccess;
     GemmArgs g = a;
     if (g.ksplit < 1) g.ksplit = 1;
     if (g.K <= 0) g.ksplit = 1;
     if (g.ksplit > 1) {
+        if (g.A2 || g.nsplit || g.bias || g.act) return cudaErrorInvalidValue;
         scale_kernel<<<1024, 256, 0, s>>>(g);
     }
     // The epilogue writes one row per lane, so it coalesces when C is
@@ -511,36 +563,15 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
         t.M = g.N; t.N = g.M;
         t.A = g.B; t.sAb0 = g.sBb0; t.sAb1 = g.sBb1; t.sAm = g.sBn; t.sAk = g.sBk;
         t.B = g.A; t.sBb0 = g.sAb0; t.sBb1 = g.sAb1; t.sBk = g.sAk; t.sBn = g.sAm;
+        t.A2 = g.B2; t.B2 = g.A2;
         t.sCm = g.sCn; t.sCn = g.sCm;
+        t.swapped = true;
         g = t;
     }
-    {
-        const int bn = g.N <= 32 ? 32 : (g.N <= 64 ? 64 : 128);
-        const int bi = bn == 32 ? 0 : (bn == 64 ? 1 : 2);
-        const long long ntm = (g.M + TBM - 1) / TBM, ntn = (g.N + bn - 1) / bn;
-        const long long ntiles = ntm * ntn * (long long)g.nb0 * g.nb1 * g.ksplit;
-        if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-        auto k = bi == 0 ? gemm_tc_kernel<32> : (bi == 1 ? gemm_tc_kernel<64> : gemm_tc_kernel<128>);
-        const int smem = bi == 0 ? TcCfg<32>::kSmem : (bi == 1 ? TcCfg<64>::kSmem : TcCfg<128>::kSmem);
-        // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
-        static int sms = 0, smem_launch[3] = {0, 0, 0};
-        const int per_sm[3] = {TcCfg<32>::kBlocks, TcCfg<64>::kBlocks, TcCfg<128>::kBlocks};
-        if (!smem_launch[bi]) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (sms < 1) sms = 1;
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return e;
-            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            if (e != cudaSuccess) return e;
-            smem_launch[bi] = smem;
-        }
-        const long long cap = (long long)sms * per_sm[bi];
-        const long long grid = ntiles < cap ? ntiles : cap;
-        k<<<(unsigned)grid, kTcThreads, smem_launch[bi], s>>>(g, (int)ntm, (int)ntn, (int)ntiles);
-        return cudaGetLastError();
-    }
+    // two accumulators of 64 columns let four blocks share the SM's tensor memory
+    if (g.A2) return g.N <= 32 ? gemm_tc_launch<32, true>(g, s) : gemm_tc_launch<64, true>(g, s);
+    return g.N <= 32 ? gemm_tc_launch<32, false>(g, s)
+                     : g.N <= 64 ? gemm_tc_launch<64, false>(g, s) : gemm_tc_launch<128, false>(g, s);
 }
 
 namespace {
