@@ -415,6 +415,7 @@ struct GemmArgs {
     float alpha, beta;
     int ksplit;
     // Optional (null / 0), with ksplit 1:
+    // (A2 with neither of the others, nsplit not with bias or act)
     //  A2, B2  a second product of the same shape and strides, accumulated apart:
     //          C = alpha A2 B2 + alpha A B + beta C, added in that order;
     //  nsplit  columns n >= nsplit of C lie c_split elements further on;

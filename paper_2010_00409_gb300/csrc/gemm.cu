@@ -174,12 +174,16 @@ __device__ __forceinline__ void tc_ld8(uint32_t (&r)[8], uint32_t addr) {
 
 __device__ __forceinline__ float tc_gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 
+// Epilogue forms: the plain one; a bias and an activation; a split output.
+enum TcEpi { EPI_PLAIN = 0, EPI_ACT = 1, EPI_SPLIT = 2 };
+
 // Epilogue.  Warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the rows of its
 // lane quarter); the two warps of one quarter split the columns, read in loads of 8.
 // With a bias or an activation the result passes through them here: as a pass of its
 // own over the field (read, write back, write the activation) they took 235 us a layer
-// at 8 x 32 x 64^3 values, 0.2 ms of an inference.
-template <int BN, bool DUAL>
+// at 8 x 32 x 64^3 values, 0.2 ms of an inference.  The forms are compiled apart: one
+// epilogue with all of them in it slowed the plain one by 15 to 60 %.
+template <int BN, bool DUAL, int EPI>
 __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, uint32_t acc_addr, bool have) {
     constexpr int parts = kTcThreads / 128, cols = BN / parts;
     static_assert(cols % 8 == 0, "column split");
@@ -188,20 +192,28 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
     const int m = t.m0 + 32 * quarter + lane, c0 = (warp >> 2) * cols;
     const bool row = m < g.M, need = g.ksplit == 1 && g.beta != 0.f && row;
     long long crow = t.offC + m * g.sCm;
-    if (g.swapped && g.nsplit > 0 && m >= g.nsplit) crow += g.c_split;
-    const float brow = (g.bias && !g.swapped && row) ? g.bias[m] : 0.f;
+    if (EPI == EPI_SPLIT && g.swapped && m >= g.nsplit) crow += g.c_split;
+    const float brow = (EPI == EPI_ACT && g.bias && !g.swapped && row) ? g.bias[m] : 0.f;
 #pragma unroll 1
     for (int cc = 0; cc < cols; cc += 8) {
         const int n0 = t.n0 + c0 + cc;
         if (n0 >= g.N) break;                                  // (the same for every lane)
         const int nv = min(8, g.N - n0);
-        long long at = crow + n0 * g.sCn;
-        // a column split falls on a multiple of 8 or is found column by column
-        const int split = (!g.swapped && g.nsplit > 0) ? g.nsplit - n0 : 8;
-        auto off = [&](int i) { return at + i * g.sCn + (i >= split ? g.c_split : 0); };
+        const long long at = crow + n0 * g.sCn;
+        float* dst = g.C + at;
+        // columns from `split` on lie c_split further
+        const int split = (EPI == EPI_SPLIT && !g.swapped) ? g.nsplit - n0 : 8;
+        if (EPI == EPI_SPLIT && split <= 0) dst += g.c_split;
         float cv[8];
+        {
+            const float* p = dst;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) cv[i] = (need && i < nv) ? g.C[off(i)] : 0.f;
+            for (int i = 0; i < 8; ++i) {
+                if (EPI == EPI_SPLIT && i > 0 && i == split) p += g.c_split;
+                cv[i] = (need && i < nv) ? *p : 0.f;
+                p += g.sCn;
+            }
+        }
         uint32_t r[8], r2[8];
         const uint32_t col = acc_addr + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(c0 + cc);
         if (have) {
@@ -213,27 +225,36 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
             for (int i = 0; i < 8; ++i) r[i] = r2[i] = 0u;
         }
         if (row) {
+            float* p = dst;
+            float* pa = EPI == EPI_ACT ? g.act + at : nullptr;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
+                if (EPI == EPI_SPLIT && i > 0 && i == split) p += g.c_split;
                 if (i < nv) {
                     float v = g.alpha * __uint_as_float(r[i]);
-                    if (g.ksplit > 1) {
-                        atomicAdd(&g.C[off(i)], v);
-                        continue;
+                    if (EPI == EPI_PLAIN && !DUAL && g.ksplit > 1) {
+                        atomicAdd(p, v);
+                    } else {
+                        if (g.beta != 0.f) v = v + g.beta * cv[i];
+                        if constexpr (DUAL) v = g.alpha * __uint_as_float(r2[i]) + v;
+                        if constexpr (EPI == EPI_ACT) {
+                            v = v + (g.swapped ? (g.bias ? g.bias[n0 + i] : 0.f) : brow);
+                            if (g.act) pa[0] = g.gelu ? tc_gelu(v) : v;
+                            if (g.store_c) *p = v;
+                        } else {
+                            *p = v;
+                        }
                     }
-                    if (g.beta != 0.f) v = v + g.beta * cv[i];
-                    if constexpr (DUAL) v = g.alpha * __uint_as_float(r2[i]) + v;
-                    if (g.bias) v = v + (g.swapped ? g.bias[n0 + i] : brow);
-                    if (g.store_c) g.C[off(i)] = v;
-                    if (g.act) g.act[off(i)] = g.gelu ? tc_gelu(v) : v;
                 }
+                p += g.sCn;
+                if (EPI == EPI_ACT) pa += g.sCn;
             }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
 
-template <int BN, bool DUAL>
+template <int BN, bool DUAL, int EPI>
 __global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
     using Cfg = TcCfg<BN, DUAL>;
     extern __shared__ __align__(1024) unsigned char tc_raw[];
@@ -304,7 +325,7 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_
         if (tid == 0) tc_commit(&abar);
         ok = tc_wait(&abar, tl & 1) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tc_epilogue<BN, DUAL>(g, t, acc, t.nkb > 0);
+        tc_epilogue<BN, DUAL, EPI>(g, t, acc, t.nkb > 0);
     }
     if (!ok) {
         if (tid == 0) atomicExch(&g_gemm_error, 1);
@@ -520,13 +541,13 @@ __global__ void scale_kernel(GemmArgs g) {
 }  // namespace
 
 namespace {
-template <int BN, bool DUAL>
+template <int BN, bool DUAL, int EPI>
 cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
     using Cfg = TcCfg<BN, DUAL>;
     const long long ntm = (g.M + TBM - 1) / TBM, ntn = (g.N + BN - 1) / BN;
     const long long ntiles = ntm * ntn * (long long)g.nb0 * g.nb1 * g.ksplit;
     if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    auto k = gemm_tc_kernel<BN, DUAL>;
+    auto k = gemm_tc_kernel<BN, DUAL, EPI>;
     // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
     static int sms = 0;
     if (!sms) {
@@ -568,10 +589,20 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
         t.swapped = true;
         g = t;
     }
+    const bool act = g.bias || g.act, split = g.nsplit > 0;
+    if ((g.A2 && (act || split)) || (act && split)) return cudaErrorInvalidValue;
     // two accumulators of 64 columns let four blocks share the SM's tensor memory
-    if (g.A2) return g.N <= 32 ? gemm_tc_launch<32, true>(g, s) : gemm_tc_launch<64, true>(g, s);
-    return g.N <= 32 ? gemm_tc_launch<32, false>(g, s)
-                     : g.N <= 64 ? gemm_tc_launch<64, false>(g, s) : gemm_tc_launch<128, false>(g, s);
+    if (g.A2) return g.N <= 32 ? gemm_tc_launch<32, true, EPI_PLAIN>(g, s) : gemm_tc_launch<64, true, EPI_PLAIN>(g, s);
+    if (act)
+        return g.N <= 32 ? gemm_tc_launch<32, false, EPI_ACT>(g, s)
+                         : g.N <= 64 ? gemm_tc_launch<64, false, EPI_ACT>(g, s) : gemm_tc_launch<128, false, EPI_ACT>(g, s);
+    if (split)
+        return g.N <= 32 ? gemm_tc_launch<32, false, EPI_SPLIT>(g, s)
+                         : g.N <= 64 ? gemm_tc_launch<64, false, EPI_SPLIT>(g, s)
+                                     : gemm_tc_launch<128, false, EPI_SPLIT>(g, s);
+    return g.N <= 32 ? gemm_tc_launch<32, false, EPI_PLAIN>(g, s)
+                     : g.N <= 64 ? gemm_tc_launch<64, false, EPI_PLAIN>(g, s)
+                                 : gemm_tc_launch<128, false, EPI_PLAIN>(g, s);
 }
 
 namespace {
