@@ -111,7 +111,7 @@ struct PulseF32 {
     double cps, sps;        // cos, sin of the polarisation angle (float64 storage)
     FF x0, y0, z0, dx, dy, dz, D;      // the grid
     FF R0, k0, phase, two_pi, prof_z0, prof_inv_dz;
-    float halfL, inv2pi, lo2, hi2, pi_over_L, th, eps, inv_th2, g4, amp, amp_R0, ell;
+    float halfL, inv2pi, lo2, hi2, cos_max, pi_over_L, th, eps, inv_th2, g4, amp, amp_R0, ell;
     float cp[2], sp[2];     // cos, sin of the carrier phases cep and cep + pi/2 (profile kind)
     float cf, sf;           // cos, sin of the polarisation angle
 };
@@ -131,6 +131,12 @@ __device__ __forceinline__ bool shell_point(int i, int j, int l, int m, const Gr
     const float yf = fmaf((float)j, k.dy.h, k.y0.h), zf = fmaf((float)l, k.dz.h, k.z0.h);
     const float r2 = xf * xf + yf * yf + zf * zf;
     if (r2 < k.lo2 || r2 > k.hi2) return false;        // well outside the shell (margin 1e-4 in R^2)
+    // well outside the angular support: alpha > a_max means -x < R cos(a_max) (the margin
+    // in cos_max covers the float32 error of either side).  About two thirds of the
+    // shell's points of a replica fall to this, before their double-float geometry,
+    // carrier and window are worked out only to be multiplied by zero (256^3 real one-shot
+    // 938 -> 855 us).
+    if (-xf < sqrtf(r2) * k.cos_max) return false;
     const FF X = ff_add(ff_add(k.x0, ff_mul_f(k.dx, (float)i)), ff_mul_f(k.D, (float)m));
     const FF Y = ff_add(k.y0, ff_mul_f(k.dy, (float)j)), Z = ff_add(k.z0, ff_mul_f(k.dz, (float)l));
     const FF S = ff_add(ff_add(ff_sqr(X), ff_sqr(Y)), ff_sqr(Z));
@@ -313,6 +319,14 @@ PulseF32 pulse_f32(const PulseParams& p, const ShellGeom& sh, const GridGeom& g)
     const float lo = (float)(sh.R0 - 0.5 * sh.L), hi = (float)(sh.R0 + 0.5 * sh.L);
     k.lo2 = lo * lo * 0.9999f;
     k.hi2 = hi * hi * 1.0001f;
+    // the support ends at alpha = theta + eps/2 (Gaussian: 2 theta + eps/2); at pi or
+    // beyond no angle is outside
+    const double a_max = (p.kind == 1 ? 2.0 : 1.0) * p.theta + 0.5 * p.eps;
+    // (margin: also ten times the float32 rounding of the coordinates against R_min)
+    const double r_min = sh.R0 - 0.5 * sh.L, far = 2 * fabs(g.x_min) + g.Nx * g.dx + sh.R0 + 0.5 * sh.L +
+                                                   fabs(g.y_min) + g.Ny * g.dy + fabs(g.z_min) + g.Nz * g.dz;
+    const double margin = r_min > 0.0 ? fmax(1e-4, 1e-6 * far / r_min) : 2.0;
+    k.cos_max = (a_max >= kPi || !(margin < 1.0)) ? -2.f : (float)(cos(a_max) - margin);
     k.pi_over_L = (float)(kPi / sh.L);
     k.th = (float)p.theta;
     k.eps = (float)p.eps;
