@@ -157,6 +157,24 @@ __device__ __forceinline__ double cell_energy3(cplx<T> a, cplx<T> b, cplx<T> c) 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Host: launch k on s with programmatic completion, so that its blocks fill the SMs
+// as the previous kernel's last blocks leave.  k must call pdl_wait() in every thread
+// before it touches memory that kernels write.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // 1D plan of one axis: N = prod(radix[0..npass)), radices up to 16 (narrow plans)
 // or 32 out of those fft_mixed.cuh has a register DFT for; N = 1 is one radix 1
@@ -214,6 +232,7 @@ template <typename T> struct Tables {
     const ModeCoef<T>* coef;    // (Nz/2+1) x (Ny/2+1) x (Nx/2+1)
     AxisPlan plan[3];
     const cplx<T>* twp[3];      // the plan's twiddles in position order (fft_mixed.cuh)
+    const cplx<T>* twn[3];      // the same of the plan of radices up to 16
     int tile_shift = 0;         // generic kernels: tile width scaled by 2^tile_shift (autotuner)
 };
 
@@ -280,6 +299,11 @@ cudaError_t launch_fft_axis_fast(cplx<T>* data, int ncomp, const GridGeom& g, co
                                  int axis, int dir, cudaStream_t s);
 template <typename T>
 cudaError_t launch_kspace_fast(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, cudaStream_t s);
+
+// float32 y or z transform of 512 or 1024 points (fft_three.cu), tp the twiddles
+// Tables::twn of the axis; cudaErrorNotSupported (nothing launched) otherwise.
+cudaError_t launch_fft_three(float2* data, int ncomp, const GridGeom& g, const float2* tp, int axis, int dir,
+                             cudaStream_t s);
 
 // Fused x pass of a step in z, y, x order (N_x = 512 or 1024 in float32,
 // complex storage): forward x, the Eq. 3-4 update of every mode, inverse x, one

@@ -55,6 +55,8 @@ fft_axis_kernel(cplx<T>* __restrict__ data, int axis, int Nx, int Ny, int Nz, in
         t.nw = min(W, Nx - x0);
         t.P = t.run = t.gap = 0;
     }
+    pdl_launch_dependents();
+    pdl_wait();
     mix_transform<T, S, MAXR, ROWS, false>(t, sm, pl, tp);
 }
 
@@ -104,9 +106,9 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
         auto k = fft_axis_kernel<T, decltype(sc)::value, decltype(mc)::value, decltype(rc)::value>;
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k<<<(unsigned)nblocks, threads, smem, s>>>(data, axis, g.Nx, g.Ny, g.Nz, ncomp, W, logw, pl, tb.twp[axis]);
         if (nlaunch) ++*nlaunch;
-        return cudaGetLastError();
+        return launch_pdl(k, dim3((unsigned)nblocks), dim3(threads), smem, s, data, axis, g.Nx, g.Ny, g.Nz, ncomp, W,
+                          logw, pl, tb.twp[axis]);
     };
     auto by_rows = [&](auto sc, auto mc) {
         return axis == 0 ? launch(sc, mc, std::true_type{}) : launch(sc, mc, std::false_type{});

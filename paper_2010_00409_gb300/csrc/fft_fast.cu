@@ -27,29 +27,8 @@ template <typename T, int N1, int N2> struct RowsCfg {
     static constexpr int threads = G * N2;
 };
 
-// columns per block for the strided kernel: 128 contiguous bytes per row of the
-// tile, halved until the exchange buffer fits the shared-memory budget.  Along
-// z, whose rows lie a whole plane apart, 128 KB (at 1024^2 planes, 32-byte runs
-// 8 MB apart used the DRAM bursts poorly: the z transforms took 2.3 times as
-// long as with 128-byte runs, and 64-byte runs at two blocks per SM 1.16
-// times).  Along y (rows one plane row apart) 48 KB, or 64 KB for 1024-point
-// columns: eight columns, 256 threads held to 128 registers so that two blocks
-// share an SM (at 1024^3, 47.1 against 51.4 ms per step in one process for four
-// columns at 166 registers, three blocks per SM).
-#ifndef PSATD_COLS_Y_BUDGET
-#define PSATD_COLS_Y_BUDGET (48 * 1024)
-#endif
-template <typename T, int N, bool ZAXIS> constexpr int cols_width() {
-    const int budget = ZAXIS ? 128 * 1024 : (N >= 1024 ? 64 * 1024 : PSATD_COLS_Y_BUDGET);
-    int w = 128 / (int)sizeof(cplx<T>);
-    while (w > 1 && N * w * (int)sizeof(cplx<T>) > budget) w /= 2;
-    return w;
-}
-// 1024-point columns: blocks per SM for the launch bounds, so that 512 threads
-// share the register file (at most 128 registers a thread)
-template <int N, int THREADS> constexpr int cols_min_blocks() {
-    return (N >= 1024 && THREADS < 512) ? 512 / THREADS : 1;
-}
+// columns per block for the strided kernel: 128 contiguous bytes per row of the tile
+template <typename T> constexpr int cols_width() { return 128 / (int)sizeof(cplx<T>); }
 
 template <typename T, int N1, int N2, int S>
 __global__ void __launch_bounds__(RowsCfg<T, N1, N2>::threads)
@@ -60,6 +39,8 @@ fft_rows_kernel(cplx<T>* __restrict__ data, long long rows, const cplx<T>* __res
     __shared__ cplx<T> scratch[G * N1 * RS];
     const int g = threadIdx.x / N2, j = threadIdx.x % N2;
     const long long row = (long long)blockIdx.x * G + g;
+    pdl_launch_dependents();
+    pdl_wait();
     if (row >= rows) return;          // whole groups exit together; groups never straddle warps
     // barrier mask of this group's N2 lanes only (other groups of the warp may have exited)
     const unsigned lane0 = (threadIdx.x & 31u) & ~(unsigned)(N2 - 1);
@@ -100,7 +81,7 @@ fft_rows_kernel(cplx<T>* __restrict__ data, long long rows, const cplx<T>* __res
 // Block = W columns x N2 threads (c fastest).  Tile g -> (comp, o, x-tile);
 // element n of column c at base + n*stride + c.
 template <typename T, int N1, int N2, int W, int S>
-__global__ void __launch_bounds__(W * N2, cols_min_blocks<N1 * N2, W * N2>())
+__global__ void __launch_bounds__(W * N2)
 fft_cols_kernel(cplx<T>* __restrict__ data, int Nx, int Ny, int Nz, int axis, const cplx<T>* __restrict__ tw) {
     constexpr int RS = N2 * W, ES = W;
     extern __shared__ __align__(16) unsigned char cols_smem[];
@@ -118,6 +99,8 @@ fft_cols_kernel(cplx<T>* __restrict__ data, int Nx, int Ny, int Nz, int axis, co
     const GBuf<cplx<T>> F{data, (long long)(gridDim.x / (ntile * outerN)) * plane * Nz};
     cplx<T>* sc = scratch + c;
     cplx<T> v[N1];
+    pdl_launch_dependents();
+    pdl_wait();
     if constexpr (S < 0) {
         static_for<0, N1>([&](auto nc) { v[decltype(nc)::value] = F.at(base, (long long)(j + N2 * decltype(nc)::value) * stride); });
         stage_a_fwd<T, S, N1, N2>(v, j, tw);
@@ -170,6 +153,8 @@ kspace_cols_kernel(cplx<T>* __restrict__ data, int Nx, int Ny, const cplx<T>* __
     cplx<T>* base = data + (size_t)y * Nx + ix;
     const GBuf<cplx<T>> F{data, 6LL * (long long)cstride};
     cplx<T> v[N1];
+    pdl_launch_dependents();
+    pdl_wait();
 
     // forward z transforms: spectrum of component q -> slot q
     for (int q = 0; q < 6; ++q) {
@@ -243,24 +228,23 @@ cudaError_t cols_launch(cplx<T>* data, int ncomp, const GridGeom& g, const cplx<
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k<<<(unsigned)blocks, W * N2, smem, s>>>(data, g.Nx, g.Ny, g.Nz, axis, tw);
-    return cudaGetLastError();
+    return launch_pdl(k, dim3((unsigned)blocks), dim3(W * N2), smem, s, data, g.Nx, g.Ny, g.Nz, axis, tw);
+}
+
+template <typename T, int N1, int N2>
+cudaError_t rows_fast(cplx<T>* data, int ncomp, const GridGeom& g, const cplx<T>* tw, int dir, cudaStream_t s) {
+    const long long rows = (long long)ncomp * g.Nz * g.Ny;
+    using Cfg = RowsCfg<T, N1, N2>;
+    const unsigned blocks = (unsigned)((rows + Cfg::G - 1) / Cfg::G);
+    auto k = dir < 0 ? fft_rows_kernel<T, N1, N2, -1> : fft_rows_kernel<T, N1, N2, +1>;
+    return launch_pdl(k, dim3(blocks), dim3(Cfg::threads), 0, s, data, rows, tw);
 }
 
 template <typename T, int N1, int N2>
 cudaError_t axis_fast(cplx<T>* data, int ncomp, const GridGeom& g, const cplx<T>* tw, int axis, int dir,
                       cudaStream_t s) {
-    constexpr int N = N1 * N2;
-    if (axis == 0) {
-        const long long rows = (long long)ncomp * g.Nz * g.Ny;
-        using Cfg = RowsCfg<T, N1, N2>;
-        const unsigned blocks = (unsigned)((rows + Cfg::G - 1) / Cfg::G);
-        if (dir < 0) fft_rows_kernel<T, N1, N2, -1><<<blocks, Cfg::threads, 0, s>>>(data, rows, tw);
-        else fft_rows_kernel<T, N1, N2, +1><<<blocks, Cfg::threads, 0, s>>>(data, rows, tw);
-        return cudaGetLastError();
-    }
-    return axis == 2 ? cols_launch<T, N1, N2, cols_width<T, N, true>()>(data, ncomp, g, tw, axis, dir, s)
-                     : cols_launch<T, N1, N2, cols_width<T, N, false>()>(data, ncomp, g, tw, axis, dir, s);
+    if (axis == 0) return rows_fast<T, N1, N2>(data, ncomp, g, tw, dir, s);
+    return cols_launch<T, N1, N2, cols_width<T>()>(data, ncomp, g, tw, axis, dir, s);
 }
 
 }  // namespace
@@ -276,10 +260,12 @@ cudaError_t launch_fft_axis_fast(cplx<T>* data, int ncomp, const GridGeom& g, co
         case 128: return axis_fast<T, 16, 8>(data, ncomp, g, tw, axis, dir, s);
         case 256: return axis_fast<T, 16, 16>(data, ncomp, g, tw, axis, dir, s);
         case 512:
-            if constexpr (sizeof(T) == 4) return axis_fast<T, 32, 16>(data, ncomp, g, tw, axis, dir, s);
-            return cudaErrorNotSupported;
         case 1024:
-            if constexpr (sizeof(T) == 4) return axis_fast<T, 32, 32>(data, ncomp, g, tw, axis, dir, s);
+            if constexpr (sizeof(T) == 4) {
+                if (axis != 0) return launch_fft_three(data, ncomp, g, tb.twn[axis], axis, dir, s);
+                return N == 512 ? rows_fast<T, 32, 16>(data, ncomp, g, tw, dir, s)
+                                : rows_fast<T, 32, 32>(data, ncomp, g, tw, dir, s);
+            }
             return cudaErrorNotSupported;
         default: return cudaErrorNotSupported;
     }
@@ -292,8 +278,8 @@ cudaError_t kspace_fast_launch(cplx<T>* data, const GridGeom& g, const Tables<T>
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((long long)g.Ny * (g.Nx / W));
-    k<<<blocks, W * N2, smem, s>>>(data, g.Nx, g.Ny, tb.tw[2], tb.k[0], tb.k[1], tb.k[2], tb.coef);
-    return cudaGetLastError();
+    return launch_pdl(k, dim3(blocks), dim3(W * N2), smem, s, data, g.Nx, g.Ny, tb.tw[2], tb.k[0], tb.k[1], tb.k[2],
+                      tb.coef);
 }
 
 template <typename T>

@@ -83,6 +83,8 @@ two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
     float2* base = a.data + comp * plane * a.Nz + (a.axis == 1 ? o * plane : (size_t)o * a.Nx) + x0 + c;
     const GBuf<float2> F{a.data, (long long)a.ncomp * plane * a.Nz};
     const bool col = x0 + c < (unsigned)a.Nx;
+    pdl_launch_dependents();
+    pdl_wait();
     if (col && t < R2) {
         float2 v[R1];
         const float2* p = base + t * stride;
@@ -118,6 +120,8 @@ two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
     float2* base = a.data + row0 * N;
     const GBuf<float2> F{a.data, rows * N};
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
     if (tid < nrow * R2) {
         const int w = tid / R2, j = tid - w * R2;
         const float2* p = base + w * N + j;
@@ -153,6 +157,8 @@ two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__
     float2* base = a.data + (size_t)y * Nx + x0;
     const GBuf<float2> G{a.data, 6LL * (long long)cstride};
     const int nw = min(W, Nx - x0);
+    pdl_launch_dependents();
+    pdl_wait();
 
     // forward: level 0 from the field, level 1 in place
 #pragma unroll 1

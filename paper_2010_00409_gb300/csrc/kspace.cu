@@ -49,6 +49,8 @@ kspace_z_kernel(cplx<T>* __restrict__ data, int Nx, int Ny, int Nz, int W, int l
     t.nq = 6;
     t.slot = ct;
     t.P = t.run = t.gap = 0;
+    pdl_launch_dependents();
+    pdl_wait();
     mix_forward<T, MAXR, false>(t, F, pl, tp);
 
     const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1;
@@ -90,6 +92,8 @@ modes_kernel(cplx<T>* __restrict__ data, int Nx, int Ny, int Nz, const T* __rest
              T scale) {
     const size_t n = (size_t)Nx * Ny * Nz;
     const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1;
+    pdl_launch_dependents();
+    pdl_wait();
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         const int ix = (int)(e % Nx);
         const size_t r = e / Nx;
@@ -111,9 +115,8 @@ cudaError_t launch_modes(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, 
     const size_t n = (size_t)g.Nx * g.Ny * g.Nz;
     long long blocks = (long long)((n + kThreads - 1) / kThreads);
     if (blocks > 152LL * 32) blocks = 152LL * 32;
-    modes_kernel<T><<<(unsigned)blocks, kThreads, 0, s>>>(data, g.Nx, g.Ny, g.Nz, tb.k[0], tb.k[1], tb.k[2],
-                                                          tb.coef, mode, (T)scale);
-    return cudaGetLastError();
+    return launch_pdl(modes_kernel<T>, dim3((unsigned)blocks), dim3(kThreads), 0, s, data, g.Nx, g.Ny, g.Nz, tb.k[0],
+                      tb.k[1], tb.k[2], tb.coef, mode, (T)scale);
 }
 
 template cudaError_t launch_modes<float>(cplx<float>*, const GridGeom&, const Tables<float>&, int, double, cudaStream_t);
@@ -145,10 +148,9 @@ cudaError_t launch_kspace_z(cplx<T>* data, const GridGeom& g, const Tables<T>& t
         auto k = kspace_z_kernel<T, decltype(mc)::value>;
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k<<<(unsigned)nblocks, threads, smem, s>>>(data, g.Nx, g.Ny, g.Nz, W, logw, pl, tb.twp[2], tb.k[0], tb.k[1],
-                                                   tb.k[2], tb.coef, mode, (T)scale);
         if (nlaunch) ++*nlaunch;
-        return cudaGetLastError();
+        return launch_pdl(k, dim3((unsigned)nblocks), dim3(threads), smem, s, data, g.Nx, g.Ny, g.Nz, W, logw, pl,
+                          tb.twp[2], tb.k[0], tb.k[1], tb.k[2], tb.coef, mode, (T)scale);
     };
     return maxr <= kNarrow ? launch(std::integral_constant<int, kNarrow>{})
                            : launch(std::integral_constant<int, kWide>{});

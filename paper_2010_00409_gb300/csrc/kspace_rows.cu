@@ -1,5 +1,5 @@
-// Fused k-space pass along x for grids whose z length has no fused kernel
-// (complex storage, N_x = N1 * N2 with a register plan: 512 and 1024 in
+// Fused k-space pass along x for grids whose z length has no fused kernel or a
+// slower one (complex storage, N_x = N1 * N2 with a register plan: 512 and 1024 in
 // float32).  The step (Sec. 2.1, Eq. 3-4) then takes its transforms in the
 // order z, y, x and fuses the per-mode update into the x pass: one block takes
 // the six components of one (k_y, k_z) row, transforms each along x (one group
@@ -56,6 +56,7 @@ kspace_rows_kernel(cplx<T>* __restrict__ data, int Ny, int Nz, const cplx<T>* __
     const int ay = min(iy, Ny - iy), az = min(iz, Nz - iz);
     const long long ncoef = (long long)(Nz / 2 + 1) * Nyh * Nxh;
     const long long crow = ((long long)az * Nyh + ay) * Nxh;
+    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         // the row's Nx/2 + 1 table entries to L2 while the forward transforms run
         // (16-byte aligned range, clipped to whole 16-byte chunks of the table)
@@ -67,6 +68,7 @@ kspace_rows_kernel(cplx<T>* __restrict__ data, int Ny, int Nz, const cplx<T>* __
         if (hi > lo) prefetch_l2_bulk(reinterpret_cast<const void*>(lo), (uint32_t)(hi - lo));
     }
 
+    pdl_wait();
     // forward x transform of component q; its spectrum to the slot in natural order
     // (twiddles W^{j k1} from the [k1][j] table: a warp reads 32 consecutive entries)
     static_for<0, N1>([&](auto nc) { v[decltype(nc)::value] = F.at(p, j + N2 * decltype(nc)::value); });
@@ -157,8 +159,8 @@ cudaError_t rows_launch(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, c
     if (e != cudaSuccess) return e;
     const long long blocks = (long long)g.Ny * g.Nz;
     if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
-    k<<<(unsigned)blocks, 6 * N2, smem, s>>>(data, g.Ny, g.Nz, tb.tw2[0], tb.k[0], tb.k[1], tb.k[2], tb.coef);
-    return cudaGetLastError();
+    return launch_pdl(k, dim3((unsigned)blocks), dim3(6 * N2), smem, s, data, g.Ny, g.Nz, tb.tw2[0], tb.k[0], tb.k[1],
+                      tb.k[2], tb.coef);
 }
 
 }  // namespace

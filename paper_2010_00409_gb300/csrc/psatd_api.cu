@@ -327,6 +327,7 @@ Tables<T> tables(const psatd_ctx* c) {
         tb.k[a] = static_cast<const T*>(c->k[a].p);
         tb.plan[a] = c->plan[a];
         tb.twp[a] = static_cast<const cplx<T>*>(c->twp[a].p) + c->twp_at[a][0];
+        tb.twn[a] = static_cast<const cplx<T>*>(c->twp[a].p) + c->twp_at[a][1];
     }
     tb.coef = static_cast<const ModeCoef<T>*>(c->coef.p);
     for (int a = 0; a < 3; ++a) tb.tw2[a] = static_cast<const cplx<T>*>(c->tw2[a].p);
@@ -594,9 +595,8 @@ cudaError_t fft_axis_two(cplx<T>* data, int ncomp, const GridGeom& g, const Tabl
             axis == 0 ? ((long long)ncomp * g.Nz * g.Ny + e->rows_per_block - 1) / e->rows_per_block
                       : (long long)ncomp * (axis == 1 ? g.Nz : g.Ny) * ((g.Nx + 15) / 16);
         if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
-        void* args[] = {const_cast<TwoPassArgs*>(&a)};
-        const void* k = reinterpret_cast<const void*>(axis == 0 ? e->rows[dir > 0] : e->cols[dir > 0]);
-        return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(axis == 0 ? e->rows_threads : e->cols_threads), args, 0, s);
+        return launch_pdl(axis == 0 ? e->rows[dir > 0] : e->cols[dir > 0], dim3((unsigned)blocks),
+                          dim3(axis == 0 ? e->rows_threads : e->cols_threads), 0, s, a);
     }
     return cudaErrorNotSupported;
 }
@@ -610,12 +610,10 @@ cudaError_t kspace_two(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, in
         if (!e || pl.npass != 2 || pl.radix[0] != e->R1) return cudaErrorNotSupported;
         const TwoPassArgs a{data, tb.twp[2], 2, g.Nx, g.Ny, g.Nz, 6};
         const TwoPassModes m{tb.k[0], tb.k[1], tb.k[2], tb.coef, mode, (float)scale};
-        const void* k = reinterpret_cast<const void*>(e->kspace);
-        const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, e->kspace_smem);
+        const cudaError_t r = cudaFuncSetAttribute(e->kspace, cudaFuncAttributeMaxDynamicSharedMemorySize, e->kspace_smem);
         if (r != cudaSuccess) return r;
-        void* args[] = {const_cast<TwoPassArgs*>(&a), const_cast<TwoPassModes*>(&m)};
-        return cudaLaunchKernel(k, dim3((unsigned)((long long)g.Ny * ((g.Nx + 7) / 8))), dim3(256), args,
-                                (size_t)e->kspace_smem, s);
+        return launch_pdl(e->kspace, dim3((unsigned)((long long)g.Ny * ((g.Nx + 7) / 8))), dim3(256),
+                          (size_t)e->kspace_smem, s, a, m);
     }
     return cudaErrorNotSupported;
 }
@@ -684,10 +682,15 @@ cudaError_t spectral_pass(psatd_ctx* c, int mode, double scale) {
     const Tables<T> tb = tables<T>(c);
     cplx<T>* f = static_cast<cplx<T>*>(c->fields);
     cudaError_t e;
+    // the update fused into the x pass (N_x = 512, 1024) instead of the z pass: where the
+    // z pass has no fused kernel; at N_x = 512, whose row kernel is the faster of the
+    // two fused passes (512 x 256 x 256: 2.84 against 3.22 ms a step); and on planes of
+    // 4 MB or more, where the z pass's 64-byte rows a plane apart reach 2.3 TB/s (1024 x
+    // 512 x 256: 14.2 against 15.4 ms; 1024 x 256 x 256: 6.93 against 6.55 ms)
+    const bool fused_z = g.Nz == 64 || g.Nz == 128 || g.Nz == 256;
     if (mode == KS_ROTATE && c->kernel_path == PSATD_PATH_AUTO && kspace_rows_supported(c->prec, g) &&
-        !(g.Nz == 64 || g.Nz == 128 || g.Nz == 256)) {
-        // no fused z pass for this N_z: forward z, y; the update fused into the
-        // x pass (forward x, update, inverse x in one launch); inverse y, z
+        (!fused_z || g.Nx == 512 || (long long)g.Nx * g.Ny >= 512 * 1024)) {
+        // forward z, y; forward x, update, inverse x in one launch; inverse y, z
         if ((e = fft_axis<T>(c, f, 6, 2, -1, -1)) != cudaSuccess) return e;
         if ((e = fft_axis<T>(c, f, 6, 1, -1, -1)) != cudaSuccess) return e;
         e = timed(c, PSATD_KERNEL_KSPACE, [&] {

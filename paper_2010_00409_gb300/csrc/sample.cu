@@ -469,23 +469,6 @@ contract_yz_ff_kernel(const float4* __restrict__ A, const float4* __restrict__ B
     }
 }
 
-// Launch behind the previous kernel of the stream with programmatic completion
-// (each of these kernels waits for its predecessor before its first access).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_after(void (*k)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
-}
-
 // y and z contractions of float32 storage (g and the weights are in the scratch)
 cudaError_t contract_yz_ff(const GridGeom& g, const ShellGeom& sh, double x_phys, int ny, int nz, double y0, double y1,
                            double z0, double z1, double t, int ncomp, const SampleScratch& sc, float2* out,
@@ -498,10 +481,10 @@ cudaError_t contract_yz_ff(const GridGeom& g, const ShellGeom& sh, double x_phys
         constexpr int R = decltype(rc)::value;
         auto tiles = [](int n) { return (unsigned)((n + 8 * R - 1) / (8 * R)); };
         if constexpr (Z)
-            return launch_after(contract_yz_ff_kernel<true, R>, dim3(tiles(ny), tiles(nz), (unsigned)ncomp), kCThreads,
+            return launch_pdl(contract_yz_ff_kernel<true, R>, dim3(tiles(ny), tiles(nz), (unsigned)ncomp), kCThreads,
                                 0, s, wz, hh, nz, ny, g.Nz, (float4*)nullptr, g, sh, x_phys, y0, y1, z0, z1, t, out);
         else
-            return launch_after(contract_yz_ff_kernel<false, R>, dim3(tiles(ny), tiles(rows), 1), kCThreads, 0, s, gg,
+            return launch_pdl(contract_yz_ff_kernel<false, R>, dim3(tiles(ny), tiles(rows), 1), kCThreads, 0, s, gg,
                                 wy, rows, ny, g.Ny, reinterpret_cast<float4*>(sc.h), g, sh, x_phys, y0, y1, z0, z1, t,
                                 (float2*)nullptr);
     };
@@ -528,17 +511,17 @@ cudaError_t launch_sample_plane(const cplx<T>* data, const GridGeom& g, const Sh
     cudaError_t e;
     constexpr bool ffw = sizeof(T) == 4;               // float32 storage: double-float sums
     if (from_spectrum)
-        e = launch_after(spectral_weights_kernel<ffw>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
+        e = launch_pdl(spectral_weights_kernel<ffw>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
                          sc.wz);
     else
-        e = launch_after(weights_kernel<ffw>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
+        e = launch_pdl(weights_kernel<ffw>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
                          sc.wz);
     const long long rows = (long long)ncomp * g.Nz * g.Ny;
     if constexpr (ffw) {
         if (e != cudaSuccess) return e;
         const long long units = (rows + kXRows - 1) / kXRows;
         const unsigned xb = (unsigned)((units + kXThreads / kXL - 1) / (kXThreads / kXL));
-        e = launch_after(contract_x_ff_kernel<false>, dim3(xb), kXThreads, (size_t)g.Nx * sizeof(float4), s,
+        e = launch_pdl(contract_x_ff_kernel<false>, dim3(xb), kXThreads, (size_t)g.Nx * sizeof(float4), s,
                                      reinterpret_cast<const float*>(data), g, cl, ncomp,
                                      reinterpret_cast<const float4*>(sc.wx), reinterpret_cast<float4*>(sc.g));
         if (e == cudaSuccess)
@@ -568,10 +551,10 @@ cudaError_t launch_sample_plane_real(const float* data, const float2* nyq, const
     const dim3 wgrid((nw + kWThreads - 1) / kWThreads);
     cudaError_t e;
     if (from_spectrum)
-        e = launch_after(spectral_weights_kernel<true>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
+        e = launch_pdl(spectral_weights_kernel<true>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
                          sc.wz);
     else
-        e = launch_after(weights_kernel<true>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
+        e = launch_pdl(weights_kernel<true>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
                          sc.wz);
     const float4* wx = reinterpret_cast<const float4*>(sc.wx);
     float4* gg = reinterpret_cast<float4*>(sc.g);
@@ -579,12 +562,12 @@ cudaError_t launch_sample_plane_real(const float* data, const float2* nyq, const
     constexpr int per = kXThreads / kXL;
     if (from_spectrum) {
         const long long units = (long long)ncomp * (g.Nz / 2 + 1) * g.Ny;
-        e = launch_after(contract_x_half_ff_kernel, dim3((unsigned)((units + per - 1) / per)), kXThreads,
+        e = launch_pdl(contract_x_half_ff_kernel, dim3((unsigned)((units + per - 1) / per)), kXThreads,
                          (size_t)(g.Nx / 2 + 1) * sizeof(float4), s, reinterpret_cast<const float2*>(data), nyq, g, cl,
                          ncomp, slot_mode, wx, gg);
     } else {
         const long long units = ((long long)ncomp * g.Nz * g.Ny + kXRows - 1) / kXRows;
-        e = launch_after(contract_x_ff_kernel<true>, dim3((unsigned)((units + per - 1) / per)), kXThreads,
+        e = launch_pdl(contract_x_ff_kernel<true>, dim3((unsigned)((units + per - 1) / per)), kXThreads,
                          (size_t)g.Nx * sizeof(float4), s, data, g, cl, ncomp, wx, gg);
     }
     if (e == cudaSuccess) e = contract_yz_ff(g, sh, x_phys, ny, nz, y0, y1, z0, z1, t, ncomp, sc, out, s);

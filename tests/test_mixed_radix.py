@@ -62,3 +62,19 @@ def test_every_compile_time_length_matches_the_run_time_passes(lib):
                     ctx.advance(1)
                     out.append(ctx.get_field(-1))
             assert np.linalg.norm(out[0] - out[1]) <= 1e-6 * np.linalg.norm(out[1]), shape
+
+
+@pytest.mark.parametrize("shape", [(6, 512, 2), (18, 2, 512), (36, 1024, 1), (16, 1, 1024), (512, 3, 64), (512, 2, 512)])
+def test_three_pass_columns_and_row_fused_steps_match_oracle(lib, shape):
+    """512- and 1024-point y and z transforms over column tiles of 16 with a
+    remainder, and the row-fused step at N_x = 512 on a z length that also has a
+    fused z pass (float32, parity tolerance 1e-5)."""
+    nx, ny, nz = shape
+    g = W.GridSpec(nx, ny, nz, 0.5, 0.7, 0.3, 0.0, 0.0, 0.0, 1.0)
+    f = W.random_complex_field((6, nz, ny, nx), seed=ny)
+    with lib.Context(g, None, 0.3, 32) as ctx:
+        ctx.set_fields(f)
+        ctx.advance(1)
+        got = ctx.get_field(-1)
+    ref = O.advance(f, O.Grid(nx, ny, nz, g.dx, g.dy, g.dz, 0.0, 0.0, 0.0, 1.0), 0.3, 1)
+    assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
