@@ -249,9 +249,9 @@ long long psatd_launch_count(const psatd_ctx* ctx);
 /* Kernel selection: AUTO uses the register-resident kernels where the axis
  * length has one (64, 128, 256, 512; the k-space pass for Nz in 64, 128, 256,
  * fed by tensor copies), in float32 compile-time two-pass kernels for
- * the other lengths to 256 that are a product of two radices up to 16, and the
- * generic mixed-radix kernels elsewhere; REGISTER is AUTO without the tensor-copy feed; GENERIC forces the
- * generic kernels everywhere.  All compute the same transform; default AUTO. */
+ * the other lengths to 1024 that are a product of two radices up to 32, and the
+ * generic mixed-radix kernels elsewhere; REGISTER is AUTO without the tensor-copy
+ * feed; GENERIC forces the generic kernels everywhere.  All compute the same transform; default AUTO. */
 enum { PSATD_PATH_AUTO = 0, PSATD_PATH_GENERIC = 1, PSATD_PATH_REGISTER = 2 };
 psatd_status psatd_set_kernel_path(psatd_ctx* ctx, int path);
 

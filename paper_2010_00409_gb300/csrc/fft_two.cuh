@@ -1,4 +1,4 @@
-// float32 transforms of axis lengths N = R1 R2 (both radices at most 16) with the
+// float32 transforms of axis lengths N = R1 R2 (both radices at most 32) with the
 // radices, the tile and every shared-memory offset fixed at compile time: the
 // two-pass case of fft_mixed.cuh, whose passes this file repeats in the same
 // arithmetic order without the run-time index arithmetic.  At run time that arithmetic
@@ -15,7 +15,13 @@
 //   kspace  z forward, the per-mode update, z inverse for the six components of 8
 //           x-columns at one y, the spectra kept digit-reversed in shared memory
 //
-// Lengths: those whose plan of radices up to 16 has two passes (two_pass_entry).
+// Lengths: those to 1024 whose plan has two passes, of radices up to 16 where that is
+// enough (two_pass_entry).  Beyond 16 points a thread takes up to 128 registers, which
+// the run-time passes pay as well: 162^3 step 666 -> 530 us, 384 x 320 x 288 4.74 ->
+// 3.68 ms, 480 x 400 x 360 10.2 -> 7.2 ms.  Two limits: the 16-column tile of y and z
+// stops at 96 KB (900 points leave one block an SM: 228 us a pass of a 100 x 900 x 100
+// box, 220 us with the run-time passes' 8 columns), the k-space tile at 226 KB (588
+// points).
 // float64 stays with the run-time passes: it is bound by the float64 pipe.
 #pragma once
 
@@ -37,8 +43,9 @@ struct TwoPassModes {
 };
 struct TwoPassEntry {
     int N, R1;
-    int cols_threads, rows_threads, rows_per_block, kspace_smem;
-    void (*cols[2])(TwoPassArgs);           // forward, inverse
+    int cols_threads, cols_smem, rows_threads, rows_per_block, rows_smem;
+    int kspace_threads, kspace_smem;        // 0: the six components' tile does not fit
+    void (*cols[2])(TwoPassArgs);           // forward, inverse (null: tile too large)
     void (*rows[2])(TwoPassArgs);
     void (*kspace)(TwoPassArgs, TwoPassModes);
 };
@@ -46,18 +53,28 @@ struct TwoPassEntry {
 const TwoPassEntry* two_pass_entry(int N);
 
 #ifdef __CUDACC__
-constexpr int kTwoW = 16, kTwoKW = 8, kTwoKThreads = 256;
+constexpr int kTwoW = 16, kTwoKW = 8;
 
 template <int R1, int R2> struct TwoCfg {
     static constexpr int N = R1 * R2;
     static_assert(R1 >= R2, "the first radix is the larger");
+    // registers a thread the register DFTs of the larger radix need
+    static constexpr int regs = R1 <= 12 ? 64 : (R1 <= 16 ? 80 : (R1 <= 20 ? 96 : 128));
+    static constexpr int blocks(int threads, int smem) {
+        const int by_regs = 65536 / regs / threads, by_smem = 220 * 1024 / (smem + 1024);
+        return by_regs < 1 || by_smem < 1 ? 1 : (by_regs < by_smem ? by_regs : by_smem);
+    }
     static constexpr int cols_threads = (R1 * kTwoW + 31) / 32 * 32;
-    // registers: 64 a thread where the first DFT has at most 12 points, else 80
-    static constexpr int cols_blocks = (R1 <= 12 ? 1024 : 768) / cols_threads;
+    static constexpr int cols_smem = N * kTwoW * (int)sizeof(float2);
+    static constexpr bool cols = cols_smem < 96 * 1024;
     static constexpr int G = 256 / R1;                                  // rows per block
     static constexpr int rows_threads = (G * R1 + 31) / 32 * 32;
-    static constexpr int rows_blocks = (R1 <= 12 ? 1024 : 768) / rows_threads;
     static constexpr int run = R2 | 1, P = (R1 * run) | 1;              // row layout of fft_mixed.cuh
+    static constexpr int rows_smem = G * P * (int)sizeof(float2);
+    // k-space: 256 threads where three or more tiles share an SM, else as many as keep it busy
+    static constexpr int kspace_smem = 6 * N * kTwoKW * (int)sizeof(float2);
+    static constexpr bool kspace = kspace_smem <= 226 * 1024;
+    static constexpr int kspace_threads = kspace_smem <= 75 * 1024 ? 256 : 512;
 };
 
 // multiply v[k] by the position-ordered twiddles W_N^{jk} (conjugated for S > 0)
@@ -71,10 +88,12 @@ __device__ __forceinline__ void two_twiddle(float2 (&v)[R1], const float2* __res
 }
 
 template <int R1, int R2, int S>
-__global__ void __launch_bounds__(TwoCfg<R1, R2>::cols_threads, TwoCfg<R1, R2>::cols_blocks)
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::cols_threads,
+                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::cols_threads, TwoCfg<R1, R2>::cols_smem))
 two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
     constexpr int W = kTwoW;
-    __shared__ float2 sm[R1 * R2 * W];
+    extern __shared__ __align__(16) unsigned char two_smem[];
+    float2* sm = reinterpret_cast<float2*>(two_smem);             // [position][W]
     const unsigned ntile = (unsigned)(a.Nx + W - 1) / W, outer = a.axis == 1 ? a.Nz : a.Ny;
     const unsigned rest = blockIdx.x / ntile, x0 = (blockIdx.x - rest * ntile) * W;
     const unsigned comp = rest / outer, o = rest - comp * outer;
@@ -110,11 +129,13 @@ two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
 }
 
 template <int R1, int R2, int S>
-__global__ void __launch_bounds__(TwoCfg<R1, R2>::rows_threads, TwoCfg<R1, R2>::rows_blocks)
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::rows_threads,
+                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::rows_threads, TwoCfg<R1, R2>::rows_smem))
 two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
     using Cfg = TwoCfg<R1, R2>;
     constexpr int N = R1 * R2, G = Cfg::G;
-    __shared__ float2 sm[G * Cfg::P];
+    extern __shared__ __align__(16) unsigned char two_smem[];
+    float2* sm = reinterpret_cast<float2*>(two_smem);             // [row][P]
     const long long rows = (long long)a.ncomp * a.Nz * a.Ny, row0 = (long long)blockIdx.x * G;
     const int nrow = (int)min((long long)G, rows - row0);
     float2* base = a.data + row0 * N;
@@ -145,9 +166,10 @@ two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
 }
 
 template <int R1, int R2>
-__global__ void __launch_bounds__(kTwoKThreads, 3)
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::kspace_threads,
+                                  TwoCfg<R1, R2>::kspace_threads == 256 ? 3 : (R1 <= 16 ? 2 : 1))
 two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__ TwoPassModes md) {
-    constexpr int W = kTwoKW, N = R1 * R2, SLOT = N * W, TH = kTwoKThreads;
+    constexpr int W = kTwoKW, N = R1 * R2, SLOT = N * W, TH = TwoCfg<R1, R2>::kspace_threads;
     extern __shared__ __align__(16) unsigned char two_smem[];
     float2* F = reinterpret_cast<float2*>(two_smem);              // [6][position][W]
     const int Nx = a.Nx, Ny = a.Ny, tid = threadIdx.x;
@@ -252,14 +274,21 @@ template <int R1, int R2> TwoPassEntry two_pass_make() {
     e.N = R1 * R2;
     e.R1 = R1;
     e.cols_threads = Cfg::cols_threads;
+    e.cols_smem = Cfg::cols_smem;
     e.rows_threads = Cfg::rows_threads;
     e.rows_per_block = Cfg::G;
-    e.kspace_smem = 6 * R1 * R2 * kTwoKW * (int)sizeof(float2);
-    e.cols[0] = two_cols_kernel<R1, R2, -1>;
-    e.cols[1] = two_cols_kernel<R1, R2, +1>;
+    e.rows_smem = Cfg::rows_smem;
+    if constexpr (Cfg::cols) {
+        e.cols[0] = two_cols_kernel<R1, R2, -1>;
+        e.cols[1] = two_cols_kernel<R1, R2, +1>;
+    }
     e.rows[0] = two_rows_kernel<R1, R2, -1>;
     e.rows[1] = two_rows_kernel<R1, R2, +1>;
-    e.kspace = two_kspace_kernel<R1, R2>;
+    if constexpr (Cfg::kspace) {
+        e.kspace_threads = Cfg::kspace_threads;
+        e.kspace_smem = Cfg::kspace_smem;
+        e.kspace = two_kspace_kernel<R1, R2>;
+    }
     return e;
 }
 #endif
@@ -269,5 +298,9 @@ const TwoPassEntry* two_pass_part0(int N);
 const TwoPassEntry* two_pass_part1(int N);
 const TwoPassEntry* two_pass_part2(int N);
 const TwoPassEntry* two_pass_part3(int N);
+const TwoPassEntry* two_pass_part4(int N);
+const TwoPassEntry* two_pass_part5(int N);
+const TwoPassEntry* two_pass_part6(int N);
+const TwoPassEntry* two_pass_part7(int N);
 
 }  // namespace psatd

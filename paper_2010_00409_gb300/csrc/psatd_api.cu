@@ -572,11 +572,11 @@ psatd_status check_device_error(psatd_ctx* c) {
 }  // namespace
 
 const TwoPassEntry* psatd::two_pass_entry(int N) {
-    const TwoPassEntry* e = two_pass_part0(N);
-    if (!e) e = two_pass_part1(N);
-    if (!e) e = two_pass_part2(N);
-    if (!e) e = two_pass_part3(N);
-    return e;
+    const TwoPassEntry* (*const parts[])(int) = {two_pass_part0, two_pass_part1, two_pass_part2, two_pass_part3,
+                                                 two_pass_part4, two_pass_part5, two_pass_part6, two_pass_part7};
+    for (auto part : parts)
+        if (const TwoPassEntry* e = part(N)) return e;
+    return nullptr;
 }
 
 namespace {
@@ -595,8 +595,15 @@ cudaError_t fft_axis_two(cplx<T>* data, int ncomp, const GridGeom& g, const Tabl
             axis == 0 ? ((long long)ncomp * g.Nz * g.Ny + e->rows_per_block - 1) / e->rows_per_block
                       : (long long)ncomp * (axis == 1 ? g.Nz : g.Ny) * ((g.Nx + 15) / 16);
         if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
-        return launch_pdl(axis == 0 ? e->rows[dir > 0] : e->cols[dir > 0], dim3((unsigned)blocks),
-                          dim3(axis == 0 ? e->rows_threads : e->cols_threads), 0, s, a);
+        auto k = axis == 0 ? e->rows[dir > 0] : e->cols[dir > 0];
+        if (!k) return cudaErrorNotSupported;
+        const int smem = axis == 0 ? e->rows_smem : e->cols_smem;
+        if (smem > 48 * 1024) {
+            const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (r != cudaSuccess) return r;
+        }
+        return launch_pdl(k, dim3((unsigned)blocks), dim3(axis == 0 ? e->rows_threads : e->cols_threads), (size_t)smem, s,
+                          a);
     }
     return cudaErrorNotSupported;
 }
@@ -607,12 +614,12 @@ cudaError_t kspace_two(cplx<T>* data, const GridGeom& g, const Tables<T>& tb, in
     if constexpr (sizeof(T) == 4) {
         const AxisPlan& pl = tb.plan[2];
         const TwoPassEntry* e = two_pass_entry(pl.N);
-        if (!e || pl.npass != 2 || pl.radix[0] != e->R1) return cudaErrorNotSupported;
+        if (!e || !e->kspace || pl.npass != 2 || pl.radix[0] != e->R1) return cudaErrorNotSupported;
         const TwoPassArgs a{data, tb.twp[2], 2, g.Nx, g.Ny, g.Nz, 6};
         const TwoPassModes m{tb.k[0], tb.k[1], tb.k[2], tb.coef, mode, (float)scale};
         const cudaError_t r = cudaFuncSetAttribute(e->kspace, cudaFuncAttributeMaxDynamicSharedMemorySize, e->kspace_smem);
         if (r != cudaSuccess) return r;
-        return launch_pdl(e->kspace, dim3((unsigned)((long long)g.Ny * ((g.Nx + 7) / 8))), dim3(256),
+        return launch_pdl(e->kspace, dim3((unsigned)((long long)g.Ny * ((g.Nx + 7) / 8))), dim3(e->kspace_threads),
                           (size_t)e->kspace_smem, s, a, m);
     }
     return cudaErrorNotSupported;
@@ -738,6 +745,13 @@ cudaError_t spectral_pass(psatd_ctx* c, int mode, double scale) {
             }
         }
         if (c->kernel_path != PSATD_PATH_GENERIC) {
+            cudaError_t r = kspace_two<T>(f, g, tb, mode, scale, c->stream);
+            if (r != cudaErrorNotSupported) {
+                ++c->launches;
+                return r;
+            }
+        }
+        if (c->kernel_path != PSATD_PATH_GENERIC) {
             // a z length with a register plan but no fused kernel (1024 in float32,
             // 512): forward z, the per-mode update, inverse z as three launches
             cudaError_t r = launch_fft_axis_fast<T>(f, 6, g, tb, 2, -1, c->stream);
@@ -747,13 +761,6 @@ cudaError_t spectral_pass(psatd_ctx* c, int mode, double scale) {
                 if ((r = launch_modes<T>(f, g, tb, mode, scale, c->stream)) != cudaSuccess) return r;
                 ++c->launches;
                 r = launch_fft_axis_fast<T>(f, 6, g, tb, 2, +1, c->stream);
-                ++c->launches;
-                return r;
-            }
-        }
-        if (c->kernel_path != PSATD_PATH_GENERIC) {
-            cudaError_t r = kspace_two<T>(f, g, tb, mode, scale, c->stream);
-            if (r != cudaErrorNotSupported) {
                 ++c->launches;
                 return r;
             }

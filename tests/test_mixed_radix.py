@@ -47,10 +47,10 @@ def test_transforms_and_step_match_oracle(lib, shape, prec, tol, path):
 def test_every_compile_time_length_matches_the_run_time_passes(lib):
     """The compile-time kernels of every length against the run-time passes of the
     same plan, along x, y and z (float32, same arithmetic order: 1e-6)."""
-    lengths = [n for n in range(18, 257) if any(n == 2 ** a * 3 ** b * 5 ** c for a in range(9) for b in range(6)
+    lengths = [n for n in range(18, 1025) if any(n == 2 ** a * 3 ** b * 5 ** c for a in range(9) for b in range(6)
                                                 for c in range(4))]
     for n in lengths:
-        for shape in ((n, 3, 4), (18, n, 2), (18, 3, n)):
+        for shape in ((n, 2, 1), (18, n, 1), (18, 1, n)) if n > 256 else ((n, 3, 4), (18, n, 2), (18, 3, n)):
             nx, ny, nz = shape
             g = W.GridSpec(nx, ny, nz, 0.5, 0.7, 0.3, 0.0, 0.0, 0.0, 1.0)
             f = W.random_complex_field((6, nz, ny, nx), seed=n)
