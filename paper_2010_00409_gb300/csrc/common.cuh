@@ -140,14 +140,18 @@ template <typename V> __host__ __device__ __forceinline__ V cmul_si(V a, int s) 
 // the allocation-free energy kernel share it, so their results differ only in
 // the order of the float64 sums.
 template <typename T>
-__device__ __forceinline__ double cell_energy3(cplx<T> a, cplx<T> b, cplx<T> c) {
+__device__ __forceinline__ T cell_energy3_t(cplx<T> a, cplx<T> b, cplx<T> c) {
     T s = a.x * a.x;
     s = fma(a.y, a.y, s);
     s = fma(b.x, b.x, s);
     s = fma(b.y, b.y, s);
     s = fma(c.x, c.x, s);
     s = fma(c.y, c.y, s);
-    return (double)s;
+    return s;
+}
+template <typename T>
+__device__ __forceinline__ double cell_energy3(cplx<T> a, cplx<T> b, cplx<T> c) {
+    return (double)cell_energy3_t<T>(a, b, c);
 }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream

@@ -25,17 +25,30 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return r;
 }
 
-__device__ __forceinline__ double block_max(double v, double* sh) {
+template <typename T>
+__device__ __forceinline__ T block_max(T v, double* sh) {
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    T* s = reinterpret_cast<T*>(sh);
     __syncthreads();
-    if (lane == 0) sh[wid] = v;
+    if (lane == 0) s[wid] = v;
     __syncthreads();
-    double r = 0.0;
+    T r = 0;
     if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmax(r, sh[w]);
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmax(r, s[w]);
     return r;
 }
+
+// Threads of a block over rows of nx values: as many rows at once as fit.
+struct RowThreads {
+    int wide, rows, row, first;
+    __device__ __forceinline__ explicit RowThreads(int nx) {
+        wide = min(nx, (int)blockDim.x);
+        rows = blockDim.x / wide;
+        row = threadIdx.x / wide;
+        first = row < rows ? (int)threadIdx.x - row * wide : nx;       // (spare threads take nothing)
+    }
+};
 
 // partial[b][0] = sum |E|^2, partial[b][1] = sum |B|^2 over this block's cells
 template <typename T>
@@ -63,11 +76,12 @@ divergence_kernel(const cplx<T>* __restrict__ F, GridGeom g, const T* __restrict
     const size_t n = (size_t)g.Nx * g.Ny * g.Nz;
     const int rows = g.Ny * g.Nz;
     T md2 = 0, mf2 = 0;                                // squared maxima
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
+    const RowThreads rt(g.Nx);
+    for (int row = blockIdx.x * rt.rows + rt.row; row < rows; row += gridDim.x * rt.rows) {
         const int iy = row % g.Ny, iz = row / g.Ny;
         const T b = ky[PSATD_IX(iy, g.Ny)], c = kz[PSATD_IX(iz, g.Nz)];
         const size_t base = (size_t)row * g.Nx;
-        for (int ix = threadIdx.x; ix < g.Nx; ix += blockDim.x) {
+        for (int ix = rt.first; ix < g.Nx; ix += rt.wide) {
             const T a = kx[PSATD_IX(ix, g.Nx)];
             const T k2 = a * a + b * b + c * c;
             const size_t i = base + ix;
@@ -76,11 +90,14 @@ divergence_kernel(const cplx<T>* __restrict__ F, GridGeom g, const T* __restrict
             const T dr = a * X.x + b * Y.x + c * Z.x;
             const T di = a * X.y + b * Y.y + c * Z.y;
             if (k2 > T(0)) md2 = max(md2, (dr * dr + di * di) / k2);
-            mf2 = max(mf2, (T)cell_energy3<T>(X, Y, Z));
+            mf2 = max(mf2, cell_energy3_t<T>(X, Y, Z));
         }
     }
-    const double bd = block_max(sqrt((double)md2), sh);
-    const double bf = block_max(sqrt((double)mf2), sh);
+    // the root of the block's maximum is the maximum of the roots: one float64 root a block
+    // (a root, two conversions and float64 comparisons per thread took most of the 20 us
+    // of a 64^3 spectrum)
+    const double bd = sqrt((double)block_max(md2, sh));
+    const double bf = sqrt((double)block_max(mf2, sh));
     const GBuf<double> Pt{partial, 2LL * gridDim.x};
     if (threadIdx.x == 0) { Pt[2 * blockIdx.x] = bd; Pt[2 * blockIdx.x + 1] = bf; }
 }
@@ -116,10 +133,11 @@ divergence_half_kernel(const float2* __restrict__ S, const float2* __restrict__ 
     const int nh = g.Nx / 2, rows = g.Ny * g.Nz;
     const GBuf<const float2> SF{S, 3LL * rows * nh}, QF{Q, 3LL * rows};
     float md2 = 0.f, mf2 = 0.f;
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
+    const RowThreads rt(nh + 1);
+    for (int row = blockIdx.x * rt.rows + rt.row; row < rows; row += gridDim.x * rt.rows) {
         const int iy = row % g.Ny, iz = row / g.Ny;
         const float b = ky[PSATD_IX(iy, g.Ny)], c = kz[PSATD_IX(iz, g.Nz)];
-        for (int p = threadIdx.x; p <= nh; p += blockDim.x) {
+        for (int p = rt.first; p <= nh; p += rt.wide) {
             const float a = p < nh ? kxs[PSATD_IX(p, nh)] : kx_nyq;
             float2 X, Y, Z;
             if (p < nh) {
@@ -132,11 +150,14 @@ divergence_half_kernel(const float2* __restrict__ S, const float2* __restrict__ 
             const float dr = a * X.x + b * Y.x + c * Z.x;
             const float di = a * X.y + b * Y.y + c * Z.y;
             if (k2 > 0.f) md2 = fmaxf(md2, (dr * dr + di * di) / k2);
-            mf2 = fmaxf(mf2, (float)cell_energy3<float>(X, Y, Z));
+            mf2 = fmaxf(mf2, cell_energy3_t<float>(X, Y, Z));
         }
     }
-    const double bd = block_max(sqrt((double)md2), sh);
-    const double bf = block_max(sqrt((double)mf2), sh);
+    // the root of the block's maximum is the maximum of the roots: one float64 root a block
+    // (a root, two conversions and float64 comparisons per thread took most of the 20 us
+    // of a 64^3 spectrum)
+    const double bd = sqrt((double)block_max(md2, sh));
+    const double bf = sqrt((double)block_max(mf2, sh));
     const GBuf<double> Pt{partial, 2LL * gridDim.x};
     if (threadIdx.x == 0) { Pt[2 * blockIdx.x] = bd; Pt[2 * blockIdx.x + 1] = bf; }
 }
