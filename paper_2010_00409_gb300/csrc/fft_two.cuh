@@ -75,6 +75,12 @@ template <int R1, int R2> struct TwoCfg {
     static constexpr int kspace_smem = 6 * N * kTwoKW * (int)sizeof(float2);
     static constexpr bool kspace = kspace_smem <= 226 * 1024;
     static constexpr int kspace_threads = kspace_smem <= 75 * 1024 ? 256 : 512;
+    // Blocks an SM: four of 256 threads (64 registers) to 120 points with radices up to
+    // 12, k-space pass of 192 x 192 x 96 110 -> 102 us, 180 x 150 x 108 86 -> 82 us,
+    // 180 x 180 x 120 127 -> 121 us against three; at 144 points four tiles take all of
+    // the SM's shared memory from its L1 (144^3 101 -> 108 us).
+    static constexpr int kspace_blocks =
+        kspace_threads == 256 ? (R1 <= 12 && N <= 120 ? 4 : 3) : (R1 <= 16 ? 2 : 1);
 };
 
 // multiply v[k] by the position-ordered twiddles W_N^{jk} (conjugated for S > 0)
@@ -166,8 +172,7 @@ two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
 }
 
 template <int R1, int R2>
-__global__ void __launch_bounds__(TwoCfg<R1, R2>::kspace_threads,
-                                  TwoCfg<R1, R2>::kspace_threads == 256 ? 3 : (R1 <= 16 ? 2 : 1))
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::kspace_threads, TwoCfg<R1, R2>::kspace_blocks)
 two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__ TwoPassModes md) {
     constexpr int W = kTwoKW, N = R1 * R2, SLOT = N * W, TH = TwoCfg<R1, R2>::kspace_threads;
     extern __shared__ __align__(16) unsigned char two_smem[];
