@@ -251,6 +251,7 @@ template <typename T> struct MultiProblem {
     int N[3];
     int W[3];
     int nsteps;                 // this box's steps (the launch runs the largest count)
+    int two[3];                 // compile-time tile of the axis (fft_two.cuh), -1: run-time passes
     AxisPlan plan[3];
 };
 

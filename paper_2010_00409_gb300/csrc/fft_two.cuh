@@ -30,6 +30,26 @@
 
 namespace psatd {
 
+// The lengths of two radices up to 16 (index, R1, R2), for the batched advance's tiles.
+#define PSATD_TWO_PAIRS(X) \
+    X(0, 6, 3) X(1, 5, 4) X(2, 6, 4) X(3, 5, 5) X(4, 9, 3) X(5, 6, 5) X(6, 8, 4) X(7, 6, 6) X(8, 8, 5) \
+    X(9, 9, 5) X(10, 8, 6) X(11, 10, 5) X(12, 9, 6) X(13, 10, 6) X(14, 8, 8) X(15, 9, 8) X(16, 15, 5) \
+    X(17, 10, 8) X(18, 9, 9) X(19, 10, 9) X(20, 12, 8) X(21, 10, 10) X(22, 12, 9) X(23, 12, 10) X(24, 16, 8) \
+    X(25, 15, 9) X(26, 12, 12) X(27, 15, 10) X(28, 16, 10) X(29, 15, 12) X(30, 16, 12) X(31, 15, 15) \
+    X(32, 16, 15) X(33, 16, 16)
+
+// The index of a plan's pair in that list, or -1.
+inline int two_pair_index(const AxisPlan& pl) {
+    if (pl.npass != 2) return -1;
+#define PSATD_TWO_CASE(i, r1, r2) \
+    if (pl.radix[0] == r1 && pl.radix[1] == r2) return i;
+    PSATD_TWO_PAIRS(PSATD_TWO_CASE)
+#undef PSATD_TWO_CASE
+    return -1;
+}
+// Rows a block of 256 threads takes at once along x.
+inline int two_rows_per_tile(const AxisPlan& pl) { return 256 / pl.radix[0]; }
+
 struct TwoPassArgs {
     float2* data;
     const float2* tp;                       // position-ordered twiddles, W_N^{jk} at k R2 + j
@@ -93,32 +113,26 @@ __device__ __forceinline__ void two_twiddle(float2 (&v)[R1], const float2* __res
     });
 }
 
-template <int R1, int R2, int S>
-__global__ void __launch_bounds__(TwoCfg<R1, R2>::cols_threads,
-                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::cols_threads, TwoCfg<R1, R2>::cols_smem))
-two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
+// CG: loads of the field go around L1 (values other SMs wrote during this launch).
+template <bool CG> __device__ __forceinline__ float2 two_load(const GBuf<float2>& F, const float2* p, size_t i) {
+    if constexpr (CG) return __ldcg(&F.at(p, i));
+    else return F.at(p, i);
+}
+
+// One column tile: lane c of kTwoW on column base (its pointer), t = 0 .. R1 - 1.
+template <int R1, int R2, int S, bool CG>
+__device__ __forceinline__ void two_cols_tile(float2* base, size_t stride, int t, int c, bool col,
+                                              const float2* __restrict__ tp, float2* sm, const GBuf<float2>& F) {
     constexpr int W = kTwoW;
-    extern __shared__ __align__(16) unsigned char two_smem[];
-    float2* sm = reinterpret_cast<float2*>(two_smem);             // [position][W]
-    const unsigned ntile = (unsigned)(a.Nx + W - 1) / W, outer = a.axis == 1 ? a.Nz : a.Ny;
-    const unsigned rest = blockIdx.x / ntile, x0 = (blockIdx.x - rest * ntile) * W;
-    const unsigned comp = rest / outer, o = rest - comp * outer;
-    const size_t plane = (size_t)a.Nx * a.Ny, stride = a.axis == 1 ? (size_t)a.Nx : plane;
-    const unsigned c = threadIdx.x % W, t = threadIdx.x / W;
-    float2* base = a.data + comp * plane * a.Nz + (a.axis == 1 ? o * plane : (size_t)o * a.Nx) + x0 + c;
-    const GBuf<float2> F{a.data, (long long)a.ncomp * plane * a.Nz};
-    const bool col = x0 + c < (unsigned)a.Nx;
-    pdl_launch_dependents();
-    pdl_wait();
     if (col && t < R2) {
         float2 v[R1];
         const float2* p = base + t * stride;
         static_for<0, R1>([&](auto rc) {
-            v[decltype(rc)::value] = F.at(p, 0);
+            v[decltype(rc)::value] = two_load<CG>(F, p, 0);
             p += R2 * stride;
         });
         reg_dft<float, S, R1>(v);
-        two_twiddle<S, R1, R2>(v, a.tp, t);
+        two_twiddle<S, R1, R2>(v, tp, t);
         static_for<0, R1>([&](auto rc) { sm[(decltype(rc)::value * R2 + t) * W + c] = v[decltype(rc)::value]; });
     }
     __syncthreads();
@@ -134,28 +148,20 @@ two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
     }
 }
 
-template <int R1, int R2, int S>
-__global__ void __launch_bounds__(TwoCfg<R1, R2>::rows_threads,
-                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::rows_threads, TwoCfg<R1, R2>::rows_smem))
-two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
+// nrow <= TwoCfg::G consecutive rows at base.
+template <int R1, int R2, int S, bool CG>
+__device__ __forceinline__ void two_rows_tile(float2* base, int nrow, const float2* __restrict__ tp, float2* sm,
+                                              const GBuf<float2>& F) {
     using Cfg = TwoCfg<R1, R2>;
-    constexpr int N = R1 * R2, G = Cfg::G;
-    extern __shared__ __align__(16) unsigned char two_smem[];
-    float2* sm = reinterpret_cast<float2*>(two_smem);             // [row][P]
-    const long long rows = (long long)a.ncomp * a.Nz * a.Ny, row0 = (long long)blockIdx.x * G;
-    const int nrow = (int)min((long long)G, rows - row0);
-    float2* base = a.data + row0 * N;
-    const GBuf<float2> F{a.data, rows * N};
+    constexpr int N = R1 * R2;
     const int tid = threadIdx.x;
-    pdl_launch_dependents();
-    pdl_wait();
     if (tid < nrow * R2) {
         const int w = tid / R2, j = tid - w * R2;
         const float2* p = base + w * N + j;
         float2 v[R1];
-        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = F.at(p, decltype(rc)::value * R2); });
+        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = two_load<CG>(F, p, decltype(rc)::value * R2); });
         reg_dft<float, S, R1>(v);
-        two_twiddle<S, R1, R2>(v, a.tp, j);
+        two_twiddle<S, R1, R2>(v, tp, j);
         float2* s = sm + w * Cfg::P + j;
         static_for<0, R1>([&](auto rc) { s[decltype(rc)::value * Cfg::run] = v[decltype(rc)::value]; });
     }
@@ -169,6 +175,106 @@ two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
         float2* p = base + w * N + u;
         static_for<0, R2>([&](auto rc) { F.at(p, decltype(rc)::value * R1) = v[decltype(rc)::value]; });
     }
+}
+
+// z passes of a k-space tile (six components of kTwoKW columns, [6][position][kTwoKW] in
+// sm, nw of them in the field).  The forward one ends with a barrier.
+template <int R1, int R2, int TH, bool CG>
+__device__ __forceinline__ void two_z_forward(const float2* base, size_t plane, size_t cstride, int nw,
+                                              const float2* __restrict__ tp, float2* sm, const GBuf<float2>& F) {
+    constexpr int W = kTwoKW, SLOT = R1 * R2 * W;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 6 * R2 * W; i += TH) {
+        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
+        if (c >= nw) continue;
+        const float2* p = base + q * cstride + j * plane + c;
+        float2 v[R1];
+        static_for<0, R1>([&](auto rc) {
+            v[decltype(rc)::value] = two_load<CG>(F, p, 0);
+            p += R2 * plane;
+        });
+        reg_dft<float, -1, R1>(v);
+        two_twiddle<-1, R1, R2>(v, tp, j);
+        float2* s = sm + q * SLOT + j * W + c;
+        static_for<0, R1>([&](auto rc) { s[decltype(rc)::value * R2 * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 6 * R1 * W; i += TH) {
+        const int c = i % W, u = i / W;                           // u = q R1 + k1: runs of R2 positions
+        if (c >= nw) continue;
+        float2* s = sm + u * (R2 * W) + c;
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
+        reg_dft<float, -1, R2>(v);
+        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+}
+
+template <int R1, int R2, int TH>
+__device__ __forceinline__ void two_z_inverse(float2* base, size_t plane, size_t cstride, int nw,
+                                              const float2* __restrict__ tp, float2* sm, const GBuf<float2>& F) {
+    constexpr int W = kTwoKW, SLOT = R1 * R2 * W;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 6 * R1 * W; i += TH) {
+        const int c = i % W, u = i / W;
+        if (c >= nw) continue;
+        float2* s = sm + u * (R2 * W) + c;
+        float2 v[R2];
+        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
+        reg_dft<float, +1, R2>(v);
+        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 6 * R2 * W; i += TH) {
+        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
+        if (c >= nw) continue;
+        const float2* s = sm + q * SLOT + j * W + c;
+        float2 v[R1];
+        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * R2 * W]; });
+        two_twiddle<+1, R1, R2>(v, tp, j);
+        reg_dft<float, +1, R1>(v);
+        float2* p = base + q * cstride + j * plane + c;
+        static_for<0, R1>([&](auto rc) {
+            F.at(p, 0) = v[decltype(rc)::value];
+            p += R2 * plane;
+        });
+    }
+}
+
+template <int R1, int R2, int S>
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::cols_threads,
+                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::cols_threads, TwoCfg<R1, R2>::cols_smem))
+two_cols_kernel(const __grid_constant__ TwoPassArgs a) {
+    constexpr int W = kTwoW;
+    extern __shared__ __align__(16) unsigned char two_smem[];
+    float2* sm = reinterpret_cast<float2*>(two_smem);             // [position][W]
+    const unsigned ntile = (unsigned)(a.Nx + W - 1) / W, outer = a.axis == 1 ? a.Nz : a.Ny;
+    const unsigned rest = blockIdx.x / ntile, x0 = (blockIdx.x - rest * ntile) * W;
+    const unsigned comp = rest / outer, o = rest - comp * outer;
+    const size_t plane = (size_t)a.Nx * a.Ny, stride = a.axis == 1 ? (size_t)a.Nx : plane;
+    const unsigned c = threadIdx.x % W, t = threadIdx.x / W;
+    float2* base = a.data + comp * plane * a.Nz + (a.axis == 1 ? o * plane : (size_t)o * a.Nx) + x0 + c;
+    const GBuf<float2> F{a.data, (long long)a.ncomp * plane * a.Nz};
+    pdl_launch_dependents();
+    pdl_wait();
+    two_cols_tile<R1, R2, S, false>(base, stride, (int)t, (int)c, x0 + c < (unsigned)a.Nx, a.tp, sm, F);
+}
+
+template <int R1, int R2, int S>
+__global__ void __launch_bounds__(TwoCfg<R1, R2>::rows_threads,
+                                  TwoCfg<R1, R2>::blocks(TwoCfg<R1, R2>::rows_threads, TwoCfg<R1, R2>::rows_smem))
+two_rows_kernel(const __grid_constant__ TwoPassArgs a) {
+    constexpr int N = R1 * R2, G = TwoCfg<R1, R2>::G;
+    extern __shared__ __align__(16) unsigned char two_smem[];
+    const long long rows = (long long)a.ncomp * a.Nz * a.Ny, row0 = (long long)blockIdx.x * G;
+    const int nrow = (int)min((long long)G, rows - row0);
+    pdl_launch_dependents();
+    pdl_wait();
+    two_rows_tile<R1, R2, S, false>(a.data + row0 * N, nrow, a.tp, reinterpret_cast<float2*>(two_smem),
+                                    GBuf<float2>{a.data, rows * N});
 }
 
 template <int R1, int R2>
@@ -186,35 +292,7 @@ two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__
     const int nw = min(W, Nx - x0);
     pdl_launch_dependents();
     pdl_wait();
-
-    // forward: level 0 from the field, level 1 in place
-#pragma unroll 1
-    for (int i = tid; i < 6 * R2 * W; i += TH) {
-        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
-        if (c >= nw) continue;
-        const float2* p = base + q * cstride + j * plane + c;
-        float2 v[R1];
-        static_for<0, R1>([&](auto rc) {
-            v[decltype(rc)::value] = G.at(p, 0);
-            p += R2 * plane;
-        });
-        reg_dft<float, -1, R1>(v);
-        two_twiddle<-1, R1, R2>(v, a.tp, j);
-        float2* s = F + q * SLOT + j * W + c;
-        static_for<0, R1>([&](auto rc) { s[decltype(rc)::value * R2 * W] = v[decltype(rc)::value]; });
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int i = tid; i < 6 * R1 * W; i += TH) {
-        const int c = i % W, u = i / W;                           // u = q R1 + k1: runs of R2 positions
-        if (c >= nw) continue;
-        float2* s = F + u * (R2 * W) + c;
-        float2 v[R2];
-        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
-        reg_dft<float, -1, R2>(v);
-        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
-    }
-    __syncthreads();
+    two_z_forward<R1, R2, TH, false>(base, plane, cstride, nw, a.tp, F, G);
 
     // the update of every mode: position k1 R2 + k2 holds k_z = k1 + R1 k2
     const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1, ay = min(y, Ny - y);
@@ -244,33 +322,7 @@ two_kspace_kernel(const __grid_constant__ TwoPassArgs a, const __grid_constant__
     if (spectral) return;
     __syncthreads();
 
-    // inverse: the levels backwards, level 0 to the field
-#pragma unroll 1
-    for (int i = tid; i < 6 * R1 * W; i += TH) {
-        const int c = i % W, u = i / W;
-        if (c >= nw) continue;
-        float2* s = F + u * (R2 * W) + c;
-        float2 v[R2];
-        static_for<0, R2>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * W]; });
-        reg_dft<float, +1, R2>(v);
-        static_for<0, R2>([&](auto rc) { s[decltype(rc)::value * W] = v[decltype(rc)::value]; });
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int i = tid; i < 6 * R2 * W; i += TH) {
-        const int c = i % W, u = i / W, q = u / R2, j = u - q * R2;
-        if (c >= nw) continue;
-        const float2* s = F + q * SLOT + j * W + c;
-        float2 v[R1];
-        static_for<0, R1>([&](auto rc) { v[decltype(rc)::value] = s[decltype(rc)::value * R2 * W]; });
-        two_twiddle<+1, R1, R2>(v, a.tp, j);
-        reg_dft<float, +1, R1>(v);
-        float2* p = base + q * cstride + j * plane + c;
-        static_for<0, R1>([&](auto rc) {
-            G.at(p, 0) = v[decltype(rc)::value];
-            p += R2 * plane;
-        });
-    }
+    two_z_inverse<R1, R2, TH>(base, plane, cstride, nw, a.tp, F, G);
 }
 
 template <int R1, int R2> TwoPassEntry two_pass_make() {

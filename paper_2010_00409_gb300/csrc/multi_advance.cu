@@ -11,14 +11,19 @@
 // launch runs n steps, i.e. 5 n - 1 barriers, without returning to the host;
 // a box with fewer steps of its own skips its items in the later steps.
 //
-// Work items (the in-place mixed-radix passes of fft_mixed.cuh with radices up to
-// 16, so any axis length with factors 2, 3, 5 works):
+// Work items:
 //   x: W_x consecutive rows of one box (contiguous in memory);
 //   y: W_y consecutive x-columns at one (component, z);
 //   z: W_z consecutive x-columns at one y, all six components: forward z
 //      transforms, the update of every mode of the tile, inverse z transforms.
-// The radix schedule of each axis and the three tile widths come from the host
-// (the batch autotuner picks them per axis length).
+// Any axis length with factors 2, 3, 5 runs the in-place passes of fft_mixed.cuh with
+// radices up to 16; the radix schedule of each axis and the three tile widths come
+// from the host (the batch autotuner picks them per axis length).  In float32 a length
+// of two such radices, at the untuned tile widths, runs the compile-time tiles of
+// fft_two.cuh instead (MultiProblem::two), which leave out the run-time index
+// arithmetic: 16 sweep boxes of 96 to 192 points an axis, two to three steps, 11.2 ms
+// with the run-time passes, 9.45 ms with these (five sweeps of the boxes at the
+// copy bandwidth take 5.6 ms).
 //
 // The barrier: every block adds one to a global counter after a fence, and
 // thread 0 polls the counter (acquire loads, a short sleep between polls) until
@@ -29,6 +34,7 @@
 // forever.  Field loads go around L1 (cache-global) so that no block reads a
 // line another block rewrote in the previous phase.
 #include "fft_mixed.cuh"
+#include "fft_two.cuh"
 #include "tma.cuh"
 
 namespace psatd {
@@ -161,6 +167,81 @@ __device__ __forceinline__ void z_tile(const MultiProblem<T>& P, long long item,
     mix_inverse<T, kNarrow>(t, sm, P.plan[2], P.tp[2]);
 }
 
+// ---------------------------------------------------------------------------
+// float32 lengths of two radices up to 16: the compile-time tiles of fft_two.cuh,
+// each a function of its own, with the tile at its fixed place in shared memory.  As
+// calls they keep the kernel at 80 registers without spills (three blocks an SM) and
+// cost a jump an item, which is 2 us of work or more.
+__device__ __forceinline__ float2* multi_tile() {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    return reinterpret_cast<float2*>(smem_raw + desc_bytes<float>());
+}
+
+template <int R1, int R2, int S>
+__device__ __noinline__ void x_two(const MultiProblem<float>& P, int item) {
+    constexpr int G = TwoCfg<R1, R2>::G;
+    const long long rows = 6LL * P.N[1] * P.N[2], row0 = (long long)item * G;
+    two_rows_tile<R1, R2, S, true>(P.f + row0 * (R1 * R2), (int)min((long long)G, rows - row0), P.tp[0], multi_tile(),
+                                   GBuf<float2>{P.f, rows * (R1 * R2)});
+}
+
+template <int R1, int R2, int S>
+__device__ __noinline__ void y_two(const MultiProblem<float>& P, int item) {
+    const int Nx = P.N[0], ntile = (Nx + kTwoW - 1) / kTwoW;
+    const unsigned rest = (unsigned)item / (unsigned)ntile;                    // comp * Nz + z
+    const int x0 = ((int)((unsigned)item - rest * ntile)) * kTwoW, c = threadIdx.x % kTwoW, t = threadIdx.x / kTwoW;
+    const long long plane = (long long)Nx * (R1 * R2);
+    two_cols_tile<R1, R2, S, true>(P.f + rest * plane + x0 + c, (size_t)Nx, t, c, x0 + c < Nx, P.tp[1], multi_tile(),
+                                   GBuf<float2>{P.f, 6LL * plane * P.N[2]});
+}
+
+template <int R1, int R2>
+__device__ __noinline__ void z_two(const MultiProblem<float>& P, int item) {
+    constexpr int W = kTwoKW, N = R1 * R2, SLOT = N * W;
+    float2* sm = multi_tile();
+    const int Nx = P.N[0], Ny = P.N[1], ntile = (Nx + W - 1) / W;
+    const int y = (int)((unsigned)item / (unsigned)ntile), x0 = (item - y * ntile) * W, nw = min(W, Nx - x0);
+    const size_t plane = (size_t)Nx * Ny, cstride = plane * N;
+    float2* base = P.f + (size_t)y * Nx + x0;
+    const GBuf<float2> F{P.f, 6LL * (long long)cstride};
+    two_z_forward<R1, R2, kMT, true>(base, plane, cstride, nw, P.tp[2], sm, F);
+    const int Nxh = Nx / 2 + 1, Nyh = Ny / 2 + 1, ay = min(y, Ny - y);
+    const float ky = P.k[1][PSATD_IX(y, Ny)];
+    const long long ncoef = (long long)(N / 2 + 1) * Nyh * Nxh;
+#pragma unroll 1
+    for (int e = threadIdx.x; e < SLOT; e += kMT) {
+        const int c = e % W, pos = e / W, k1 = pos / R2, n = k1 + (pos - k1 * R2) * R1;
+        if (c >= nw) continue;
+        const int ix = x0 + c, ax = min(ix, Nx - ix), az = min(n, N - n);
+        const ModeCoef<float> m = P.coef[PSATD_IX(((size_t)az * Nyh + ay) * Nxh + ax, ncoef)];
+        float2* o = sm + e;
+        float2 Ex = o[0], Ey = o[SLOT], Ez = o[2 * SLOT], Bx = o[3 * SLOT], By = o[4 * SLOT], Bz = o[5 * SLOT];
+        rotate_mode<float>(Ex, Ey, Ez, Bx, By, Bz, P.k[0][PSATD_IX(ix, Nx)] * m.kinv, ky * m.kinv,
+                           P.k[2][PSATD_IX(n, N)] * m.kinv, m.C, m.S);
+        o[0] = Ex; o[SLOT] = Ey; o[2 * SLOT] = Ez;
+        o[3 * SLOT] = Bx; o[4 * SLOT] = By; o[5 * SLOT] = Bz;
+    }
+    __syncthreads();
+    two_z_inverse<R1, R2, kMT>(base, plane, cstride, nw, P.tp[2], sm, F);
+}
+
+// Phase ph of the item with the compile-time tile `id`.
+__device__ __forceinline__ void two_phase(int ph, int id, const MultiProblem<float>& P, int item) {
+    switch (id) {
+#define PSATD_TWO_CASE(i, r1, r2)                            \
+    case i:                                                  \
+        if (ph == 0) x_two<r1, r2, -1>(P, item);             \
+        else if (ph == 1) y_two<r1, r2, -1>(P, item);        \
+        else if (ph == 2) z_two<r1, r2>(P, item);            \
+        else if (ph == 3) y_two<r1, r2, +1>(P, item);        \
+        else x_two<r1, r2, +1>(P, item);                     \
+        break;
+        PSATD_TWO_PAIRS(PSATD_TWO_CASE)
+#undef PSATD_TWO_CASE
+        default: break;
+    }
+}
+
 // float32: three blocks per SM (85 registers a thread, tiles of at most 72 KB)
 template <typename T>
 __global__ void __launch_bounds__(kMT, sizeof(T) == 4 ? 3 : 2)
@@ -206,7 +287,14 @@ multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long*
                     __syncthreads();
                 }
                 const long long item = g - pre[lo];
-                if (s < P->nsteps) {                            // a box past its own step count is skipped
+                bool done = s >= P->nsteps;                     // a box past its own step count is skipped
+                if constexpr (sizeof(T) == 4) {
+                    if (!done && P->two[a] >= 0) {
+                        two_phase(ph, P->two[a], *P, (int)item);
+                        done = true;
+                    }
+                }
+                if (!done) {
                     if (ph == 0) x_tile<T, -1>(*P, item, tile);
                     else if (ph == 1) y_tile<T, -1>(*P, item, tile);
                     else if (ph == 2) z_tile<T>(*P, item, tile);

@@ -78,3 +78,29 @@ def test_three_pass_columns_and_row_fused_steps_match_oracle(lib, shape):
         got = ctx.get_field(-1)
     ref = O.advance(f, O.Grid(nx, ny, nz, g.dx, g.dy, g.dz, 0.0, 0.0, 0.0, 1.0), 0.3, 1)
     assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def test_batched_compile_time_tiles_match_the_run_time_passes(lib):
+    """One batched launch over boxes with every length of two radices up to 16 along
+    x, y and z (remainders of all three tiles) against the run-time passes of a
+    context each (float32, same arithmetic order: 1e-6)."""
+    lengths = [n for n in range(18, 257) if any(n == 2 ** a * 3 ** b * 5 ** c for a in range(9) for b in range(6)
+                                               for c in range(4))]
+    ctxs, want = [], []
+    for n in lengths:
+        for shape in ((n, 3, 5), (18, n, 2), (20 if n % 2 else 10, 3, n)):
+            nx, ny, nz = shape
+            g = W.GridSpec(nx, ny, nz, 0.5, 0.7, 0.3, 0.0, 0.0, 0.0, 1.0)
+            f = W.random_complex_field((6, nz, ny, nx), seed=n)
+            with lib.Context(g, None, 0.3, 32) as ctx:
+                ctx.set_kernel_path(lib.PATH_GENERIC)
+                ctx.set_fields(f)
+                ctx.advance(1)
+                want.append(ctx.get_field(-1))
+            ctxs.append(lib.Context(g, None, 0.3, 32))
+            ctxs[-1].set_fields(f)
+    lib.multi_advance(ctxs, 1)
+    for ctx, w in zip(ctxs, want):
+        got = ctx.get_field(-1)
+        assert np.linalg.norm(got - w) <= 1e-6 * np.linalg.norm(w), w.shape
+        ctx.close()
