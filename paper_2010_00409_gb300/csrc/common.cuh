@@ -179,6 +179,17 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
     return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// Host: let launches of k use up to LIMIT bytes of dynamic shared memory.  The limit
+// belongs to the kernel for the whole process, so a kernel whose tile varies from call
+// to call always gets the same one, its largest: with each call's own size, a context
+// stepped on another host thread could lower it between this call's set and its launch,
+// and the launch was refused.
+template <int LIMIT, typename K>
+cudaError_t allow_smem(K k) {
+    static_assert(LIMIT <= 227 * 1024, "an SM's limit for one block");
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LIMIT);
+}
+
 // ---------------------------------------------------------------------------
 // 1D plan of one axis: N = prod(radix[0..npass)), radices up to 16 (narrow plans)
 // or 32 out of those fft_mixed.cuh has a register DFT for; N = 1 is one radix 1
@@ -259,6 +270,13 @@ template <typename T> struct MultiProblem {
 // W pencils): the pencils of one component for x and y, of six for the fused z
 // pass.
 template <typename T> size_t multi_tile_bytes(int axis, const AxisPlan& pl, int W);
+
+// Shared-memory budget of one tile: three blocks of 256 threads per SM in float32
+// (80 registers a thread), two in float64 (more registers).  Every length the batched
+// advance takes has a tile within it.
+template <typename T> constexpr size_t multi_tile_budget() {
+    return sizeof(T) == 4 ? (size_t)(72 * 1024) : (size_t)(100 * 1024);
+}
 
 // Persistent cooperative launch advancing nprob boxes by up to nsteps PSATD
 // steps (box p by its own probs[p].nsteps <= nsteps).

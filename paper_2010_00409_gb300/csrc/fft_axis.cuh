@@ -19,6 +19,7 @@ namespace psatd {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kTileCap = 64 * 1024;
 
 // narrow plans (radices to 16): three blocks of 256 threads per SM in float32
 template <typename T, int MAXR> constexpr int axis_min_blocks() {
@@ -113,7 +114,7 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
     int W, maxr = 0, logw = 0;
     size_t smem;
     // a tile of 64 KB leaves three blocks on an SM
-    mix_tile_shape<T>(axis, pl, g.Nx, tb.tile_shift, 64 * 1024, &W, &smem);
+    mix_tile_shape<T>(axis, pl, g.Nx, tb.tile_shift, kTileCap, &W, &smem);
     while ((1 << logw) < W) ++logw;
     for (int p = 0; p < pl.npass; ++p) maxr = max(maxr, pl.radix[p]);
     const long long nblocks = axis == 0 ? ((long long)ncomp * g.Nz * g.Ny + W - 1) / W
@@ -126,7 +127,7 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
     const int threads = (int)(items >= kThreads ? kThreads : (items + 31) / 32 * 32);
     auto launch = [&](auto sc, auto mc, auto rc) {
         auto k = fft_axis_kernel<T, decltype(sc)::value, decltype(mc)::value, decltype(rc)::value>;
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem<kTileCap>(k);
         if (e != cudaSuccess) return e;
         if (nlaunch) ++*nlaunch;
         return launch_pdl(k, dim3((unsigned)nblocks), dim3(threads), smem, s, data, axis, g.Nx, g.Ny, g.Nz, ncomp, W,

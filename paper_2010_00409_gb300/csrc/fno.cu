@@ -673,10 +673,10 @@ namespace {
 
 // Launches of the mixing kernels: shared memory for the staged spectra (sets, four
 // bytes a value) and, backward through the input, as many weight rows as fit.
-template <typename K>
+// A launch asks for up to LIMIT bytes.
+template <int LIMIT, typename K>
 cudaError_t mix_smem(K k, size_t bytes) {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-                             : cudaSuccess;
+    return bytes > 48 * 1024 ? allow_smem<LIMIT>(k) : cudaSuccess;
 }
 int mix_threads(int n) { return std::min(256, std::max(32, (n + 31) / 32 * 32)); }
 
@@ -689,7 +689,7 @@ cudaError_t mix_fwd(psatd_fno* f, const float* V, const float* R, float* U, int 
     const int per_block = std::max(1, 256 / items);
     const size_t need = (size_t)2 * per_block * B * f->C * sizeof(float);
     const int stage = need <= (size_t)kMixStage;
-    const cudaError_t e = mix_smem(mix_fwd_kernel, stage ? need : 0);
+    const cudaError_t e = mix_smem<kMixStage>(mix_fwd_kernel, stage ? need : 0);
     if (e != cudaSuccess) return e;
     mix_fwd_kernel<<<(f->MODES + per_block - 1) / per_block, mix_threads(per_block * items), stage ? need : 0,
                      f->stream>>>(V, R, U, f->MODES, B, f->C, per_block, stage);
@@ -700,7 +700,7 @@ cudaError_t mix_back(psatd_fno* f, const float* gU, const float* V, const float*
     const int C = f->C;
     const size_t spec = (size_t)2 * B * C * sizeof(float);
     int stage = 2 * spec <= (size_t)kMixStage;
-    cudaError_t e = mix_smem(mix_back_weight_kernel, stage ? 2 * spec : 0);
+    cudaError_t e = mix_smem<kMixStage>(mix_back_weight_kernel, stage ? 2 * spec : 0);
     if (e != cudaSuccess) return e;
     mix_back_weight_kernel<<<f->MODES, mix_threads((C + 3) / 4 * C), stage ? 2 * spec : 0, f->stream>>>(
         gU, V, gR, f->MODES, B, C, stage);
@@ -708,7 +708,7 @@ cudaError_t mix_back(psatd_fno* f, const float* gU, const float* V, const float*
     const size_t row = (size_t)2 * (C + 1) * sizeof(float);
     const int rows = (int)std::min<size_t>(C, kMixStage / row);
     const size_t bytes = (stage ? spec : 0) + rows * row;
-    if ((e = mix_smem(mix_back_input_kernel, bytes)) != cudaSuccess) return e;
+    if ((e = mix_smem<2 * kMixStage>(mix_back_input_kernel, bytes)) != cudaSuccess) return e;
     mix_back_input_kernel<<<f->MODES, mix_threads((B + 3) / 4 * rows), bytes, f->stream>>>(gU, R, gV, f->MODES, B, C,
                                                                                          rows, stage);
     return cudaGetLastError();

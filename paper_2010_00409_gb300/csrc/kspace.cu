@@ -25,6 +25,7 @@ namespace psatd {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kTileMax = 227 * 1024;
 
 template <typename T, int MAXR>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? (MAXR <= kNarrow ? 3 : 2) : 1)
@@ -137,7 +138,7 @@ cudaError_t launch_kspace_z(cplx<T>* data, const GridGeom& g, const Tables<T>& t
     if (tb.tile_shift < 0) W = max(1, W >> -tb.tile_shift);
     while (W > 1 && bytes(W) > (es == 8 ? 112 : 100) * 1024) W /= 2;
     const size_t smem = bytes(W);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (smem > kTileMax) return cudaErrorInvalidValue;
     int logw = 0, maxr = 0;
     while ((1 << logw) < W) ++logw;
     for (int p = 0; p < pl.npass; ++p) maxr = max(maxr, pl.radix[p]);
@@ -146,7 +147,7 @@ cudaError_t launch_kspace_z(cplx<T>* data, const GridGeom& g, const Tables<T>& t
     const int threads = (int)(items >= kThreads ? kThreads : (items + 31) / 32 * 32);
     auto launch = [&](auto mc) {
         auto k = kspace_z_kernel<T, decltype(mc)::value>;
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem<kTileMax>(k);
         if (e != cudaSuccess) return e;
         if (nlaunch) ++*nlaunch;
         return launch_pdl(k, dim3((unsigned)nblocks), dim3(threads), smem, s, data, g.Nx, g.Ny, g.Nz, W, logw, pl,

@@ -328,7 +328,7 @@ cudaError_t launch_multi_advance(const MultiProblem<T>* probs, const long long* 
                                  unsigned long long limit_ns, unsigned extra, cudaStream_t s, int* grid_out) {
     auto k = multi_advance_kernel<T>;
     const size_t smem = desc_bytes<T>() + tile_bytes;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem<(int)(desc_bytes<T>() + multi_tile_budget<T>())>(k);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

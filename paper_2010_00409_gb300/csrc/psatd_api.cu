@@ -887,11 +887,6 @@ bool same_plan(const AxisPlan& a, const AxisPlan& b) {
     return true;
 }
 
-// Shared-memory budget of one tile: three blocks of 256 threads per SM in float32
-// (85 registers a thread), two in float64 (more registers).
-template <typename T> constexpr size_t multi_tile_budget() {
-    return sizeof(T) == 4 ? (size_t)(72 * 1024) : (size_t)(100 * 1024);
-}
 constexpr size_t kMultiHeader = 256;              // barrier counter at the start of the batch buffer
 constexpr int kMultiMaxN = 1024;
 constexpr unsigned long long kMultiWaitNs = 2000000000ull;   // 2 s per barrier wait
