@@ -2,6 +2,8 @@
 // per-axis FFT plan, and the launch interfaces of the kernel translation units.
 #pragma once
 
+#include <atomic>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -189,6 +191,21 @@ cudaError_t allow_smem(K k) {
     static_assert(LIMIT <= 227 * 1024, "an SM's limit for one block");
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LIMIT);
 }
+
+// Host: a kernel's one-time settings, made once on each device it is launched on (a
+// device has its own copy of a kernel and of its attributes).  A failed setup is tried
+// again; two threads that meet here both make the same settings.
+struct PerDevice {
+    std::atomic<unsigned long long> done{0};
+    template <typename F>
+    cudaError_t once(int dev, F setup) {
+        const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+        if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+        const cudaError_t e = setup();
+        if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+};
 
 // ---------------------------------------------------------------------------
 // 1D plan of one axis: N = prod(radix[0..npass)), radices up to 16 (narrow plans)

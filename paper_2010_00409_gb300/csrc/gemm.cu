@@ -8,6 +8,8 @@
 // tensor memory).  Split-K (ksplit > 1) partitions K over tiles and adds partial
 // tiles to C with float atomics (C must hold beta * C beforehand; the launcher
 // scales it).
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -549,18 +551,18 @@ cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
     if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     auto k = gemm_tc_kernel<BN, DUAL, EPI>;
     // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        sms = n < 1 ? 1 : n;
-    }
-    const long long cap = (long long)sms * Cfg::kBlocks;
+    static PerDevice set;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    e = set.once(dev, [&] {
+        const cudaError_t r = allow_smem<Cfg::kSmem>(k);
+        return r != cudaSuccess ? r : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                           cudaSharedmemCarveoutMaxShared);
+    });
+    if (e != cudaSuccess) return e;
+    const long long cap = (long long)std::max(sms, 1) * Cfg::kBlocks;
     k<<<(unsigned)(ntiles < cap ? ntiles : cap), kTcThreads, Cfg::kSmem, s>>>(g, (int)ntm, (int)ntn, (int)ntiles);
     return cudaGetLastError();
 }
@@ -642,18 +644,13 @@ cudaError_t launch_gemm_tma(const void* A, const void* B, float* C, int M, int N
         return cudaErrorInvalidValue;
     CUtensorMap ma, mb;
     if (!gemm_map(&ma, A, M, K, GT_BM) || !gemm_map(&mb, B, N, K, GT_BN)) return cudaErrorInvalidValue;
-    static int sms = 0;
-    static bool attr = false;
-    if (!attr) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms < 1) sms = 1;
-        const cudaError_t e = cudaFuncSetAttribute(gemm_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   GT_SMEM);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice set;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = set.once(dev, [] { return allow_smem<GT_SMEM>(gemm_tma_kernel); })) != cudaSuccess) return e;
+    if (sms < 1) sms = 1;
     const int ntm = M / GT_BM, ntn = N / GT_BN;
     const long long ntiles = (long long)ntm * ntn;
     const int grid = (int)(ntiles < sms ? ntiles : sms);
