@@ -63,16 +63,52 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // ------------------------------------------------------------ reductions
-// Sums over voxels run in double-float (ff.cuh) per thread and in float64 from the
-// block's partial sum on: a float64 sum of every element is bound by the float64
-// pipe (1/64 of the float32 rate) and took 2.1 ms for 67 M gradients, one block a
-// channel.  Rows are cut into kRowChunks pieces so that every SM takes part.
+// Sums over voxels run in three float32 parts up to a warp's sum (72 bits: no less than
+// the 53 of a float64 sum of every element, which is bound by the float64 pipe, 1/64 of
+// the float32 rate, and took 2.1 ms for 67 M gradients, one block a channel) and in
+// float64 from there on.  Rows are cut into kRowChunks pieces so that every SM takes part.
 constexpr int kRowChunks = 32;
 
-// Block sum of one double-float per thread; thread 0 returns it.
-__device__ __forceinline__ double block_sum_ff(FF s) {
+// SumK with K = 3 of Ogita, Rump and Oishi, "Accurate sum and dot product", 2005: a
+// takes the values, b the exact rounding errors of a, c those of b.
+struct Sum3 {
+    float a, b, c;
+};
+__device__ __forceinline__ void sum3_add(Sum3& s, float x) {
+    const FF t = two_sum(s.a, x), u = two_sum(s.b, t.l);
+    s.a = t.h;
+    s.b = u.h;
+    s.c += u.l;
+}
+
+// s, t -> the sum of both
+__device__ __forceinline__ Sum3 sum3_merge(const Sum3& s, const Sum3& t) {
+    const FF a = two_sum(s.a, t.a), b = two_sum(s.b, t.b), d = two_sum(b.h, a.l);
+    return {a.h, d.h, (s.c + t.c) + (b.l + d.l)};
+}
+
+// Block sum of one Sum3 per thread (256 threads); thread 0 returns it.
+__device__ __forceinline__ double block_sum(Sum3 s) {
+    __shared__ Sum3 sh[8];
+    for (int o = 16; o > 0; o >>= 1)
+        s = sum3_merge(s, Sum3{__shfl_down_sync(0xffffffffu, s.a, o), __shfl_down_sync(0xffffffffu, s.b, o),
+                               __shfl_down_sync(0xffffffffu, s.c, o)});
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < 32) {
+        if (threadIdx.x < 8) {
+            const Sum3 t = sh[threadIdx.x];
+            v = (double)t.a + ((double)t.b + (double)t.c);
+        }
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    }
+    return v;
+}
+
+// Block sum of one float64 value per thread; thread 0 returns it.
+__device__ __forceinline__ double block_sum(double v) {
     __shared__ double sh[32];
-    double v = (double)s.h + (double)s.l;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -94,7 +130,7 @@ act_back_kernel(const float* __restrict__ z, const float* ga, float* gz, int B, 
     const long long lo = chunk * per, hi = min(n4, lo + per), off = (long long)row * n4;
     const float4 *z4 = reinterpret_cast<const float4*>(z) + off, *g4 = reinterpret_cast<const float4*>(ga) + off;
     float4* o4 = reinterpret_cast<float4*>(gz) + off;
-    FF s{0.f, 0.f};
+    Sum3 s{0.f, 0.f, 0.f};
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
         float4 g = g4[i];
         if constexpr (GELU) {
@@ -102,10 +138,23 @@ act_back_kernel(const float* __restrict__ z, const float* ga, float* gz, int B, 
             g = make_float4(g.x * gelu_grad(v.x), g.y * gelu_grad(v.y), g.z * gelu_grad(v.z), g.w * gelu_grad(v.w));
             o4[i] = g;
         }
-        const FF p = two_sum(g.x, g.y), q = two_sum(g.z, g.w);
-        s = ff_add(s, ff_add(p, q));
+        sum3_add(s, g.x);
+        sum3_add(s, g.y);
+        sum3_add(s, g.z);
+        sum3_add(s, g.w);
     }
-    const double t = block_sum_ff(s);
+    double t;
+    if (__syncthreads_or(!isfinite(s.a + s.b + s.c))) {
+        // an infinity, a NaN or an overflow, after which the errors are NaN: in float64
+        double v = 0.0;
+        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+            const float4 g = GELU ? o4[i] : g4[i];
+            v += ((double)g.x + (double)g.y) + ((double)g.z + (double)g.w);
+        }
+        t = block_sum(v);
+    } else {
+        t = block_sum(s);
+    }
     if (threadIdx.x == 0) partial[(long long)c * B * kRowChunks + b * kRowChunks + chunk] = t;
 }
 
