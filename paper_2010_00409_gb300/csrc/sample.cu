@@ -11,7 +11,8 @@
 //     phi = 2 pi s / (N d)   (w = 1 at phi = 0; w is N d-periodic in s).
 // The three contractions (x, then y, then z) run in float64 for float64
 // storage and in double-float arithmetic (ff.cuh: float32 pairs, ~48 bits) for
-// float32 storage, whose inputs are float32: the same sums to ~1e-14 without
+// float32 storage, whose inputs are float32: the same sums (to about 1e-14 of the sum
+// of the magnitudes over 2048 points, less over fewer) without
 // float64 instructions, which GB300 issues at 1/64 of the float32 rate.  The
 // weights and the partial sums g, h then live in the scratch buffers as float4
 // {re.h, re.l, im.h, im.l} (the size of a double2).
@@ -241,7 +242,7 @@ __global__ void contract_z_kernel(const double2* __restrict__ h, GridGeom g, She
 // float32 storage: the same three contractions in double-float arithmetic
 // (weights, g and h as float4 double-float complex values; the sums are the
 // compensated ones of ff.cuh's Dot2).  All three are bound by the float32 pipe
-// (11 or 12 instructions per real product), so each is laid out to keep every
+// (12 or 13 instructions per real product), so each is laid out to keep every
 // SM's pipe busy: 8 lanes a row instead of a warp a row along x (3 instead of 5
 // rounds of the cross-lane sum), and register tiles with the sum split over the
 // warps of a block along y and z.
@@ -301,19 +302,26 @@ contract_x_ff_kernel(const float* __restrict__ f, GridGeom g, CompList cl, int n
     }
     const GBuf<const float2> F{f2, 6LL * per_comp * n2};
     Dot2C acc[kXRows] = {};
-#pragma unroll 4
-    for (int i = lane; i < n2; i += kXL) {
+    auto mac = [&](int i) {
 #pragma unroll
         for (int r = 0; r < kXRows; ++r) {
             const float2 v = F.at(p[r], i);
             if constexpr (REAL) {
-                dot2_mac_real(acc[r], sw[2 * i], v.x);
-                dot2_mac_real(acc[r], sw[2 * i + 1], v.y);
+                dot2_mac_real(acc[r], sw[2 * i], sw[2 * i + 1], v);
             } else {
                 dot2_mac(acc[r], sw[i], v);
             }
         }
+    };
+    int i = lane;
+#pragma unroll 2
+    for (; i + kXL < n2; i += 2 * kXL) {
+        mac(i);
+        mac(i + kXL);
+#pragma unroll
+        for (int r = 0; r < kXRows; ++r) dot2_norm(acc[r]);
     }
+    if (i < n2) mac(i);
 #pragma unroll
     for (int r = 0; r < kXRows; ++r) {
         const CFF t = group_sum(dot2_value(acc[r]));
@@ -357,11 +365,19 @@ contract_x_half_ff_kernel(const float2* __restrict__ S, const float2* __restrict
     Dot2C A{}, Am{};
     if (have) {
         // slot 0 holds x mode 0: its term belongs to Z
-#pragma unroll 4
-        for (int p = lane ? lane : kXL; p < nh; p += kXL) {
+        auto mac = [&](int p) {
             dot2_mac(A, sw[p], SF.at(pa, p));
             dot2_mac(Am, sw[p], SF.at(pm, p));
+        };
+        int p = lane ? lane : kXL;
+#pragma unroll 2
+        for (; p + kXL < nh; p += 2 * kXL) {
+            mac(p);
+            mac(p + kXL);
+            dot2_norm(A);
+            dot2_norm(Am);
         }
+        if (p < nh) mac(p);
     }
     const CFF sa = group_sum(dot2_value(A)), sm = group_sum(dot2_value(Am));
     if (have && lane < 2) {                                   // lane 0 writes the row, lane 1 its mirror
@@ -382,7 +398,7 @@ contract_x_half_ff_kernel(const float2* __restrict__ S, const float2* __restrict
 // of 64 threads, whose sums are added in a fixed order at the end: without the
 // split the smallest planes leave a warp or two per SM.  R = 2 when it still gives
 // every SM two tiles, else R = 1 (four times the tiles; the float32 pipe stays the
-// bound, 48 instructions per product against two shared loads).  Operands come in chunks of 32 k
+// bound, 51 instructions per product against two shared loads).  Operands come in chunks of 32 k
 // through shared memory, the next chunk loaded while one is multiplied; rows are
 // 33 float4 apart, so the eight rows a quarter-warp reads lie on distinct banks.
 //   y: m = (a, l), k = j, n = p:  A = g, B[k][n] = wy[n][k];
@@ -434,16 +450,21 @@ contract_yz_ff_kernel(const float4* __restrict__ A, const float4* __restrict__ B
         }
         __syncthreads();
         if (k0 + kCK < K) fetch(k0 + kCK);
-#pragma unroll 2
-        for (int k = grp; k < kCK; k += kCS) {
-            float4 av[R], bv[R];
+#pragma unroll 1
+        for (int kb = grp; kb < kCK; kb += 2 * kCS) {
 #pragma unroll
-            for (int i = 0; i < R; ++i) {
-                av[i] = sA[(ty + 8 * i) * kCRow + k];
-                bv[i] = sB[(tx + 8 * i) * kCRow + k];
+            for (int k = kb; k < kb + 2 * kCS; k += kCS) {
+                float4 av[R], bv[R];
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    av[i] = sA[(ty + 8 * i) * kCRow + k];
+                    bv[i] = sB[(tx + 8 * i) * kCRow + k];
+                }
+#pragma unroll
+                for (int i = 0; i < R * R; ++i) dot2_mac_cff(acc[i / R][i % R], av[i / R], bv[i % R]);
             }
 #pragma unroll
-            for (int i = 0; i < R * R; ++i) dot2_mac_cff(acc[i / R][i % R], av[i / R], bv[i % R]);
+            for (int i = 0; i < R * R; ++i) dot2_norm(acc[i / R][i % R]);
         }
     }
     if (grp > 0) {
