@@ -94,6 +94,20 @@ bool make_plan(int N, AxisPlan* p, int max_radix) {
     return p->npass > 0;
 }
 
+// The plan of a context's axis: radices beyond 16 only where they save a pass;
+// float64 stops at 20 (a register DFT of more points would not fit the register file).
+// In float32 two radices up to 16 are never joined into one of 18 to 32 points: one
+// pass has an item a pencil, half a warp in a 16-column block, and the two
+// compile-time passes of fft_two.cuh are faster for all seven such lengths in the mean
+// (a step of 32^3 points 50.4 -> 12.7 us, 24^3 30.4 -> 11.2 us, 240 x 250 x 25 220 ->
+// 155 us, 20 x 240 x 250 185 -> 138 us; the other way 1000 x 27 x 90 334 -> 341 us).
+bool context_plan(int N, int precision, AxisPlan* p) {
+    AxisPlan wide;
+    if (!make_plan(N, p) || !make_plan(N, &wide, precision == 64 ? 20 : 32)) return false;
+    if (wide.npass < p->npass && !(precision == 32 && p->npass == 2)) *p = wide;
+    return true;
+}
+
 }  // namespace psatd
 
 namespace {
@@ -1110,14 +1124,7 @@ psatd_status psatd_init_grid(const psatd_grid* grid, const psatd_mapping* mappin
     c->prec = precision;
     c->real_fields = real;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
-    // radices beyond 16 only where they save a pass; float64 stops at 20 (a register
-    // DFT of more points would not fit the register file)
-    for (int a = 0; a < 3; ++a) {
-        AxisPlan wide;
-        make_plan(Ns[a], &c->plan[a]);
-        make_plan(Ns[a], &wide, precision == 64 ? 20 : 32);
-        if (wide.npass < c->plan[a].npass) c->plan[a] = wide;
-    }
+    for (int a = 0; a < 3; ++a) context_plan(Ns[a], precision, &c->plan[a]);
 
     cudaError_t e = cudaGetDevice(&c->device);
     psatd_status st = PSATD_OK;
