@@ -207,6 +207,17 @@ struct PerDevice {
     }
 };
 
+// Host: the number of SMs of device dev, asked for once (0.7 us a query).
+inline cudaError_t sm_count(int dev, int* n) {
+    static std::atomic<int> known[64];
+    const bool keep = dev >= 0 && dev < 64;
+    *n = keep ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (*n > 0) return cudaSuccess;
+    const cudaError_t e = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && keep) known[dev].store(*n, std::memory_order_relaxed);
+    return e;
+}
+
 // ---------------------------------------------------------------------------
 // 1D plan of one axis: N = prod(radix[0..npass)), radices up to 16 (narrow plans)
 // or 32 out of those fft_mixed.cuh has a register DFT for; N = 1 is one radix 1

@@ -555,7 +555,7 @@ cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = sm_count(dev, &sms)) != cudaSuccess) return e;
     e = set.once(dev, [&] {
         const cudaError_t r = allow_smem<Cfg::kSmem>(k);
         return r != cudaSuccess ? r : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -648,7 +648,7 @@ cudaError_t launch_gemm_tma(const void* A, const void* B, float* C, int M, int N
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = sm_count(dev, &sms)) != cudaSuccess) return e;
     if ((e = set.once(dev, [] { return allow_smem<GT_SMEM>(gemm_tma_kernel); })) != cudaSuccess) return e;
     if (sms < 1) sms = 1;
     const int ntm = M / GT_BM, ntn = N / GT_BN;

@@ -44,3 +44,9 @@ def test_gemm_launchers_remember_no_device_but_the_one_they_set():
     src = open(os.path.join(CSRC, "gemm.cu")).read()
     assert "static int sms" not in src and "static bool attr" not in src
     assert src.count("static PerDevice set;") == 2
+
+
+def test_sm_counts_come_from_the_cache():
+    """A launch asks the driver for nothing but the current device."""
+    src = open(os.path.join(CSRC, "gemm.cu")).read()
+    assert "cudaDeviceGetAttribute" not in src and src.count("sm_count(dev, &sms)") == 2
