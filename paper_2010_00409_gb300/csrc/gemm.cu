@@ -46,7 +46,7 @@ namespace {
 // refilled) and, after a tile's last K block, to the accumulator's mbarrier
 // (the tile may be read).  All waits are bounded; an expired wait sets
 // g_gemm_error (gemm_take_error reads and clears it).
-constexpr int TBM = 128, TBK = 64, kTcThreads = 256;
+constexpr int TBM = 128, TBK = 64, kTcThreads = 256, kTcLoneThreads = 512;
 __device__ int g_gemm_error;
 
 __device__ __forceinline__ uint32_t tc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -117,15 +117,15 @@ __device__ __forceinline__ TcTile tc_tile(const GemmArgs& g, int tile, int ntm, 
 // (then 8 consecutive k from a multiple of 8 are two aligned float4 loads)
 // Only the first kcs 8-column chunks are staged (the MMAs of a short last K
 // block read no further).
-template <int ROWS> constexpr int tc_items() { return (ROWS * (TBK / 8) + kTcThreads - 1) / kTcThreads; }
+template <int ROWS, int TH> constexpr int tc_items() { return (ROWS * (TBK / 8) + TH - 1) / TH; }
 
 // Row r and chunk kc of a thread's n-th item.  Contiguous k (vec): a warp takes 8 rows
 // x 4 chunks, 128 contiguous bytes of each row, and its 8-lane groups store 8 rows of
 // one chunk, one core matrix (conflict-free); with 32 rows a warp, each load touched
 // 32 lines.  Otherwise 32 rows of one chunk (contiguous where the rows are).
-template <int ROWS>
+template <int ROWS, int TH>
 __device__ __forceinline__ bool tc_item(int n, bool vec, int kcs, int& r, int& kc) {
-    const int i = threadIdx.x + n * kTcThreads;
+    const int i = threadIdx.x + n * TH;
     if (vec) {
         const int w = i >> 5, lane = i & 31;
         r = (w % (ROWS / 8)) * 8 + (lane & 7);
@@ -137,13 +137,13 @@ __device__ __forceinline__ bool tc_item(int n, bool vec, int kcs, int& r, int& k
     return kc < kcs;
 }
 
-template <int ROWS>
+template <int ROWS, int TH>
 __device__ __forceinline__ void tc_stage(unsigned char* dst, const float* __restrict__ src, long long s_r,
                                          long long s_k, int r0, int nrows, int k0, int kend, bool vec, int kcs) {
 #pragma unroll
-    for (int n = 0; n < tc_items<ROWS>(); ++n) {
+    for (int n = 0; n < tc_items<ROWS, TH>(); ++n) {
         int r, kc;
-        if (!tc_item<ROWS>(n, vec, kcs, r, kc)) continue;
+        if (!tc_item<ROWS, TH>(n, vec, kcs, r, kc)) continue;
         const int gr = r0 + r, gk = k0 + kc * 8;
         float v[8];
         if (vec && gr < nrows && gk + 8 <= kend) {
@@ -180,14 +180,14 @@ __device__ __forceinline__ float tc_gelu(float x) { return 0.5f * x * (1.f + erf
 enum TcEpi { EPI_PLAIN = 0, EPI_ACT = 1, EPI_SPLIT = 2 };
 
 // Epilogue.  Warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the rows of its
-// lane quarter); the two warps of one quarter split the columns, read in loads of 8.
+// lane quarter); the warps of one quarter split the columns, read in loads of 8.
 // With a bias or an activation the result passes through them here: as a pass of its
 // own over the field (read, write back, write the activation) they took 235 us a layer
 // at 8 x 32 x 64^3 values, 0.2 ms of an inference.  The forms are compiled apart: one
 // epilogue with all of them in it slowed the plain one by 15 to 60 %.
-template <int BN, bool DUAL, int EPI>
+template <int BN, bool DUAL, int EPI, int TH>
 __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, uint32_t acc_addr, bool have) {
-    constexpr int parts = kTcThreads / 128, cols = BN / parts;
+    constexpr int parts = TH / 128, cols = BN / parts;
     static_assert(cols % 8 == 0, "column split");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quarter = warp & 3;
@@ -256,8 +256,9 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& g, const TcTile& t, 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
 
-template <int BN, bool DUAL, int EPI>
-__global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
+template <int BN, bool DUAL, int EPI, int TH>
+__global__ void __launch_bounds__(TH, TH == kTcThreads ? TcCfg<BN, DUAL>::kBlocks : 1)
+gemm_tc_kernel(GemmArgs g, int ntm, int ntn, int ntiles) {
     using Cfg = TcCfg<BN, DUAL>;
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     __shared__ uint32_t tmem_base;
@@ -300,8 +301,8 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_
             unsigned char* Bs = As + Cfg::kStageA;
             const int k0 = t.kbeg + kb * TBK;
             const int nkk = min(TBK / 16, (t.kend - k0 + 15) / 16);         // K = 16 MMAs with data
-            tc_stage<TBM>(As, (second ? g.A2 : g.A) + t.offA, g.sAm, g.sAk, t.m0, g.M, k0, t.kend, vecA, 2 * nkk);
-            tc_stage<BN>(Bs, (second ? g.B2 : g.B) + t.offB, g.sBn, g.sBk, t.n0, g.N, k0, t.kend, vecB, 2 * nkk);
+            tc_stage<TBM, TH>(As, (second ? g.A2 : g.A) + t.offA, g.sAm, g.sAk, t.m0, g.M, k0, t.kend, vecA, 2 * nkk);
+            tc_stage<BN, TH>(Bs, (second ? g.B2 : g.B) + t.offB, g.sBn, g.sBk, t.n0, g.N, k0, t.kend, vecB, 2 * nkk);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> tensor-core reads
             // (every thread has also read the previous tile's accumulator by now)
             __syncthreads();
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<BN, DUAL>::kBlocks) gemm_tc_
         if (tid == 0) tc_commit(&abar);
         ok = tc_wait(&abar, tl & 1) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tc_epilogue<BN, DUAL, EPI>(g, t, acc, t.nkb > 0);
+        tc_epilogue<BN, DUAL, EPI, TH>(g, t, acc, t.nkb > 0);
     }
     if (!ok) {
         if (tid == 0) atomicExch(&g_gemm_error, 1);
@@ -543,28 +544,43 @@ __global__ void scale_kernel(GemmArgs g) {
 }  // namespace
 
 namespace {
-template <int BN, bool DUAL, int EPI>
-cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
+template <int BN, bool DUAL, int EPI, int TH>
+cudaError_t gemm_tc_run(const GemmArgs& g, int ntm, int ntn, int ntiles, int dev, int sms, cudaStream_t s) {
     using Cfg = TcCfg<BN, DUAL>;
-    const long long ntm = (g.M + TBM - 1) / TBM, ntn = (g.N + BN - 1) / BN;
-    const long long ntiles = ntm * ntn * (long long)g.nb0 * g.nb1 * g.ksplit;
-    if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    auto k = gemm_tc_kernel<BN, DUAL, EPI>;
-    // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
+    auto k = gemm_tc_kernel<BN, DUAL, EPI, TH>;
     static PerDevice set;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if ((e = sm_count(dev, &sms)) != cudaSuccess) return e;
-    e = set.once(dev, [&] {
+    const cudaError_t e = set.once(dev, [&] {
         const cudaError_t r = allow_smem<Cfg::kSmem>(k);
         return r != cudaSuccess ? r : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                            cudaSharedmemCarveoutMaxShared);
     });
     if (e != cudaSuccess) return e;
-    const long long cap = (long long)std::max(sms, 1) * Cfg::kBlocks;
-    k<<<(unsigned)(ntiles < cap ? ntiles : cap), kTcThreads, Cfg::kSmem, s>>>(g, (int)ntm, (int)ntn, (int)ntiles);
+    // persistent over the tiles, the blocks per SM that fit (TcCfg::kBlocks)
+    const long long cap = (long long)sms * (TH == kTcThreads ? Cfg::kBlocks : 1);
+    k<<<(unsigned)(ntiles < cap ? ntiles : cap), TH, Cfg::kSmem, s>>>(g, ntm, ntn, ntiles);
     return cudaGetLastError();
+}
+
+template <int BN, bool DUAL, int EPI>
+cudaError_t gemm_tc_launch(const GemmArgs& g, cudaStream_t s) {
+    const long long ntm = (g.M + TBM - 1) / TBM, ntn = (g.N + BN - 1) / BN;
+    const long long ntiles = ntm * ntn * (long long)g.nb0 * g.nb1 * g.ksplit;
+    if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = sm_count(dev, &sms)) != cudaSuccess) return e;
+    sms = std::max(sms, 1);
+    // No more tiles than SMs: a block has its SM to itself and the loads of one K block
+    // are all that is in flight there, so 512 threads issue them.
+    // 1024 x 1024 x 16384 1380 -> 790 us, 37 x 4100 x 16384 1034 -> 596 us, 256 x 256 x
+    // 128 13.3 -> 10.2 us against 256 threads (one block of 512 with two accumulators,
+    // the form before those: 905, 716 and 12.4 us).  With a second block per SM, 256
+    // threads each have as much in flight, and their chains overlap.
+    if constexpr (!DUAL && EPI == EPI_PLAIN)
+        if (ntiles <= sms)
+            return gemm_tc_run<BN, DUAL, EPI, kTcLoneThreads>(g, (int)ntm, (int)ntn, (int)ntiles, dev, sms, s);
+    return gemm_tc_run<BN, DUAL, EPI, kTcThreads>(g, (int)ntm, (int)ntn, (int)ntiles, dev, sms, s);
 }
 }  // namespace
 
