@@ -26,7 +26,7 @@ template <typename T, int MAXR> constexpr int axis_min_blocks() {
     return sizeof(T) == 4 ? (MAXR <= kNarrow ? 3 : 2) : (MAXR <= kNarrow ? 2 : 1);
 }
 
-template <typename T, int S, int MAXR, bool ROWS>
+template <typename T, int S, int MAXR, bool ROWS, bool PAD>
 __global__ void __launch_bounds__(kThreads, axis_min_blocks<T, MAXR>())
 fft_axis_kernel(cplx<T>* __restrict__ data, int axis, int Nx, int Ny, int Nz, int ncomp, int W, int logw,
                 const __grid_constant__ AxisPlan pl, const cplx<T>* __restrict__ tp) {
@@ -44,9 +44,10 @@ fft_axis_kernel(cplx<T>* __restrict__ data, int axis, int Nx, int Ny, int Nz, in
         t.base = data + row0 * Nx;
         t.stride = 1;
         t.nw = (int)min((long long)W, rows - row0);
-        t.P = row_stride(Nx, pl.radix[0]);
-        t.run = row_run(Nx, pl.radix[0]);
-        t.gap = t.run - Nx / pl.radix[0];
+        const int n = Nx / pl.radix[0];                                 // values of a run
+        t.run = PAD ? row_run_padded(pl) : row_run(Nx, pl.radix[0]);
+        t.P = pl.radix[0] * t.run | 1;
+        t.gap = t.run - n - (PAD ? n / pl.radix[2] : 0);
     } else {
         const unsigned ntile = (unsigned)(Nx + W - 1) >> logw, outer = axis == 1 ? Nz : Ny;
         const unsigned rest = blockIdx.x / ntile, tile = blockIdx.x - rest * ntile;
@@ -58,7 +59,7 @@ fft_axis_kernel(cplx<T>* __restrict__ data, int axis, int Nx, int Ny, int Nz, in
     }
     pdl_launch_dependents();
     pdl_wait();
-    mix_transform<T, S, MAXR, ROWS, false>(t, sm, pl, tp);
+    mix_transform<T, S, MAXR, ROWS, false, PAD>(t, sm, pl, tp);
 }
 
 }  // namespace
@@ -80,7 +81,8 @@ inline double lane_share(const AxisPlan& pl, int Nx, int W) {
 template <typename T>
 void mix_tile_shape(int axis, const AxisPlan& pl, int Nx, int shift, size_t cap, int* W, size_t* bytes) {
     const int es = (int)sizeof(cplx<T>), N = pl.N;
-    const size_t per = (size_t)(axis == 0 ? row_stride(N, pl.radix[0]) : N) * es;
+    const int row = sizeof(T) == 4 && row_padded(pl) ? pl.radix[0] * row_run_padded(pl) | 1 : row_stride(N, pl.radix[0]);
+    const size_t per = (size_t)(axis == 0 ? row : N) * es;
     int w;
     if (axis == 0) {
         w = max(1, min(128, 256 * pl.radix[0] / N));
@@ -125,8 +127,8 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
     for (int p = 0; p < pl.npass; ++p) minr = min(minr, pl.radix[p]);
     const long long items = (long long)W * (pl.N / minr);
     const int threads = (int)(items >= kThreads ? kThreads : (items + 31) / 32 * 32);
-    auto launch = [&](auto sc, auto mc, auto rc) {
-        auto k = fft_axis_kernel<T, decltype(sc)::value, decltype(mc)::value, decltype(rc)::value>;
+    auto launch = [&](auto sc, auto mc, auto rc, auto pc) {
+        auto k = fft_axis_kernel<T, decltype(sc)::value, decltype(mc)::value, decltype(rc)::value, decltype(pc)::value>;
         const cudaError_t e = allow_smem<kTileCap>(k);
         if (e != cudaSuccess) return e;
         if (nlaunch) ++*nlaunch;
@@ -134,7 +136,11 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
                           logw, pl, tb.twp[axis]);
     };
     auto by_rows = [&](auto sc, auto mc) {
-        return axis == 0 ? launch(sc, mc, std::true_type{}) : launch(sc, mc, std::false_type{});
+        if constexpr (sizeof(T) == 4)
+            if (axis == 0 && row_padded(pl))
+                return launch(sc, std::integral_constant<int, kNarrow>{}, std::true_type{}, std::true_type{});
+        return axis == 0 ? launch(sc, mc, std::true_type{}, std::false_type{})
+                         : launch(sc, mc, std::false_type{}, std::false_type{});
     };
     auto by_radix = [&](auto sc) {
         return maxr <= kNarrow ? by_rows(sc, std::integral_constant<int, kNarrow>{})

@@ -50,6 +50,19 @@ __host__ __device__ __forceinline__ unsigned div_multiplier(int d) {
 // Rows: the spacing of the first level's runs, and a row's values in all.
 __host__ __device__ __forceinline__ int row_run(int N, int R0) { return (N / R0) | 1; }
 __host__ __device__ __forceinline__ int row_stride(int N, int R0) { return R0 * row_run(N, R0) | 1; }
+// Padded rows (PAD below): float32 plans of three levels, radices to 16, the last a multiple of 8.
+// The last pass's lanes read that many consecutive values each, so an even spacing puts
+// half a warp on one or two banks (2048 = 16 x 16 x 8: eight ways); a spare value behind
+// each such block spreads them, and runs R values apart mod 16 line the middle pass's
+// blocks of R lanes up behind each other.  2048 x 64 x 64 step 1208 -> 1092 us, 1536 x
+// 64 x 64 812 -> 776 us.  In float64, bound by its pipe, it changes nothing.
+__host__ __device__ __forceinline__ bool row_padded(const AxisPlan& pl) {
+    return pl.npass == 3 && pl.radix[0] <= kNarrow && pl.radix[2] % 8 == 0;
+}
+__host__ __device__ __forceinline__ int row_run_padded(const AxisPlan& pl) {
+    const int R = pl.radix[2], n = pl.N / pl.radix[0], run = n + n / R;
+    return run + ((R - run) & 15);
+}
 
 // Position-ordered twiddle entries of a plan (all levels but the last, whose
 // twiddles are 1).
@@ -104,7 +117,8 @@ template <typename T> struct MixTile {
 // level).  DIT (the levels backwards): operands from shared memory, to_g stores to
 // global memory (first level).  CG: global loads go around L1 (values other SMs
 // wrote during this launch).
-template <typename T, int S, int R, bool ROWS, bool DIT, bool CG>
+// PAD (rows): the padded layout of row_run_padded.
+template <typename T, int S, int R, bool ROWS, bool DIT, bool CG, bool PAD>
 __device__ __forceinline__ void mix_pass(const MixTile<T>& t, cplx<T>* sm, const AxisPlan& pl, int p, int M,
                                          const cplx<T>* __restrict__ tp, bool from_g, bool to_g) {
     const int N = pl.N, nb = N / R, L = M / R;                  // (divisions by a compile-time R)
@@ -133,11 +147,13 @@ __device__ __forceinline__ void mix_pass(const MixTile<T>& t, cplx<T>* sm, const
             // first level: value r in run r; deeper levels lie inside one run
             if (p == 0) {
                 s0 = sm + c * t.P + j;
+                if constexpr (PAD) s0 += fdiv(j, pl.div_l[1]);          // (the last radix is the second level's L)
                 ss = t.run;
             } else {
                 const int run0 = fdiv(pos0, pl.div_run);
                 s0 = sm + c * t.P + pos0 + run0 * t.gap;
-                ss = L;
+                if constexpr (PAD) s0 += p == 1 ? blk * R : blk;        // last-level blocks before pos0
+                ss = PAD && p == 1 ? L + 1 : L;
             }
         } else {
             s0 = sm + q * t.slot + (pos0 << t.logw) + c;
@@ -198,12 +214,12 @@ __device__ __forceinline__ void mix_pass(const MixTile<T>& t, cplx<T>* sm, const
     }
 }
 
-template <typename T, int S, int MAXR, bool ROWS, bool DIT, bool CG>
+template <typename T, int S, int MAXR, bool ROWS, bool DIT, bool CG, bool PAD = false>
 __device__ __forceinline__ void mix_dispatch(const MixTile<T>& t, cplx<T>* sm, const AxisPlan& pl, int p, int M,
                                              const cplx<T>* tp, bool from_g, bool to_g) {
     const int R = pl.radix[p];
 #define PSATD_MIX(r) \
-    case r: mix_pass<T, S, r, ROWS, DIT, CG>(t, sm, pl, p, M, tp, from_g, to_g); return
+    case r: mix_pass<T, S, r, ROWS, DIT, CG, PAD>(t, sm, pl, p, M, tp, from_g, to_g); return
     switch (R) {
         PSATD_MIX(1); PSATD_MIX(2); PSATD_MIX(3); PSATD_MIX(4); PSATD_MIX(5); PSATD_MIX(6); PSATD_MIX(8);
         PSATD_MIX(9); PSATD_MIX(10); PSATD_MIX(12); PSATD_MIX(15); PSATD_MIX(16);
@@ -221,14 +237,14 @@ __device__ __forceinline__ void mix_dispatch(const MixTile<T>& t, cplx<T>* sm, c
 
 // The whole transform of a tile from global to global memory.  Called by the whole
 // block; ends without a barrier (the last pass reads shared memory).
-template <typename T, int S, int MAXR, bool ROWS, bool CG>
+template <typename T, int S, int MAXR, bool ROWS, bool CG, bool PAD = false>
 __device__ __forceinline__ void mix_transform(const MixTile<T>& t, cplx<T>* sm, const AxisPlan& pl,
                                               const cplx<T>* tp) {
     int M = pl.N;
 #pragma unroll 1
     for (int p = 0; p < pl.npass; ++p) {
         if (p > 0) __syncthreads();
-        mix_dispatch<T, S, MAXR, ROWS, false, CG>(t, sm, pl, p, M, tp, p == 0, p == pl.npass - 1);
+        mix_dispatch<T, S, MAXR, ROWS, false, CG, PAD>(t, sm, pl, p, M, tp, p == 0, p == pl.npass - 1);
         tp += M;
         M /= pl.radix[p];
     }
