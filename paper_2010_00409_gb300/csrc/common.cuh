@@ -237,8 +237,8 @@ struct AxisPlan {
 // smallest largest radix), largest first.  Returns false if N has a prime factor
 // other than 2, 3 and 5.
 bool make_plan(int N, AxisPlan* p, int max_radix = 16);
-// Host: the plan of a context's axis of N points (precision 32 or 64).
-bool context_plan(int N, int precision, AxisPlan* p);
+// Host: the plan of a context's axis (0 x, 1 y, 2 z) of N points (precision 32 or 64).
+bool context_plan(int N, int precision, int axis, AxisPlan* p);
 // Set a plan's division multipliers from its radices.
 void finish_plan(AxisPlan* p);
 

@@ -94,17 +94,22 @@ bool make_plan(int N, AxisPlan* p, int max_radix) {
     return p->npass > 0;
 }
 
-// The plan of a context's axis: radices beyond 16 only where they save a pass;
-// float64 stops at 20 (a register DFT of more points would not fit the register file).
+// The plan of a context's axis (0 x, 1 y, 2 z): radices beyond 16 only where they save
+// a pass.  In float64 a wide kernel takes all the registers of an SM for one block, so
+// along x and y three narrow passes beat two wide ones (step of 64 x 360 x 64 2.67 ->
+// 2.39 ms, 360 x 64 x 64 2.61 -> 2.39 ms, 2000 x 64 x 64 16.4 -> 15.3 ms); along z, where
+// a pass fewer is a trip of six components through shared memory and back, radices to
+// 20 stay where they make two passes (64 x 64 x 162: 6 % faster so).
 // In float32 two radices up to 16 are never joined into one of 18 to 32 points: one
 // pass has an item a pencil, half a warp in a 16-column block, and the two
 // compile-time passes of fft_two.cuh are faster for all seven such lengths in the mean
 // (a step of 32^3 points 50.4 -> 12.7 us, 24^3 30.4 -> 11.2 us, 240 x 250 x 25 220 ->
 // 155 us, 20 x 240 x 250 185 -> 138 us; the other way 1000 x 27 x 90 334 -> 341 us).
-bool context_plan(int N, int precision, AxisPlan* p) {
+bool context_plan(int N, int precision, int axis, AxisPlan* p) {
     AxisPlan wide;
     if (!make_plan(N, p) || !make_plan(N, &wide, precision == 64 ? 20 : 32)) return false;
-    if (wide.npass < p->npass && !(precision == 32 && p->npass == 2)) *p = wide;
+    const bool take = precision == 64 ? axis == 2 && wide.npass == 2 : p->npass > 2;
+    if (take && wide.npass < p->npass) *p = wide;
     return true;
 }
 
@@ -1124,7 +1129,7 @@ psatd_status psatd_init_grid(const psatd_grid* grid, const psatd_mapping* mappin
     c->prec = precision;
     c->real_fields = real;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
-    for (int a = 0; a < 3; ++a) context_plan(Ns[a], precision, &c->plan[a]);
+    for (int a = 0; a < 3; ++a) context_plan(Ns[a], precision, a, &c->plan[a]);
 
     cudaError_t e = cudaGetDevice(&c->device);
     psatd_status st = PSATD_OK;

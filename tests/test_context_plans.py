@@ -16,13 +16,13 @@ class Plan(C.Structure):
 @pytest.fixture(scope="module")
 def plans():
     lib = psatd.lib()
-    plan, entry = lib._ZN5psatd12context_planEiiPNS_8AxisPlanE, lib._ZN5psatd14two_pass_entryEi
-    plan.restype, plan.argtypes = C.c_bool, [C.c_int, C.c_int, C.POINTER(Plan)]
+    plan, entry = lib._ZN5psatd12context_planEiiiPNS_8AxisPlanE, lib._ZN5psatd14two_pass_entryEi
+    plan.restype, plan.argtypes = C.c_bool, [C.c_int, C.c_int, C.c_int, C.POINTER(Plan)]
     entry.restype, entry.argtypes = C.POINTER(C.c_int), [C.c_int]         # starts with N, R1
 
-    def of(n, precision):
+    def of(n, precision, axis=0):
         p = Plan()
-        return list(p.radix[:p.npass]) if plan(n, precision, C.byref(p)) else None
+        return list(p.radix[:p.npass]) if plan(n, precision, axis, C.byref(p)) else None
 
     def first_radix(n):
         e = entry(n)
@@ -46,8 +46,8 @@ def test_plans_multiply_to_their_length(plans):
         for f in (2, 3, 5):
             while smooth % f == 0:
                 smooth //= f
-        for precision, most in ((32, 32), (64, 20)):
-            r = of(n, precision)
+        for precision, axis, most in ((32, 0, 32), (32, 2, 32), (64, 0, 16), (64, 1, 16), (64, 2, 20)):
+            r = of(n, precision, axis)
             assert (r is None) == (smooth != 1), n
             if r:
                 product = 1
