@@ -19,7 +19,9 @@ namespace psatd {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kTileCap = 64 * 1024;
+// largest tile: 64 KB (three blocks an SM share its memory; their registers allow two or
+// three in float32), 100 KB in float64 (two)
+template <typename T> constexpr int axis_tile_cap() { return (sizeof(T) == 8 ? 100 : 64) * 1024; }
 
 // narrow plans (radices to 16): three blocks of 256 threads per SM in float32
 template <typename T, int MAXR> constexpr int axis_min_blocks() {
@@ -75,6 +77,19 @@ inline double lane_share(const AxisPlan& pl, int Nx, int W) {
     return (double)Nx / ((Nx + W - 1) / W * W) * pl.npass / warps;
 }
 
+// Lanes a float64 row pass of W rows spends per value's item, each pass in whole warps;
+// with two passes or fewer half of it counted in rounds of all 256 threads (an uneven
+// last round leaves warps idle; three short passes with two blocks an SM hide that).
+inline double row_cost(const AxisPlan& pl, int W) {
+    double c = 0;
+    for (int p = 0; p < pl.npass; ++p) {
+        const int items = W * (pl.N / pl.radix[p]);
+        const double warps = (items + 31) / 32 * 32, rounds = items > 256 ? (items + 255) / 256 * 256 : warps;
+        c += (pl.npass > 2 ? warps : 0.5 * (warps + rounds)) / items;
+    }
+    return c;
+}
+
 // Tile of the transform along an axis: W pencils (a power of two of x-columns, 128
 // contiguous bytes a row, along y and z; rows giving about 256 first-pass items
 // along x), scaled by 2^shift, halved until the tile fits `cap` bytes.
@@ -86,6 +101,15 @@ void mix_tile_shape(int axis, const AxisPlan& pl, int Nx, int shift, size_t cap,
     int w;
     if (axis == 0) {
         w = max(1, min(128, 256 * pl.radix[0] / N));
+        // float64 is bound by its pipe, where idle lanes cost as much as busy ones: 1000
+        // points (10 x 10 x 10) in two rows give 200 items a pass.  1000 x 64 x 64 step
+        // 7.61 -> 7.32 ms, 480 x 64 x 64 3.78 -> 3.64 ms, 60 x 20 x 60 -10 %.
+        if (sizeof(T) == 8) {
+            int best = w;
+            for (int v = max(1, w / 2); v <= 4 * w && v * per <= cap; ++v)
+                if (row_cost(pl, v) < 0.97 * row_cost(pl, best)) best = v;
+            w = best;
+        }
     } else {
         w = 1;
         while (w < Nx && w < 128 / es) w *= 2;
@@ -115,8 +139,7 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
     if (pl.N <= 1) return cudaSuccess;
     int W, maxr = 0, logw = 0;
     size_t smem;
-    // a tile of 64 KB leaves three blocks on an SM
-    mix_tile_shape<T>(axis, pl, g.Nx, tb.tile_shift, kTileCap, &W, &smem);
+    mix_tile_shape<T>(axis, pl, g.Nx, tb.tile_shift, axis == 0 ? axis_tile_cap<T>() : 64 * 1024, &W, &smem);
     while ((1 << logw) < W) ++logw;
     for (int p = 0; p < pl.npass; ++p) maxr = max(maxr, pl.radix[p]);
     const long long nblocks = axis == 0 ? ((long long)ncomp * g.Nz * g.Ny + W - 1) / W
@@ -129,7 +152,7 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
     const int threads = (int)(items >= kThreads ? kThreads : (items + 31) / 32 * 32);
     auto launch = [&](auto sc, auto mc, auto rc, auto pc) {
         auto k = fft_axis_kernel<T, decltype(sc)::value, decltype(mc)::value, decltype(rc)::value, decltype(pc)::value>;
-        const cudaError_t e = allow_smem<kTileCap>(k);
+        const cudaError_t e = allow_smem<axis_tile_cap<T>()>(k);
         if (e != cudaSuccess) return e;
         if (nlaunch) ++*nlaunch;
         return launch_pdl(k, dim3((unsigned)nblocks), dim3(threads), smem, s, data, axis, g.Nx, g.Ny, g.Nz, ncomp, W,
