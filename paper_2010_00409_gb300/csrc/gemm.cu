@@ -658,12 +658,15 @@ cudaError_t launch_gemm_tma(const void* A, const void* B, float* C, int M, int N
     if (M % GT_BM || N % GT_BN || K % GT_BK || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15)
         return cudaErrorInvalidValue;
-    CUtensorMap ma, mb;
-    if (!gemm_map(&ma, A, M, K, GT_BM) || !gemm_map(&mb, B, N, K, GT_BN)) return cudaErrorInvalidValue;
     static PerDevice set;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    // the driver's encoder wants a current context, which a host thread has only after a
+    // runtime call that binds one
+    if (e == cudaSuccess) e = cudaSetDevice(dev);
     if (e != cudaSuccess) return e;
+    CUtensorMap ma, mb;
+    if (!gemm_map(&ma, A, M, K, GT_BM) || !gemm_map(&mb, B, N, K, GT_BN)) return cudaErrorInvalidValue;
     if ((e = sm_count(dev, &sms)) != cudaSuccess) return e;
     if ((e = set.once(dev, [] { return allow_smem<GT_SMEM>(gemm_tma_kernel); })) != cudaSuccess) return e;
     if (sms < 1) sms = 1;
