@@ -25,8 +25,6 @@ namespace psatd {
 
 namespace {
 
-constexpr double kPi = 3.14159265358979323846;
-
 // The angles are kept in units of pi and reduced before the sine and cosine: one
 // sincospi (no large-argument reduction) instead of a sine and a cosine of up to
 // N pi radians.
@@ -254,12 +252,14 @@ __global__ void contract_z_kernel(const double2* __restrict__ h, GridGeom g, She
 // 0.94 ms.
 
 constexpr int kXL = 8;                          // lanes per row of the x contraction
+constexpr int kXLFew = 32;                      // ... where there are few rows
 constexpr int kXThreads = 256;
 
-// sum over the kXL lanes of a row's group (every lane gets the total)
+// sum over the XL lanes of a row's group (every lane gets the total)
+template <int XL = kXL>
 __device__ __forceinline__ CFF group_sum(CFF a) {
 #pragma unroll
-    for (int o = kXL / 2; o > 0; o >>= 1) {
+    for (int o = XL / 2; o > 0; o >>= 1) {
         CFF b;
         b.re.h = __shfl_xor_sync(0xffffffffu, a.re.h, o);
         b.re.l = __shfl_xor_sync(0xffffffffu, a.re.l, o);
@@ -270,12 +270,12 @@ __device__ __forceinline__ CFF group_sum(CFF a) {
     return a;
 }
 
-// g[a][l][j] = sum_i wx[i] f[c_a][l][j][i]; kXL lanes take kXRows rows (a, l, j)
+// g[a][l][j] = sum_i wx[i] f[c_a][l][j][i]; XL lanes take kXRows rows (a, l, j)
 // half the rows apart, whose loads are in flight together and share each weight.
 // REAL: f holds float32 values (Nx even), else complex float32 ones.
 constexpr int kXRows = 2;
-template <bool REAL>
-__global__ void __launch_bounds__(kXThreads)
+template <bool REAL, int XL, int BLOCKS>
+__global__ void __launch_bounds__(kXThreads, BLOCKS)
 contract_x_ff_kernel(const float* __restrict__ f, GridGeom g, CompList cl, int ncomp,
                      const float4* __restrict__ wx, float4* __restrict__ out) {
     extern __shared__ float4 sw[];                            // the weights, [Nx]
@@ -283,10 +283,10 @@ contract_x_ff_kernel(const float* __restrict__ f, GridGeom g, CompList cl, int n
     pdl_wait();
     for (int i = threadIdx.x; i < g.Nx; i += kXThreads) sw[i] = wx[PSATD_IX(i, g.Nx)];
     __syncthreads();
-    const int lane = threadIdx.x % kXL;
+    const int lane = threadIdx.x % XL;
     const long long per_comp = (long long)g.Nz * g.Ny, rows = ncomp * per_comp;
     const long long units = (rows + kXRows - 1) / kXRows;
-    const long long unit = blockIdx.x * (long long)(kXThreads / kXL) + threadIdx.x / kXL;
+    const long long unit = blockIdx.x * (long long)(kXThreads / XL) + threadIdx.x / XL;
     long long row[kXRows];
     bool have[kXRows];                                        // (every lane takes part in the sums)
     const float2* p[kXRows];
@@ -302,31 +302,63 @@ contract_x_ff_kernel(const float* __restrict__ f, GridGeom g, CompList cl, int n
     }
     const GBuf<const float2> F{f2, 6LL * per_comp * n2};
     Dot2C acc[kXRows] = {};
-    auto mac = [&](int i) {
-#pragma unroll
-        for (int r = 0; r < kXRows; ++r) {
-            const float2 v = F.at(p[r], i);
-            if constexpr (REAL) {
-                dot2_mac_real(acc[r], sw[2 * i], sw[2 * i + 1], v);
-            } else {
-                dot2_mac(acc[r], sw[i], v);
-            }
-        }
+    auto mac = [&](int r, int i, float2 v) {
+        if constexpr (REAL) dot2_mac_real(acc[r], sw[2 * i], sw[2 * i + 1], v);
+        else dot2_mac(acc[r], sw[i], v);
     };
     int i = lane;
-#pragma unroll 2
-    for (; i + kXL < n2; i += 2 * kXL) {
-        mac(i);
-        mac(i + kXL);
+#pragma unroll 1
+    for (; i + 3 * XL < n2; i += 4 * XL) {
+        float2 v[kXRows][4];                                  // (all eight loads before the sums)
 #pragma unroll
-        for (int r = 0; r < kXRows; ++r) dot2_norm(acc[r]);
+        for (int e = 0; e < 4 * kXRows; ++e) v[e / 4][e % 4] = F.at(p[e / 4], i + e % 4 * XL);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int r = 0; r < kXRows; ++r) {
+                mac(r, i + k * XL, v[r][k]);
+                if (k % 2) dot2_norm(acc[r]);
+            }
     }
-    if (i < n2) mac(i);
+    for (; i < n2; i += XL)
+#pragma unroll
+        for (int r = 0; r < kXRows; ++r) {
+            mac(r, i, F.at(p[r], i));
+            dot2_norm(acc[r]);
+        }
 #pragma unroll
     for (int r = 0; r < kXRows; ++r) {
-        const CFF t = group_sum(dot2_value(acc[r]));
+        const CFF t = group_sum<XL>(dot2_value(acc[r]));
         if (have[r] && lane == 0) out[PSATD_IX(row[r], rows)] = cff_store(t);
     }
+}
+
+// XL lanes a row: 8 (fewer rounds of the cross-lane sum) unless that leaves the SMs
+// without two blocks each and a row is long enough for 32.  Three components of 64 x 64
+// points on 1000 x 64 x 64 118 -> 48 us, on 2048 x 32 x 32 127 -> 44 us (104 and 64 us
+// with a warp a row in renormalised sums); 32 lanes everywhere make the 256^3 real plane
+// of 128 x 128 points 167 -> 196 us.
+// Five blocks an SM (48 registers) keep a row's loads in flight together (256 x 128 x
+// 128, three components 63 -> 51 us against six).  A grid of short rows that fits six an
+// SM but not five takes six, without a second wave of a few blocks (128^3, three
+// components 46 -> 38 us; complex fields: real ones, 256 points a row, would spill).
+template <bool REAL>
+cudaError_t contract_x_ff(const float* f, const GridGeom& g, const CompList& cl, int ncomp, const float4* wx,
+                          float4* out, cudaStream_t s) {
+    const long long units = ((long long)ncomp * g.Nz * g.Ny + kXRows - 1) / kXRows;
+    auto launch = [&](auto lanes, auto blocks) {
+        constexpr int XL = decltype(lanes)::value, per = kXThreads / XL;
+        return launch_pdl(contract_x_ff_kernel<REAL, XL, decltype(blocks)::value>,
+                          dim3((unsigned)((units + per - 1) / per)), kXThreads, (size_t)g.Nx * sizeof(float4), s, f, g,
+                          cl, ncomp, wx, out);
+    };
+    using Five = std::integral_constant<int, 5>;
+    using Six = std::integral_constant<int, 6>;
+    const long long blocks = (units * kXL + kXThreads - 1) / kXThreads;
+    if (blocks < 2 * 152 && g.Nx >= 128) return launch(std::integral_constant<int, kXLFew>{}, Five{});
+    if constexpr (!REAL)
+        if (blocks > 5 * 152 && blocks <= 6 * 152 && g.Nx < 192) return launch(std::integral_constant<int, kXL>{}, Six{});
+    return launch(std::integral_constant<int, kXL>{}, Five{});
 }
 
 // Half spectrum of real fields (slots p < Nx/2 holding x mode mode[p], the x
@@ -338,7 +370,7 @@ contract_x_ff_kernel(const float* __restrict__ f, GridGeom g, CompList cl, int n
 // using conj(F) wx[-k_x] = conj(F wx[k_x]).  kXL lanes take a row and its mirror
 // and write both, so each row is read and summed once: l = 0 .. Nz/2, and the
 // pairs of l = 0 and l = Nz/2 only once (j <= their mirror).
-__global__ void __launch_bounds__(kXThreads)
+__global__ void __launch_bounds__(kXThreads, 5)
 contract_x_half_ff_kernel(const float2* __restrict__ S, const float2* __restrict__ Q, GridGeom g, CompList cl,
                           int ncomp, const int* __restrict__ mode, const float4* __restrict__ wx,
                           float4* __restrict__ out) {
@@ -365,19 +397,31 @@ contract_x_half_ff_kernel(const float2* __restrict__ S, const float2* __restrict
     Dot2C A{}, Am{};
     if (have) {
         // slot 0 holds x mode 0: its term belongs to Z
-        auto mac = [&](int p) {
+        int p = lane ? lane : kXL;
+#pragma unroll 1
+        for (; p + 3 * kXL < nh; p += 4 * kXL) {
+            float2 v[4], vm[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                v[k] = SF.at(pa, p + k * kXL);
+                vm[k] = SF.at(pm, p + k * kXL);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                dot2_mac(A, sw[p + k * kXL], v[k]);
+                dot2_mac(Am, sw[p + k * kXL], vm[k]);
+                if (k % 2) {
+                    dot2_norm(A);
+                    dot2_norm(Am);
+                }
+            }
+        }
+        for (; p < nh; p += kXL) {
             dot2_mac(A, sw[p], SF.at(pa, p));
             dot2_mac(Am, sw[p], SF.at(pm, p));
-        };
-        int p = lane ? lane : kXL;
-#pragma unroll 2
-        for (; p + kXL < nh; p += 2 * kXL) {
-            mac(p);
-            mac(p + kXL);
             dot2_norm(A);
             dot2_norm(Am);
         }
-        if (p < nh) mac(p);
     }
     const CFF sa = group_sum(dot2_value(A)), sm = group_sum(dot2_value(Am));
     if (have && lane < 2) {                                   // lane 0 writes the row, lane 1 its mirror
@@ -537,20 +581,17 @@ cudaError_t launch_sample_plane(const cplx<T>* data, const GridGeom& g, const Sh
     else
         e = launch_pdl(weights_kernel<ffw>, wgrid, kWThreads, 0, s, g, x_phys, ny, nz, y0, y1, z0, z1, sc.wx, sc.wy,
                          sc.wz);
-    const long long rows = (long long)ncomp * g.Nz * g.Ny;
     if constexpr (ffw) {
         if (e != cudaSuccess) return e;
-        const long long units = (rows + kXRows - 1) / kXRows;
-        const unsigned xb = (unsigned)((units + kXThreads / kXL - 1) / (kXThreads / kXL));
-        e = launch_pdl(contract_x_ff_kernel<false>, dim3(xb), kXThreads, (size_t)g.Nx * sizeof(float4), s,
-                                     reinterpret_cast<const float*>(data), g, cl, ncomp,
-                                     reinterpret_cast<const float4*>(sc.wx), reinterpret_cast<float4*>(sc.g));
+        e = contract_x_ff<false>(reinterpret_cast<const float*>(data), g, cl, ncomp,
+                                 reinterpret_cast<const float4*>(sc.wx), reinterpret_cast<float4*>(sc.g), s);
         if (e == cudaSuccess)
             e = contract_yz_ff(g, sh, x_phys, ny, nz, y0, y1, z0, z1, t, ncomp, sc, reinterpret_cast<float2*>(out), s);
         if (nlaunch) *nlaunch += 4;
         return e;
     }
     if (e != cudaSuccess) return e;
+    const long long rows = (long long)ncomp * g.Nz * g.Ny;
     const long long nh = (long long)ncomp * g.Nz * ny;
     const long long no = (long long)ncomp * nz * ny;
     contract_x_kernel<T><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(data, g, cl, ncomp, sc.wx, sc.g);
@@ -587,9 +628,7 @@ cudaError_t launch_sample_plane_real(const float* data, const float2* nyq, const
                          (size_t)(g.Nx / 2 + 1) * sizeof(float4), s, reinterpret_cast<const float2*>(data), nyq, g, cl,
                          ncomp, slot_mode, wx, gg);
     } else {
-        const long long units = ((long long)ncomp * g.Nz * g.Ny + kXRows - 1) / kXRows;
-        e = launch_pdl(contract_x_ff_kernel<true>, dim3((unsigned)((units + per - 1) / per)), kXThreads,
-                         (size_t)g.Nx * sizeof(float4), s, data, g, cl, ncomp, wx, gg);
+        e = contract_x_ff<true>(data, g, cl, ncomp, wx, gg, s);
     }
     if (e == cudaSuccess) e = contract_yz_ff(g, sh, x_phys, ny, nz, y0, y1, z0, z1, t, ncomp, sc, out, s);
     if (nlaunch) *nlaunch += 4;
