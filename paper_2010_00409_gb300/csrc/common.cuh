@@ -131,10 +131,6 @@ __host__ __device__ constexpr UnitF unit_f32(double c, double s) {
     }
     return best;
 }
-// multiply by s*i, s = +-1
-template <typename V> __host__ __device__ __forceinline__ V cmul_si(V a, int s) {
-    V r; if (s > 0) { r.x = -a.y; r.y = a.x; } else { r.x = a.y; r.y = -a.x; } return r;
-}
 
 // |a|^2 + |b|^2 + |c|^2 of one cell's three components, formed in the storage
 // precision (float32 storage: float32 products and sums, relative error ~1e-7)

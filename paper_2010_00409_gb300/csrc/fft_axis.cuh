@@ -159,11 +159,12 @@ cudaError_t launch_fft_axis(cplx<T>* data, int ncomp, const GridGeom& g, const T
                           logw, pl, tb.twp[axis]);
     };
     auto by_rows = [&](auto sc, auto mc) {
-        if constexpr (sizeof(T) == 4)
-            if (axis == 0 && row_padded(pl))
-                return launch(sc, std::integral_constant<int, kNarrow>{}, std::true_type{}, std::true_type{});
-        return axis == 0 ? launch(sc, mc, std::true_type{}, std::false_type{})
-                         : launch(sc, mc, std::false_type{}, std::false_type{});
+        if (axis != 0) return launch(sc, mc, std::false_type{}, std::false_type{});
+        if constexpr (sizeof(T) == 8)                             // (wide float64 plans exist along z alone)
+            return launch(sc, std::integral_constant<int, kNarrow>{}, std::true_type{}, std::false_type{});
+        else
+            return row_padded(pl) ? launch(sc, std::integral_constant<int, kNarrow>{}, std::true_type{}, std::true_type{})
+                                  : launch(sc, mc, std::true_type{}, std::false_type{});
     };
     auto by_radix = [&](auto sc) {
         return maxr <= kNarrow ? by_rows(sc, std::integral_constant<int, kNarrow>{})

@@ -227,8 +227,13 @@ __device__ __forceinline__ void mix_dispatch(const MixTile<T>& t, cplx<T>* sm, c
     }
     if constexpr (MAXR > kNarrow) {
         switch (R) {
-            PSATD_MIX(18); PSATD_MIX(20); PSATD_MIX(24); PSATD_MIX(25); PSATD_MIX(27); PSATD_MIX(30);
-            PSATD_MIX(32);
+            PSATD_MIX(18); PSATD_MIX(20);
+            default: break;
+        }
+    }
+    if constexpr (MAXR > kNarrow && sizeof(T) == 4) {             // (float64 plans stop at 20)
+        switch (R) {
+            PSATD_MIX(24); PSATD_MIX(25); PSATD_MIX(27); PSATD_MIX(30); PSATD_MIX(32);
             default: break;
         }
     }

@@ -65,8 +65,8 @@ struct TwoPassEntry {
     int N, R1;
     int cols_threads, cols_smem, rows_threads, rows_per_block, rows_smem;
     int kspace_threads, kspace_smem;        // 0: the six components' tile does not fit
-    void (*cols[2])(TwoPassArgs);           // forward, inverse (null: tile too large)
-    void (*rows[2])(TwoPassArgs);
+    void (*cols[2])(TwoPassArgs);           // forward, inverse (null: tile too large, or
+    void (*rows[2])(TwoPassArgs);           // a length that always takes another kernel)
     void (*kspace)(TwoPassArgs, TwoPassModes);
 };
 // The kernels of length N, or null.
@@ -86,8 +86,9 @@ template <int R1, int R2> struct TwoCfg {
     }
     static constexpr int cols_threads = (R1 * kTwoW + 31) / 32 * 32;
     static constexpr int cols_smem = N * kTwoW * (int)sizeof(float2);
-    static constexpr bool cols = cols_smem < 96 * 1024;
+    static constexpr bool cols = cols_smem < 96 * 1024 && N != 512;     // (512: fft_three.cu)
     static constexpr int G = 256 / R1;                                  // rows per block
+    static constexpr bool rows = N != 64 && N != 128 && N != 256 && N != 512;   // (fft_fast.cu)
     static constexpr int rows_threads = (G * R1 + 31) / 32 * 32;
     static constexpr int run = R2 | 1, P = (R1 * run) | 1;              // row layout of fft_mixed.cuh
     static constexpr int rows_smem = G * P * (int)sizeof(float2);
@@ -339,8 +340,10 @@ template <int R1, int R2> TwoPassEntry two_pass_make() {
         e.cols[0] = two_cols_kernel<R1, R2, -1>;
         e.cols[1] = two_cols_kernel<R1, R2, +1>;
     }
-    e.rows[0] = two_rows_kernel<R1, R2, -1>;
-    e.rows[1] = two_rows_kernel<R1, R2, +1>;
+    if constexpr (Cfg::rows) {
+        e.rows[0] = two_rows_kernel<R1, R2, -1>;
+        e.rows[1] = two_rows_kernel<R1, R2, +1>;
+    }
     if constexpr (Cfg::kspace) {
         e.kspace_threads = Cfg::kspace_threads;
         e.kspace_smem = Cfg::kspace_smem;

@@ -225,6 +225,12 @@ __device__ __noinline__ void z_two(const MultiProblem<float>& P, int item) {
     two_z_inverse<R1, R2, kMT>(base, plane, cstride, nw, P.tp[2], sm, F);
 }
 
+// (longer z tiles are over the budget and take the run-time passes)
+template <int R1, int R2>
+__device__ __forceinline__ void two_phase_z(const MultiProblem<float>& P, int item) {
+    if constexpr (6 * R1 * R2 * kTwoKW * sizeof(float2) <= multi_tile_budget<float>()) z_two<R1, R2>(P, item);
+}
+
 // Phase ph of the item with the compile-time tile `id`.
 __device__ __forceinline__ void two_phase(int ph, int id, const MultiProblem<float>& P, int item) {
     switch (id) {
@@ -232,7 +238,7 @@ __device__ __forceinline__ void two_phase(int ph, int id, const MultiProblem<flo
     case i:                                                  \
         if (ph == 0) x_two<r1, r2, -1>(P, item);             \
         else if (ph == 1) y_two<r1, r2, -1>(P, item);        \
-        else if (ph == 2) z_two<r1, r2>(P, item);            \
+        else if (ph == 2) two_phase_z<r1, r2>(P, item);      \
         else if (ph == 3) y_two<r1, r2, +1>(P, item);        \
         else x_two<r1, r2, +1>(P, item);                     \
         break;

@@ -589,17 +589,18 @@ cudaError_t launch_sample_plane(const cplx<T>* data, const GridGeom& g, const Sh
             e = contract_yz_ff(g, sh, x_phys, ny, nz, y0, y1, z0, z1, t, ncomp, sc, reinterpret_cast<float2*>(out), s);
         if (nlaunch) *nlaunch += 4;
         return e;
+    } else {
+        if (e != cudaSuccess) return e;
+        const long long rows = (long long)ncomp * g.Nz * g.Ny;
+        const long long nh = (long long)ncomp * g.Nz * ny;
+        const long long no = (long long)ncomp * nz * ny;
+        contract_x_kernel<T><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(data, g, cl, ncomp, sc.wx, sc.g);
+        contract_y_kernel<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(sc.g, g, ncomp, ny, sc.wy, sc.h);
+        contract_z_kernel<T><<<(unsigned)((no + 255) / 256), 256, 0, s>>>(sc.h, g, sh, ncomp, ny, nz, x_phys,
+                                                                          y0, y1, z0, z1, t, sc.wz, out);
+        if (nlaunch) *nlaunch += 4;
+        return cudaGetLastError();
     }
-    if (e != cudaSuccess) return e;
-    const long long rows = (long long)ncomp * g.Nz * g.Ny;
-    const long long nh = (long long)ncomp * g.Nz * ny;
-    const long long no = (long long)ncomp * nz * ny;
-    contract_x_kernel<T><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(data, g, cl, ncomp, sc.wx, sc.g);
-    contract_y_kernel<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(sc.g, g, ncomp, ny, sc.wy, sc.h);
-    contract_z_kernel<T><<<(unsigned)((no + 255) / 256), 256, 0, s>>>(sc.h, g, sh, ncomp, ny, nz, x_phys,
-                                                                      y0, y1, z0, z1, t, sc.wz, out);
-    if (nlaunch) *nlaunch += 4;
-    return cudaGetLastError();
 }
 
 cudaError_t launch_sample_plane_real(const float* data, const float2* nyq, const int* slot_mode, const GridGeom& g,

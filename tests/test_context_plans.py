@@ -13,6 +13,23 @@ class Plan(C.Structure):
                 ("div_l", C.c_uint * 8), ("div_run", C.c_uint)]
 
 
+class Entry(C.Structure):
+    _fields_ = [(n, C.c_int) for n in ("N", "R1", "cols_threads", "cols_smem", "rows_threads", "rows_per_block",
+                                       "rows_smem", "kspace_threads", "kspace_smem")] + [
+        ("cols", C.c_void_p * 2), ("rows", C.c_void_p * 2), ("kspace", C.c_void_p)]
+
+
+def test_no_kernel_for_axes_that_always_take_another(plans):
+    """x axes of 64, 128, 256 and 512 points and 512-point columns have register kernels
+    of their own (fft_fast.cu, fft_three.cu): no two-pass kernel is compiled for them."""
+    find = psatd.lib()["_ZN5psatd14two_pass_entryEi"]              # (a function object of its own)
+    find.restype, find.argtypes = C.c_void_p, [C.c_int]
+    entries = [Entry.from_address(find(n)) for n in range(1, 1025) if find(n)]
+    for e in entries:
+        assert bool(e.rows[0]) == bool(e.rows[1]) == (e.N not in (64, 128, 256, 512)), e.N
+        assert bool(e.cols[0]) == bool(e.cols[1]) == (e.N * 16 * 8 < 96 * 1024 and e.N != 512), e.N
+
+
 @pytest.fixture(scope="module")
 def plans():
     lib = psatd.lib()
