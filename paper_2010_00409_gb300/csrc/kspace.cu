@@ -128,9 +128,8 @@ cudaError_t launch_kspace_z(cplx<T>* data, const GridGeom& g, const Tables<T>& t
                             double scale, cudaStream_t s, long long* nlaunch) {
     const int es = (int)sizeof(cplx<T>);
     const AxisPlan& pl = tb.plan[2];
-    // 64 contiguous bytes a row of the tile; the six components' tile capped at 76 KB
-    // in float32 (three blocks per SM; two of 110 KB where eight columns need that),
-    // 100 KB in float64 (two)
+    // 64 contiguous bytes a row of the tile; the six components' tile capped at 112 KB
+    // in float32 (two blocks per SM; three from 192 points down), 100 KB in float64 (two)
     auto bytes = [&](int w) { return (size_t)6 * g.Nz * w * es; };
     int W = 1;
     while (W < g.Nx && W < 64 / es) W *= 2;

@@ -170,8 +170,8 @@ __device__ __forceinline__ void z_tile(const MultiProblem<T>& P, long long item,
 // ---------------------------------------------------------------------------
 // float32 lengths of two radices up to 16: the compile-time tiles of fft_two.cuh,
 // each a function of its own, with the tile at its fixed place in shared memory.  As
-// calls they keep the kernel at 80 registers without spills (three blocks an SM) and
-// cost a jump an item, which is 2 us of work or more.
+// calls they keep the kernel at 80 registers (three blocks an SM; 16 bytes of spills in
+// the kernel's own frame) and cost a jump an item, which is 2 us of work or more.
 __device__ __forceinline__ float2* multi_tile() {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     return reinterpret_cast<float2*>(smem_raw + desc_bytes<float>());
@@ -248,7 +248,7 @@ __device__ __forceinline__ void two_phase(int ph, int id, const MultiProblem<flo
     }
 }
 
-// float32: three blocks per SM (85 registers a thread, tiles of at most 72 KB)
+// float32: three blocks per SM (room for 85 registers a thread, tiles of at most 72 KB)
 template <typename T>
 __global__ void __launch_bounds__(kMT, sizeof(T) == 4 ? 3 : 2)
 multi_advance_kernel(const MultiProblem<T>* __restrict__ probs, const long long* __restrict__ prefix, int nprob,
